@@ -108,16 +108,13 @@ struct SweepTask {
   int b;       // instance
   int u0;      // first unique direction (directions u0..u0+D-1 share a quadrant)
   int t;       // task index within the instance (partial-sum slot)
-  int pad;
+  int n;       // directions of the task (0: as many as the kernel takes; fewer in a quadrant's last task)
 };
 
-// dsa.cu: DSA preconditioner through one multigrid V-cycle.  dsa_check: whether the meshes are covered;
-// dsa_prepare: per-parameter set-up (cross sections, cell blocks, Galerkin hierarchy); dsa_launch:
-// z = v + x (x ~ K^{-1} Sigma_s v) for instances with active[b] (and only[b], when given).
-int dsa_check(rte_problem* p);
-int dsa_prepare(rte_problem* p, int variant, cudaStream_t st);
-int dsa_launch(rte_problem* p, bool f64, const void* v, void* z, const int* active, const int* only,
-               cudaStream_t st);
+// Launch shape of an operator sweep (wavefront.cu): directions per task, warps per task, mesh rows per lane.
+struct WaveShape {
+  int D = 0, W = 1, rpl = 1;
+};
 }  // namespace rte
 
 struct rte_problem {
@@ -147,7 +144,11 @@ struct rte_problem {
   rte::DevBuf<double> d_G;                    // [ntot] source moments
   rte::DevBuf<double> d_linv64;               // [B][nu][R][nd*nd]
   rte::DevBuf<float> d_linv32;
-  rte::DevBuf<float> d_linv_df;               // the same as double-float pairs (hi, lo) [..][2]
+  rte::DevBuf<float> d_linv_df;               // 1D: the same as double-float pairs (hi, lo) [..][2]
+  // 2D operator sweeps (wavefront.cu): cell tables per (instance, unique direction, region), [8] FP32, [4] FP64 and
+  // [4][2] double-float pairs
+  rte::DevBuf<float> d_rot32, d_modal_df;
+  rte::DevBuf<double> d_modal64;
   rte::DevBuf<float> d_sig_s_df;              // [B][R][2] sigma_s as double-float pairs
   rte::DevBuf<float> d_xdf;                   // [ntot][2] operator input split into double-float pairs
   // sweep scratch (grown on demand)
@@ -155,20 +156,16 @@ struct rte_problem {
   // task lists per directions-per-warp value D (index D), built once; stable device pointers
   rte::DevBuf<rte::SweepTask> d_tasks_by_D[17];
   int ntasks_by_D[17] = {0};
-  // pipelined band kernel: runs of tasks per persistent CTA (first task, tasks, period, 0), per D
-  rte::DevBuf<int4> d_runs_by_D[17];
-  int nruns_by_D[17] = {0};
-  size_t pipe_smem_elems_by_D[17] = {0};
   int per_inst_by_D[17] = {0};
   int tasks_D = -1;                           // D of the most recent launch
-  // sweep autotuner (sweep.cu): tuned directions per warp and kernel variant per [precision][angular]
-  // (precision: PREC_F32, PREC_F64, PREC_DF; 0 = not tuned); force_* steer launches while candidates are timed
+  // sweep autotuner (sweep.cu): tuned directions per task and kernel variant per [precision][angular]
+  // (precision: PREC_F32, PREC_F64, PREC_DF; 0 = not tuned); force_* steer launches while candidates are timed.
+  // Operator sweeps of region problems have a shape (directions, warps per task, rows per lane) instead
   int tuned_D[3][2] = {{0, 0}, {0, 0}, {0, 0}};
   int tuned_var[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};
   int force_D = 0, force_var = -1;
+  rte::WaveShape tuned_shape[3], rule_shape[3], force_shape;   // rule: the cost estimate's choice, made once
   int pin_D = 0, pin_var = -1;                // rte_problem_set_sweep_variant (a user's pin; overrides the tuning)
-  int pin_run = 0;                            // tasks per run of the pipelined kernel (0: automatic)
-  float tuned_ms[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   int ntasks = 0, tasks_per_inst = 0;
   rte::DevBuf<int> d_active;                  // [B] instance mask (1 = active), all 1 by default
   rte::DevBuf<double> d_tmp64;                // [ntot] temporaries
@@ -192,6 +189,8 @@ struct rte_problem {
 namespace rte {
 // problem.cu
 int upload_params(rte_problem* p);
+// wavefront.cu: cell tables of the operator sweeps from the current cross sections
+int build_wave_tables(rte_problem* p);
 // greatest common divisor of the unique-direction counts of the quadrants (2D) or of the two half-ranges (1D):
 // a directions-per-warp value must divide it
 int quadrant_gcd(const rte_problem* p);

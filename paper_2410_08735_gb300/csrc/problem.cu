@@ -134,10 +134,11 @@ __global__ void k_linv(int B, int nu, int R, int dim, const InstInfo* inst, cons
   for (int i = 0; i < nd * nd; ++i) {
     out64[base + i] = X[i];
     out32[base + i] = (float)X[i];
-    // double-float pair: the FP32 rounding and the FP32 rounding of what it misses
-    const float h = (float)X[i];
-    outdf[2 * (base + i)] = h;
-    outdf[2 * (base + i) + 1] = (float)(X[i] - (double)h);
+    if (outdf) {   // double-float pair: the FP32 rounding and the FP32 rounding of what it misses
+      const float h = (float)X[i];
+      outdf[2 * (base + i)] = h;
+      outdf[2 * (base + i) + 1] = (float)(X[i] - (double)h);
+    }
   }
 }
 
@@ -268,6 +269,7 @@ int upload_params(rte_problem* p) {
                                                                   p->d_linv32.p, p->d_linv_df.p);
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
+  if (p->dim == 2) RTE_TRY(build_wave_tables(p));
   {
     int maxn = 0;
     for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
@@ -514,7 +516,14 @@ static int create_impl(const rte_problem_desc* d, rte_problem* p) {
   size_t nl = (size_t)p->B * p->nu * p->R * p->nd * p->nd;
   RTE_TRY(p->d_linv64.alloc(nl));
   RTE_TRY(p->d_linv32.alloc(nl));
-  RTE_TRY(p->d_linv_df.alloc(2 * nl));
+  if (p->dim == 2) {
+    const size_t nt = (size_t)p->B * p->nu * p->R;
+    RTE_TRY(p->d_rot32.alloc(8 * nt));
+    RTE_TRY(p->d_modal64.alloc(4 * nt));
+    RTE_TRY(p->d_modal_df.alloc(8 * nt));
+  } else {
+    RTE_TRY(p->d_linv_df.alloc(2 * nl));
+  }
   RTE_TRY(p->d_active.alloc(p->B));
   RTE_TRY(p->d_wq.alloc(p->ndir));
   if (p->cellsig) {

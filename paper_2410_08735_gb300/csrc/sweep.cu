@@ -5,6 +5,9 @@
 //   T s   = sum_j omega_j psi_j            fused: psi is never stored
 //   A~ z  = z - T (Sigma_s z)              fused Sigma_s scaling on load, subtraction in the reduce
 //
+// The operator's sweeps on 2D meshes with cross sections per region (T s, A~ z, b~) run in wavefront.cu; the kernels here
+// are the angular sweeps (psi stored), the sweeps with cross-section profiles, and the slab.
+//
 // 2D work decomposition.  A task is (instance, quadrant, chunk of D unique directions); one warp
 // runs one task.  Lane l owns mesh rows l, l+32, l+64, ... (rows counted in the upwind y order) and
 // marches along its row in the upwind x order.  The 32 rows of a band form a diagonal wavefront:
@@ -23,80 +26,17 @@
 // (1, -sqrt3), tx_b = psi_0b + sqrt3 psi_1b (x-outflow trace), ty_a = psi_a0 + sqrt3 psi_a1; L^{-1}
 // per (instance, direction, region) is precomputed (problem.cu) and staged in shared memory.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
 
-#include "dfloat.cuh"
-#include "internal.h"
+#include "sweep.h"
 
 namespace rte {
-
-struct SweepArgs {
-  const InstInfo* inst;
-  const UDir* udir;
-  const SweepTask* tasks;
-  int ntasks;
-  const void* linv;     // compute type, [B][nu][R][nd*nd]
-  const void* sig_s;    // compute type, [B][R]; null: no Sigma_s scaling of the input
-  const void* src;      // input type, scalar vector
-  int with_bc;
-  int inflow_mask;      // faces carrying the inflow: 1 x-low, 2 x-high, 4 y-low, 8 y-high
-  void* partial;        // compute type, [tasks_per_inst * off_b + t * N_b + i]
-  int tasks_per_inst;
-  void* psi;            // compute type, angular vector, or null
-  int ndir, nu, R, rx, ry;
-  const int* active;    // [B] or null
-  int smem_per_warp;    // elements of the compute type
-  int psi_unique;       // angular output: 0 = all N_Omega directions, 1 = one block per unique direction
-};
-
-template <typename T>
-struct Vec4;
-template <>
-struct Vec4<float> {
-  __device__ static void load(const float* p, float& a, float& b, float& c, float& d) {
-    float4 v = *reinterpret_cast<const float4*>(p);
-    a = v.x; b = v.y; c = v.z; d = v.w;
-  }
-  __device__ static void store(float* p, float a, float b, float c, float d) {
-    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
-  }
-};
-template <>
-struct Vec4<double> {
-  __device__ static void load(const double* p, double& a, double& b, double& c, double& d) {
-    double2 v0 = reinterpret_cast<const double2*>(p)[0];
-    double2 v1 = reinterpret_cast<const double2*>(p)[1];
-    a = v0.x; b = v0.y; c = v1.x; d = v1.y;
-  }
-  __device__ static void store(double* p, double a, double b, double c, double d) {
-    reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
-    reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
-  }
-};
-
-template <>
-struct Vec4<dfloat> {
-  __device__ static void load(const dfloat* p, dfloat& a, dfloat& b, dfloat& c, dfloat& d) {
-    const float4 v0 = reinterpret_cast<const float4*>(p)[0];
-    const float4 v1 = reinterpret_cast<const float4*>(p)[1];
-    a = dfloat(v0.x, v0.y); b = dfloat(v0.z, v0.w); c = dfloat(v1.x, v1.y); d = dfloat(v1.z, v1.w);
-  }
-  __device__ static void store(dfloat* p, dfloat a, dfloat b, dfloat c, dfloat d) {
-    reinterpret_cast<float4*>(p)[0] = make_float4(a.hi, a.lo, b.hi, b.lo);
-    reinterpret_cast<float4*>(p)[1] = make_float4(c.hi, c.lo, d.hi, d.lo);
-  }
-};
 
 // value of the lane below (lane - 1) in the warp
 template <typename T>
 __device__ __forceinline__ T shfl_up1(T v) { return __shfl_up_sync(0xffffffffu, v, 1); }
-template <>
-__device__ __forceinline__ dfloat shfl_up1<dfloat>(dfloat v) {
-  return dfloat(__shfl_up_sync(0xffffffffu, v.hi, 1), __shfl_up_sync(0xffffffffu, v.lo, 1));
-}
 
 // precision slot of a sweep arithmetic type (autotuner tables, partial-sum element size)
 template <typename T>
@@ -409,8 +349,10 @@ __global__ void __launch_bounds__(128) k_sweep2d(SweepArgs a) {
 // earlier group, before that group's barrier.  The critical path is the nx + ny - 1 diagonals plus the skew
 // of the bands, and a lane's cell index moves by one per step, so the step loop has no division and the
 // source prefetch is a plain +-PF offset.
-template <typename T, typename TI, int D, bool ANG>
+template <typename T, int D>
 __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
+  using TI = T;
+  constexpr bool ANG = true;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
   const int tid = blockIdx.x;
@@ -630,250 +572,6 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
   }
 }
 
-// Pipelined band variant (operator apply only): a persistent CTA sweeps a run of tasks on meshes of one size
-// back to back.  In the band kernel a band works only while the wavefront crosses its 32 rows, about half of the
-// sweep on an 8-band mesh.  Here band w starts task k at step k P + (32 + SK) w, so a band that has finished its
-// rows of task k goes straight on to task k + 1 while the bands above it still work on task k.  Run = (first
-// task, tasks, period P); the CTA first drops the tasks of inactive instances.  Task k uses table buffer k & 1,
-// loaded during the barrier group before band 0 starts it; the host picks P (a multiple of SK) with
-// 2 P >= (32 + SK)(nb - 1) + nx + 40, so the buffer's previous task has left every band by then.  The y-outflow
-// buffer between bands needs no second copy: band w writes column c of task k + 1 long after band w + 1 has read
-// column c of task k.  A lane's shuffle partner (the lane below) is always on the same task and column.
-template <typename T, typename TI, int D>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && D <= 4) ? 2 : 1) k_sweep2d_pipe(SweepArgs a, const int4* runs) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nwarps = blockDim.x >> 5;
-  const int4 run = runs[blockIdx.x];   // (first task, tasks, period, 0)
-  const int t0 = run.x, P = run.z;
-  constexpr int SK = 8, PF = 8;
-  constexpr int KMAX = 64;
-  __shared__ int klist[KMAX];          // the run's tasks whose instance is active
-  __shared__ int kcount;
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int k = 0; k < run.y && k < KMAX; ++k) {
-      const int b = a.tasks[t0 + k].b;
-      if (!a.active || a.active[b]) klist[n++] = t0 + k;
-    }
-    kcount = n;
-  }
-  __syncthreads();
-  const int K = kcount;
-  if (K == 0) return;
-  const InstInfo in0 = a.inst[a.tasks[klist[0]].b];
-  const int nx = in0.nx, ny = in0.ny, R = a.R;
-  const int nb = (ny + 31) >> 5;
-  const int R4 = (R + 3) & ~3;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tab = reinterpret_cast<T*>(smem_raw);                  // [2][D][R][16]
-  T* sgs = tab + 2 * D * R * 16;                             // [2][R4]
-  T* ybuf = sgs + 2 * R4;                                    // [nwarps-1][D][nx][2]
-  int* xreg = reinterpret_cast<int*>(ybuf + (((size_t)(nwarps > 1 ? nwarps - 1 : 1) * D * nx * 2 + 3) & ~(size_t)3));
-  const int cx = nx / a.rx, cy = ny / a.ry;
-  for (int e = threadIdx.x; e < nx; e += blockDim.x) xreg[e] = e / cx;
-  // per-task parameters, computed once per task by the loading threads (the FP64 divisions of the direction
-  // coefficients must not run once per lane): coefficients, inflow traces, signs, partial-flux offset
-  __shared__ T s_al[2][D], s_be[2][D], s_wg[2][D], s_bnd[2][2];
-  __shared__ int s_sgn[2][2];
-  __shared__ long long s_poff[2];
-  auto load_table = [&](int k) {
-    const SweepTask tk = a.tasks[klist[k]];
-    const int bf = k & 1;
-    const T* linv = reinterpret_cast<const T*>(a.linv) + ((size_t)tk.b * a.nu + tk.u0) * R * 16;
-    T* dst = tab + (size_t)bf * D * R * 16;
-    for (int e = threadIdx.x; e < D * R * 16; e += blockDim.x) dst[e] = linv[e];
-    if (a.sig_s)
-      for (int e = threadIdx.x; e < R; e += blockDim.x)
-        sgs[bf * R4 + e] = reinterpret_cast<const T*>(a.sig_s)[(size_t)tk.b * R + e];
-    if (threadIdx.x < D) {
-      const InstInfo in = a.inst[tk.b];
-      const UDir u = a.udir[tk.u0 + threadIdx.x];
-      s_al[bf][threadIdx.x] = (T)(u.ax / in.hx);
-      s_be[bf][threadIdx.x] = (T)(u.ay / in.hy);
-      s_wg[bf][threadIdx.x] = (T)u.w;
-    } else if (threadIdx.x == D) {
-      const InstInfo in = a.inst[tk.b];
-      const int tsx = a.udir[tk.u0].sx, tsy = a.udir[tk.u0].sy;
-      const double gtr = a.with_bc ? in.g * sqrt(in.hx * in.hy) : 0.0;
-      s_bnd[bf][0] = (a.inflow_mask & (tsx > 0 ? 1 : 2)) ? (T)gtr : (T)0;
-      s_bnd[bf][1] = (a.inflow_mask & (tsy > 0 ? 4 : 8)) ? (T)gtr : (T)0;
-      s_sgn[bf][0] = tsx;
-      s_sgn[bf][1] = tsy;
-      s_poff[bf] = (long long)a.tasks_per_inst * in.off + (long long)tk.t * in.ndof;
-    }
-  };
-  load_table(0);
-  __syncthreads();
-  const bool sig_s = a.sig_s != nullptr;
-  const T S3 = (T)1.7320508075688772;
-  const int band = warp;
-  const int row = band * 32 + lane;
-  const bool rowok = band < nb && row < ny;
-  const int nsteps = (K - 1) * P + (32 + SK) * (nb - 1) + 31 + nx;
-  // state of the task the lane works on (k) and of the task its prefetch cursor is in (kp)
-  int k = -1, col = -((32 + SK) * band + lane) - 1;   // advanced to step 0 below
-  int kp = -1, colp = col + PF;
-  T al[D], be[D], wg[D];
-  T bndx = (T)0, bndy = (T)0;
-  int sx = 1, sy = 1, rowreg = 0;
-  long long rowbase = 0;
-  T* part = nullptr;
-  const TI* srcp = nullptr;   // prefetch task's source
-  long long rowbase_p = 0;
-  int sxp = 1;
-#pragma unroll
-  for (int d = 0; d < D; ++d) { al[d] = be[d] = wg[d] = (T)0; }
-  auto enter_task = [&](int kk) {   // the lane's current task becomes kk (its parameters are in buffer kk & 1)
-    const int bf = kk & 1;
-    sx = s_sgn[bf][0];
-    sy = s_sgn[bf][1];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      al[d] = s_al[bf][d];
-      be[d] = s_be[bf][d];
-      wg[d] = s_wg[bf][d];
-    }
-    bndx = s_bnd[bf][0];
-    bndy = s_bnd[bf][1];
-    const int iy = sy > 0 ? row : ny - 1 - row;
-    rowbase = (long long)(rowok ? iy : 0) * nx;
-    rowreg = rowok ? (iy / cy) * a.rx : 0;
-    part = reinterpret_cast<T*>(a.partial) + s_poff[bf];
-  };
-  auto enter_prefetch = [&](int kk) {
-    const SweepTask tk = a.tasks[klist[kk]];
-    const InstInfo in = a.inst[tk.b];
-    sxp = a.udir[tk.u0].sx;
-    const int syp = a.udir[tk.u0].sy;
-    const int iy = syp > 0 ? row : ny - 1 - row;
-    rowbase_p = (long long)(rowok ? iy : 0) * nx;
-    srcp = reinterpret_cast<const TI*>(a.src) + in.off;
-  };
-  // advance a (task, column) cursor by one step; returns true when it enters a new task
-  auto step_cursor = [&](int& kk, int& cc) -> bool {
-    ++cc;
-    if (kk < 0) {
-      if (cc == 0) { kk = 0; return true; }
-      return false;
-    }
-    if (cc == P) {
-      cc = 0;
-      ++kk;
-      return kk < K;
-    }
-    return false;
-  };
-  TI q0[PF], q1[PF], q2[PF], q3[PF];
-  // fill the prefetch ring with the sources of steps 0 .. PF-1; the cursor then stands at step PF-1
-  {
-    int kq = -1, cq = col;   // the state before step 0
-#pragma unroll
-    for (int j = 0; j < PF; ++j) {
-      if (step_cursor(kq, cq) && kq < K) enter_prefetch(kq);
-      if (rowok && kq >= 0 && kq < K && cq < nx)
-        Vec4<TI>::load(srcp + 4 * (rowbase_p + (sxp > 0 ? cq : nx - 1 - cq)), q0[j], q1[j], q2[j], q3[j]);
-    }
-    kp = kq;
-    colp = cq;
-  }
-  T tx0[D], tx1[D], ty0[D], ty1[D];
-#pragma unroll
-  for (int d = 0; d < D; ++d) { tx0[d] = tx1[d] = ty0[d] = ty1[d] = (T)0; }
-  for (int s0 = 0; s0 < nsteps; s0 += PF) {
-    // the task that band 0 starts at the next group: its table goes into buffer (k & 1) now
-    if ((s0 + PF) % P == 0) {
-      const int kn = (s0 + PF) / P;
-      if (kn < K) load_table(kn);
-    }
-#pragma unroll
-    for (int kk = 0; kk < PF; ++kk) {
-      const int s = s0 + kk;
-      if (step_cursor(k, col) && k < K) enter_task(k);
-      const bool act = rowok && s < nsteps && k >= 0 && k < K && col < nx;
-      T s0v = (T)q0[kk], s1 = (T)q1[kk], s2 = (T)q2[kk], s3 = (T)q3[kk];
-      if (step_cursor(kp, colp) && kp < K) enter_prefetch(kp);
-      if (rowok && kp >= 0 && kp < K && colp < nx)
-        Vec4<TI>::load(srcp + 4 * (rowbase_p + (sxp > 0 ? colp : nx - 1 - colp)), q0[kk], q1[kk], q2[kk], q3[kk]);
-      T yi0[D], yi1[D];
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        yi0[d] = shfl_up1(ty0[d]);
-        yi1[d] = shfl_up1(ty1[d]);
-      }
-      if (act) {
-        const int buf = k & 1;
-        if (lane == 0) {
-          if (band == 0) {
-#pragma unroll
-            for (int d = 0; d < D; ++d) { yi0[d] = bndy; yi1[d] = (T)0; }
-          } else {
-            const T* yb = ybuf + (size_t)(band - 1) * D * nx * 2;
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-              yi0[d] = yb[(d * nx + col) * 2];
-              yi1[d] = yb[(d * nx + col) * 2 + 1];
-            }
-          }
-        }
-        if (col == 0) {
-#pragma unroll
-          for (int d = 0; d < D; ++d) { tx0[d] = bndx; tx1[d] = (T)0; }
-        }
-        const int ix = sx > 0 ? col : nx - 1 - col;
-        const long long c = rowbase + ix;
-        const int reg = rowreg + xreg[ix];
-        if (sig_s) {
-          const T sg = sgs[buf * R4 + reg];
-          s0v *= sg; s1 *= sg; s2 *= sg; s3 *= sg;
-        }
-        s1 = sx > 0 ? s1 : -s1;
-        s2 = sy > 0 ? s2 : -s2;
-        s3 = (sx * sy) > 0 ? s3 : -s3;
-        T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
-        const T* tb = tab + (size_t)buf * D * R * 16;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          const T ax = al[d], by = be[d];
-          const T r0 = s0v + ax * tx0[d] + by * yi0[d];
-          const T r1 = s1 - S3 * ax * tx0[d] + by * yi1[d];
-          const T r2 = s2 + ax * tx1[d] - S3 * by * yi0[d];
-          const T r3 = s3 - S3 * (ax * tx1[d] + by * yi1[d]);
-          const T* L = tb + (d * R + reg) * 16;
-          T l[16];
-          Vec4<T>::load(L, l[0], l[1], l[2], l[3]);
-          Vec4<T>::load(L + 4, l[4], l[5], l[6], l[7]);
-          Vec4<T>::load(L + 8, l[8], l[9], l[10], l[11]);
-          Vec4<T>::load(L + 12, l[12], l[13], l[14], l[15]);
-          const T p0 = l[0] * r0 + l[1] * r1 + l[2] * r2 + l[3] * r3;
-          const T p1 = l[4] * r0 + l[5] * r1 + l[6] * r2 + l[7] * r3;
-          const T p2 = l[8] * r0 + l[9] * r1 + l[10] * r2 + l[11] * r3;
-          const T p3 = l[12] * r0 + l[13] * r1 + l[14] * r2 + l[15] * r3;
-          tx0[d] = p0 + S3 * p1;
-          tx1[d] = p2 + S3 * p3;
-          ty0[d] = p0 + S3 * p2;
-          ty1[d] = p1 + S3 * p3;
-          acc0 += wg[d] * p0;
-          acc1 += wg[d] * p1;
-          acc2 += wg[d] * p2;
-          acc3 += wg[d] * p3;
-          if (lane == 31 && band + 1 < nb) {
-            T* yb = ybuf + (size_t)band * D * nx * 2;
-            yb[(d * nx + col) * 2] = ty0[d];
-            yb[(d * nx + col) * 2 + 1] = ty1[d];
-          }
-        }
-        // odd modes back from the reflected frame (the task's directions share its quadrant)
-        acc1 = sx > 0 ? acc1 : -acc1;
-        acc2 = sy > 0 ? acc2 : -acc2;
-        acc3 = (sx * sy) > 0 ? acc3 : -acc3;
-        Vec4<T>::store(part + 4 * c, acc0, acc1, acc2, acc3);
-      }
-      if (nwarps > 1 && kk == PF - 1) __syncthreads();
-      else __syncwarp();
-    }
-  }
-}
-
 // 1D slab (P1, 2 dofs per cell): one thread per (instance, direction) marches its chain.
 template <typename T, typename TI, bool ANG>
 __global__ void k_sweep1d(SweepArgs a) {
@@ -1020,7 +718,7 @@ int launch_forward_cols(int dim, int nx, int ny, double hx, double hy, const UDi
 static int pick_D(const rte_problem* p, int prec, bool ang = false) {
   if (p->dim == 1) return 1;
   if (p->force_D > 0) return p->force_D;
-  if (p->pin_D > 0 && (p->dim == 1 || quadrant_gcd(p) % p->pin_D == 0)) return p->pin_D;
+  if (p->pin_D > 0 && quadrant_gcd(p) % p->pin_D == 0) return p->pin_D;
   if (p->tuned_D[prec][ang ? 1 : 0] > 0) return p->tuned_D[prec][ang ? 1 : 0];
   const bool f64 = prec != PREC_F32;
   const int nq = quadrant_gcd(p);
@@ -1055,11 +753,12 @@ static int ensure_tasks(rte_problem* p, int D) {
         for (int u = 0; u < p->nu; ++u) tasks.push_back(SweepTask{b, u, u, 0});
     } else {
       const int nquad = 4;
-      for (int q = 0; q < nquad; ++q) per_inst += (p->quad_start[q + 1] - p->quad_start[q]) / D;
+      for (int q = 0; q < nquad; ++q) per_inst += (p->quad_start[q + 1] - p->quad_start[q] + D - 1) / D;
       for (int b = 0; b < p->B; ++b) {
         int t = 0;
         for (int q = 0; q < nquad; ++q)
-          for (int u0 = p->quad_start[q]; u0 < p->quad_start[q + 1]; u0 += D) tasks.push_back(SweepTask{b, u0, t++, 0});
+          for (int u0 = p->quad_start[q]; u0 < p->quad_start[q + 1]; u0 += D)
+            tasks.push_back(SweepTask{b, u0, t++, std::min(D, p->quad_start[q + 1] - u0)});
       }
       // longest tasks first (instances with the most cells): a static longest-processing-time order
       std::stable_sort(tasks.begin(), tasks.end(), [&](const SweepTask& x, const SweepTask& y) {
@@ -1078,57 +777,7 @@ static int ensure_tasks(rte_problem* p, int D) {
   return RTE_OK;
 }
 
-// Dynamic shared memory above the 48 KB default must be granted per kernel with cudaFuncSetAttribute, which
-// acts on the current device only; granted[dev] remembers the size already granted on each device (zero-
-// initialised statics), so a process that drives several GPUs grants it on each of them.
-constexpr int kMaxDevices = 64;
-template <typename K>
-static int grant_smem(K kern, size_t smem, std::atomic<size_t>* granted) {
-  if (smem <= 48 * 1024) return RTE_OK;
-  int dev = 0;
-  RTE_CHECK_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) {
-    set_error("sweep: device ordinal beyond the supported range");
-    return RTE_ERR_UNSUPPORTED;
-  }
-  if (smem > granted[dev].load(std::memory_order_acquire)) {
-    RTE_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    granted[dev].store(smem, std::memory_order_release);
-  }
-  return RTE_OK;
-}
-
-// Runs of the pipelined band kernel for the task list of D directions per warp (the order of ensure_tasks):
-// consecutive tasks on meshes of one size, at most K each, K chosen so that the runs fill about two CTAs per SM
-// once.  Period P of a run: a multiple of 8 with P >= nx and 2 P >= 40 (nb - 1) + nx + 40 (the table buffer of
-// task k - 2 is free when task k's table is loaded; see k_sweep2d_pipe).
-static int ensure_runs(rte_problem* p, int D) {
-  if (p->nruns_by_D[D] > 0) return RTE_OK;
-  const int nt = p->ntasks_by_D[D];
-  std::vector<SweepTask> tasks(nt);
-  RTE_CHECK_CUDA(cudaMemcpy(tasks.data(), p->d_tasks_by_D[D].p, nt * sizeof(SweepTask), cudaMemcpyDeviceToHost));
-  int dev = 0, sms = 0;
-  RTE_CHECK_CUDA(cudaGetDevice(&dev));
-  RTE_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int target = std::max(1, 2 * sms);
-  const int K = p->pin_run > 0 ? p->pin_run : std::min(64, std::max(1, (nt + target - 1) / target));
-  std::vector<int4> runs;
-  for (int i = 0; i < nt;) {
-    const int nx = p->nx[tasks[i].b], ny = p->ny[tasks[i].b];
-    int j = i;
-    while (j < nt && j - i < K && p->nx[tasks[j].b] == nx && p->ny[tasks[j].b] == ny) ++j;
-    const int nb = (ny + 31) / 32;
-    int P = std::max(std::max(nx, 24), (40 * (nb - 1) + nx + 40 + 1) / 2);
-    P = (P + 7) & ~7;
-    runs.push_back(make_int4(i, j - i, P, 0));
-    i = j;
-  }
-  RTE_TRY(p->d_runs_by_D[D].alloc(runs.size()));
-  RTE_CHECK_CUDA(cudaMemcpy(p->d_runs_by_D[D].p, runs.data(), runs.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  p->nruns_by_D[D] = (int)runs.size();
-  return RTE_OK;
-}
-
+// Angular sweeps, sweeps with cross-section profiles, and the slab: D divides every quadrant's direction count.
 template <typename T, typename TI, bool ANG>
 static int launch_sweep_t(rte_problem* p, int D, SweepArgs& a, cudaStream_t st) {
   if (p->dim == 1) {
@@ -1192,106 +841,76 @@ static int launch_sweep_t(rte_problem* p, int D, SweepArgs& a, cudaStream_t st) 
       return RTE_OK;
     }
   }
-  if constexpr (!ANG) {
-    if (tv == 2 && nbands <= 8) {
-      // pipelined band kernel: persistent CTAs over runs of tasks
-      RTE_TRY(ensure_runs(p, D));
+  if constexpr (ANG) {
+    const bool band = tv >= 0 ? ((tv == 0 || tv == 2) && nbands <= 8) : (nbands <= 8 && !fp64_throughput && !ang_throughput);
+    if (band) {
+      // band-parallel kernel: one CTA per task, one warp per 32-row band
       const int W = nbands;
-      size_t elems = (size_t)2 * D * p->R * 16 + 2 * (size_t)((p->R + 3) & ~3) +
-                     (((size_t)(W > 1 ? W - 1 : 1) * D * maxnx * 2 + 3) & ~(size_t)3);
+      size_t elems = (size_t)D * p->R * 16 + ((p->R + 3) & ~3) + (((size_t)(W > 1 ? W - 1 : 1) * D * maxnx * 2 + 3) & ~(size_t)3);
       size_t smem = elems * sizeof(T) + (size_t)((maxnx + 3) & ~3) * sizeof(int) + 16;
+      smem += (size_t)W * 32 * D * 32 * sizeof(T);   // output staging rings
       if (smem > 227 * 1024) {
-        set_error("sweep: shared-memory table too large for the pipelined kernel");
+        set_error("sweep: shared-memory table too large for this mesh/region count");
         return RTE_ERR_UNSUPPORTED;
       }
-#define RTE_PIPE_CASE(DD)                                                                                   \
-  case DD: {                                                                                                \
-    auto kern = k_sweep2d_pipe<T, TI, DD>;                                                                  \
-    static std::atomic<size_t> granted[kMaxDevices];                                                        \
-    RTE_TRY(grant_smem(kern, smem, granted));                                                               \
-    kern<<<p->nruns_by_D[D], W * 32, smem, st>>>(a, p->d_runs_by_D[D].p);                                   \
-    count_launch();                                                                                         \
-    break;                                                                                                  \
-  }
-      switch (D) {
-        RTE_PIPE_CASE(1)
-        RTE_PIPE_CASE(2)
-        RTE_PIPE_CASE(4)
-        RTE_PIPE_CASE(8)
-        default:
-          set_error("sweep: unsupported directions-per-warp");
-          return RTE_ERR_UNSUPPORTED;
-      }
-#undef RTE_PIPE_CASE
-      RTE_CHECK_CUDA(cudaGetLastError());
-      return RTE_OK;
-    }
-  }
-  const bool band = tv >= 0 ? ((tv == 0 || tv == 2) && nbands <= 8) : (nbands <= 8 && !fp64_throughput && !ang_throughput);
-  if (band) {
-    // band-parallel kernel: one CTA per task, one warp per 32-row band
-    const int W = nbands;
-    size_t elems = (size_t)D * p->R * 16 + ((p->R + 3) & ~3) + (((size_t)(W > 1 ? W - 1 : 1) * D * maxnx * 2 + 3) & ~(size_t)3);
-    size_t smem = elems * sizeof(T) + (size_t)((maxnx + 3) & ~3) * sizeof(int) + 16;
-    if (ANG) smem += (size_t)W * 32 * D * 32 * sizeof(T);   // output staging rings
-    if (smem > 227 * 1024) {
-      set_error("sweep: shared-memory table too large for this mesh/region count");
-      return RTE_ERR_UNSUPPORTED;
-    }
 #define RTE_BAND_CASE(DD)                                                                                   \
   case DD: {                                                                                                \
-    auto kern = k_sweep2d_bands<T, TI, DD, ANG>;                                                            \
+    auto kern = k_sweep2d_bands<T, DD>;                                                            \
     static std::atomic<size_t> granted[kMaxDevices];                                                        \
     RTE_TRY(grant_smem(kern, smem, granted));                                                               \
     kern<<<a.ntasks, W * 32, smem, st>>>(a);                                                                \
     count_launch();                                                                                         \
     break;                                                                                                  \
-  }
-    switch (D) {
-      RTE_BAND_CASE(1)
-      RTE_BAND_CASE(2)
-      RTE_BAND_CASE(4)
-      RTE_BAND_CASE(8)
-      default:
-        set_error("sweep: unsupported directions-per-warp");
-        return RTE_ERR_UNSUPPORTED;
     }
+      switch (D) {
+        RTE_BAND_CASE(1)
+        RTE_BAND_CASE(2)
+        RTE_BAND_CASE(4)
+        RTE_BAND_CASE(8)
+        default:
+          set_error("sweep: unsupported directions-per-warp");
+          return RTE_ERR_UNSUPPORTED;
+      }
 #undef RTE_BAND_CASE
-    RTE_CHECK_CUDA(cudaGetLastError());
-    return RTE_OK;
-  }
-  a.smem_per_warp = D * p->R * 16 + D * maxnx * 2 + p->R;
-  a.smem_per_warp = (a.smem_per_warp + 3) & ~3;
-  size_t per_warp = (size_t)a.smem_per_warp * sizeof(T) + (ANG ? (size_t)32 * D * 32 * sizeof(T) : 0);
-  int wpb = 4;
-  while (wpb > 1 && per_warp * wpb > 96 * 1024) --wpb;
-  size_t smem = per_warp * wpb;
-  if (smem > 227 * 1024) {
-    set_error("sweep: shared-memory table too large for this mesh/region count");
-    return RTE_ERR_UNSUPPORTED;
-  }
-  int blocks = (a.ntasks + wpb - 1) / wpb;
+      RTE_CHECK_CUDA(cudaGetLastError());
+      return RTE_OK;
+    }
+    a.smem_per_warp = D * p->R * 16 + D * maxnx * 2 + p->R;
+    a.smem_per_warp = (a.smem_per_warp + 3) & ~3;
+    size_t per_warp = (size_t)a.smem_per_warp * sizeof(T) + (size_t)32 * D * 32 * sizeof(T);
+    int wpb = 4;
+    while (wpb > 1 && per_warp * wpb > 96 * 1024) --wpb;
+    size_t smem = per_warp * wpb;
+    if (smem > 227 * 1024) {
+      set_error("sweep: shared-memory table too large for this mesh/region count");
+      return RTE_ERR_UNSUPPORTED;
+    }
+    int blocks = (a.ntasks + wpb - 1) / wpb;
 #define RTE_SWEEP_CASE(DD)                                                                                  \
   case DD: {                                                                                                \
-    auto kern = k_sweep2d<T, TI, DD, ANG>;                                                                  \
+    auto kern = k_sweep2d<T, TI, DD, true>;                                                                  \
     static std::atomic<size_t> granted[kMaxDevices];                                                        \
     RTE_TRY(grant_smem(kern, smem, granted));                                                               \
     kern<<<blocks, wpb * 32, smem, st>>>(a);                                                                \
     count_launch();                                                                                         \
     break;                                                                                                  \
-  }
-  switch (D) {
-    RTE_SWEEP_CASE(1)
-    RTE_SWEEP_CASE(2)
-    RTE_SWEEP_CASE(4)
-    RTE_SWEEP_CASE(8)
-    default:
-      set_error("sweep: unsupported directions-per-warp");
-      return RTE_ERR_UNSUPPORTED;
-  }
+    }
+    switch (D) {
+      RTE_SWEEP_CASE(1)
+      RTE_SWEEP_CASE(2)
+      RTE_SWEEP_CASE(4)
+      RTE_SWEEP_CASE(8)
+      default:
+        set_error("sweep: unsupported directions-per-warp");
+        return RTE_ERR_UNSUPPORTED;
+    }
 #undef RTE_SWEEP_CASE
-  RTE_CHECK_CUDA(cudaGetLastError());
-  return RTE_OK;
+    RTE_CHECK_CUDA(cudaGetLastError());
+    return RTE_OK;
+  } else {
+    set_error("sweep: operator sweeps of region problems run in wavefront.cu");
+    return RTE_ERR_INVALID_ARG;
+  }
 }
 
 // Sigma_s of the fused scaling: per region, or the cell blocks of cross-section profiles
@@ -1300,7 +919,7 @@ static const void* sigma_s_arg(const rte_problem* p, bool f64) {
   return f64 ? (const void*)p->d_sig_s.p : (const void*)p->d_sig_s32.p;
 }
 
-static void fill_args(rte_problem* p, SweepArgs& a, int prec) {
+static void fill_args(rte_problem* p, SweepArgs& a, int prec, bool op = true) {
   std::memset(&a, 0, sizeof(a));
   a.inst = p->d_inst.p;
   a.udir = p->d_udir.p;
@@ -1311,6 +930,9 @@ static void fill_args(rte_problem* p, SweepArgs& a, int prec) {
   else
     a.linv = prec == PREC_F64 ? (const void*)p->d_linv64.p
                               : (prec == PREC_DF ? (const void*)p->d_linv_df.p : (const void*)p->d_linv32.p);
+  if (op && p->dim == 2 && !p->cellsig)
+    a.linv = prec == PREC_F64 ? (const void*)p->d_modal64.p
+                              : (prec == PREC_DF ? (const void*)p->d_modal_df.p : (const void*)p->d_rot32.p);
   a.inflow_mask = p->inflow_mask;
   a.tasks_per_inst = p->tasks_per_inst;
   a.ndir = p->ndir;
@@ -1325,23 +947,76 @@ static int ensure_partial(rte_problem* p, int prec) {
   return p->d_partial.ensure(bytes);
 }
 
-// Sweep autotuner: times every valid (kernel variant, directions per warp) pair for one precision and
-// output mode on this problem (two launches each after a warm-up, CUDA events on the stream) and keeps
-// the fastest.  Candidates: D in {1, 2, 4, 8} dividing the directions of a quadrant (FP64 and
-// double-float: D <= 4; angular output: D <= 4), variant band (ny <= 256) or warp-per-task.  The operator
-// apply is timed with its partial-sum reduction, since D also sets the number of partials.
+// Largest number of 32-row bands of the problem's meshes.
+static int max_bands(const rte_problem* p) {
+  int maxny = 0;
+  for (int b = 0; b < p->B; ++b) maxny = std::max(maxny, p->ny[b]);
+  return (maxny + 31) / 32;
+}
+
+// Launch shape of an operator sweep: a candidate being timed, a user's pin, the tuned shape, or the estimate's choice.
+static WaveShape op_shape(rte_problem* p, int prec) {
+  if (p->dim == 1 || p->cellsig) return WaveShape{pick_D(p, prec), 1, 1};
+  if (p->force_shape.D > 0) return p->force_shape;
+  if (p->pin_var >= 0) {
+    const int nb = std::min(max_bands(p), 8);
+    const WaveShape s{p->pin_D, p->pin_var == 0 ? nb : (p->pin_var == 1 ? 1 : std::min(nb, 2)), 1};
+    if (wave_shape_ok(p, prec, s) || prec == PREC_F32) return s;
+    return WaveShape{4, s.W, 1};   // the wider types take at most 8 (FP64) or 4 directions a task
+  }
+  if (p->tuned_shape[prec].D > 0) return p->tuned_shape[prec];
+  if (p->rule_shape[prec].D == 0) {
+    const std::vector<WaveShape> s = wave_shapes(p, prec, 1);
+    p->rule_shape[prec] = s.empty() ? WaveShape{1, 1, 1} : s[0];
+  }
+  return p->rule_shape[prec];
+}
+
+// Task list and partial-sum space of an operator sweep, and its launch with that shape.
+static int ensure_op(rte_problem* p, int prec, WaveShape s) {
+  RTE_TRY(ensure_tasks(p, s.D));
+  return ensure_partial(p, prec);
+}
+
+static int launch_op_sweep(rte_problem* p, int prec, WaveShape s, bool in64, SweepArgs& a, cudaStream_t st) {
+  if (p->dim == 2 && !p->cellsig) return launch_wave(p, prec, s, in64, a, st);
+  if (prec == PREC_DF) return launch_sweep_t<dfloat, dfloat, false>(p, s.D, a, st);
+  if (prec == PREC_F64) return launch_sweep_t<double, double, false>(p, s.D, a, st);
+  if (in64) return launch_sweep_t<float, double, false>(p, s.D, a, st);
+  return launch_sweep_t<float, float, false>(p, s.D, a, st);
+}
+
+// Sweep autotuner: times candidates for one precision and output mode on this problem (the best of a few launches each
+// after a warm-up, CUDA events on the stream) and keeps the fastest.  Operator sweeps of region problems: the shapes
+// that the cost estimate ranks first (wavefront.cu), four in FP32 where an apply is short and the estimate coarse, two
+// in the wider types.  Angular sweeps and cross-section profiles: every (kernel variant, directions per warp) pair with
+// D in {1, 2, 4, 8} dividing the directions of a quadrant (angular or FP64: D <= 4), variant band (ny <= 256) or
+// warp-per-task.  The operator apply is timed with its partial-sum reduction, since D also sets the number of partials.
 int autotune(rte_problem* p, int prec, bool ang, const void* src, void* psi, cudaStream_t st, bool scale_sigma_s,
              bool unique_layout) {
   const int fi = prec, ai = ang ? 1 : 0;
   const bool f64 = prec == PREC_F64;
   if (p->tuned_D[fi][ai] > 0 || p->dim == 1) return RTE_OK;
   const int nq = quadrant_gcd(p);
-  int maxny = 0;
-  for (int b = 0; b < p->B; ++b) maxny = std::max(maxny, p->ny[b]);
   RTE_TRY(p->d_tmp64.ensure((size_t)p->ntot));
-  // partials for the largest candidate task count (D = 1)
-  RTE_TRY(ensure_tasks(p, 1));
-  RTE_TRY(ensure_partial(p, prec));
+  struct Cand {
+    int D, var;
+    WaveShape shape;
+  };
+  std::vector<Cand> cands;
+  if (!ang && !p->cellsig) {
+    for (const WaveShape& s : wave_shapes(p, prec, prec == PREC_F32 ? 4 : 2)) cands.push_back({s.D, -1, s});
+  } else {
+    // partials for the largest candidate task count (D = 1)
+    RTE_TRY(ensure_tasks(p, 1));
+    RTE_TRY(ensure_partial(p, prec));
+    for (int var = 0; var < 2; ++var) {
+      if (p->cellsig && var != 1) continue;   // cross-section profiles: the warp-per-task kernel only
+      if (var == 0 && max_bands(p) > 8) continue;
+      for (int D : {1, 2, 4, 8})
+        if (nq % D == 0 && (prec == PREC_F32 || D <= 4) && (!ang || D <= 4)) cands.push_back({D, var, WaveShape{}});
+    }
+  }
   const void* in = src;
   // the FP32 operator is timed with an FP32 input and output, as the inner solves launch it
   const bool in32 = prec == PREC_F32 && !ang && !src;
@@ -1356,51 +1031,47 @@ int autotune(rte_problem* p, int prec, bool ang, const void* src, void* psi, cud
   RTE_CHECK_CUDA(cudaEventCreate(&e0));
   RTE_CHECK_CUDA(cudaEventCreate(&e1));
   float best = 1e30f;
-  int bestD = 0, bestV = -1;
-  for (int var = 0; var < 3; ++var) {
-    if (p->cellsig && var != 1) continue;   // cross-section profiles: the warp-per-task kernel only
-    if ((var == 0 || var == 2) && (maxny + 31) / 32 > 8) continue;
-    if (var == 2 && ang) continue;   // the pipelined kernel has no angular output
-    for (int D : {1, 2, 4, 8}) {
-      if (nq % D || (prec != PREC_F32 && D > 4) || (ang && D > 4)) continue;
-      p->force_D = D;
-      p->force_var = var;
-      // one warm-up launch, then the best of five timed launches (robust to a slow outlier)
-      int rc = RTE_OK;
-      float cand = 1e30f;
-      for (int rep = 0; rep < 6 && rc == RTE_OK; ++rep) {
-        if (rep > 0) cudaEventRecord(e0, st);
-        if (ang) rc = launch_angular(p, f64, in, 0, psi, st, scale_sigma_s, unique_layout);
-        else if (in32) rc = launch_T(p, MODE_OP, false, in, false, nullptr, p->d_tmp32.p + p->ntot, false, nullptr, st);
-        else if (prec == PREC_DF)
-          rc = launch_T_df(p, MODE_OP, reinterpret_cast<const double*>(in), nullptr, p->d_tmp64.p, nullptr, st);
-        else rc = launch_T(p, MODE_OP, f64, in, !f64 && src ? false : true, nullptr, p->d_tmp64.p, true, nullptr, st);
-        if (rep > 0 && rc == RTE_OK) {
-          float ms = 0.f;
-          cudaEventRecord(e1, st);
-          cudaEventSynchronize(e1);
-          if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) cand = std::min(cand, ms);
-        }
+  Cand pick{0, -1, WaveShape{}};
+  const int reps = ang || p->cellsig ? 6 : 4;
+  for (const Cand& c : cands) {
+    p->force_D = c.D;
+    p->force_var = c.var;
+    p->force_shape = c.shape;
+    // one warm-up launch, then the best of the timed ones (robust to a slow outlier)
+    int rc = RTE_OK;
+    float cand = 1e30f;
+    for (int rep = 0; rep < reps && rc == RTE_OK; ++rep) {
+      if (rep > 0) cudaEventRecord(e0, st);
+      if (ang) rc = launch_angular(p, f64, in, 0, psi, st, scale_sigma_s, unique_layout);
+      else if (in32) rc = launch_T(p, MODE_OP, false, in, false, nullptr, p->d_tmp32.p + p->ntot, false, nullptr, st);
+      else if (prec == PREC_DF)
+        rc = launch_T_df(p, MODE_OP, reinterpret_cast<const double*>(in), nullptr, p->d_tmp64.p, nullptr, st);
+      else rc = launch_T(p, MODE_OP, f64, in, !f64 && src ? false : true, nullptr, p->d_tmp64.p, true, nullptr, st);
+      if (rep > 0 && rc == RTE_OK) {
+        float ms = 0.f;
+        cudaEventRecord(e1, st);
+        cudaEventSynchronize(e1);
+        if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) cand = std::min(cand, ms);
       }
-      if (rc == RTE_OK && cand < best) {
-        best = cand;
-        bestD = D;
-        bestV = var;
-      }
-      cudaGetLastError();
     }
+    if (rc == RTE_OK && cand < best) {
+      best = cand;
+      pick = c;
+    }
+    cudaGetLastError();
   }
+  p->force_shape = WaveShape{};
   p->force_D = 0;
   p->force_var = -1;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (bestD == 0) {
+  if (pick.D == 0) {
     set_error("sweep autotuner: no candidate ran");
     return RTE_ERR_CUDA;
   }
-  p->tuned_D[fi][ai] = bestD;
-  p->tuned_var[fi][ai] = bestV;
-  p->tuned_ms[fi][ai] = best;
+  p->tuned_D[fi][ai] = pick.D;
+  p->tuned_var[fi][ai] = pick.var;
+  if (!ang) p->tuned_shape[fi] = pick.shape;
   return RTE_OK;
 }
 
@@ -1415,8 +1086,7 @@ int prepare_sweeps(rte_problem* p) {
   size_t bytes = 0;
   for (int prec : {PREC_F32, PREC_F64, PREC_DF}) {
     if (p->cellsig && prec == PREC_DF) continue;
-    RTE_TRY(ensure_tasks(p, pick_D(p, prec)));
-    if (p->dim == 2) RTE_TRY(ensure_runs(p, pick_D(p, prec)));   // the pipelined kernel's runs, before any capture
+    RTE_TRY(ensure_tasks(p, op_shape(p, prec).D));
     bytes = std::max(bytes, (size_t)p->tasks_per_inst * (size_t)p->ntot * (size_t)(prec == PREC_F32 ? 4 : 8));
   }
   return p->d_partial.ensure(bytes);
@@ -1442,9 +1112,8 @@ int launch_T_df(rte_problem* p, int mode, const double* x, const double* bvec, d
     return RTE_ERR_UNSUPPORTED;
   }
   RTE_TRY(p->d_xdf.ensure((size_t)2 * p->ntot));
-  const int D = pick_D(p, PREC_DF);
-  RTE_TRY(ensure_tasks(p, D));
-  RTE_TRY(ensure_partial(p, PREC_DF));
+  const WaveShape shape = op_shape(p, PREC_DF);
+  RTE_TRY(ensure_op(p, PREC_DF, shape));
   float2* xdf = reinterpret_cast<float2*>(p->d_xdf.p);
   k_split_df<<<(unsigned)std::min<long long>(4096, (p->ntot + 255) / 256), 256, 0, st>>>(x, p->ntot, xdf);
   count_launch();
@@ -1455,7 +1124,7 @@ int launch_T_df(rte_problem* p, int mode, const double* x, const double* bvec, d
   a.sig_s = p->d_sig_s_df.p;
   a.partial = p->d_partial.p;
   a.active = d_active;
-  RTE_TRY((launch_sweep_t<dfloat, dfloat, false>(p, D, a, st)));
+  RTE_TRY(launch_op_sweep(p, PREC_DF, shape, true, a, st));
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
   dim3 grid((maxn + 255) / 256, p->B);
@@ -1469,9 +1138,8 @@ int launch_T_df(rte_problem* p, int mode, const double* x, const double* bvec, d
 int launch_T(rte_problem* p, int mode, bool f64, const void* src, bool in_f64, const void* bvec, void* out,
              bool out_f64, const int* d_active, cudaStream_t st) {
   const int prec = f64 ? PREC_F64 : PREC_F32;
-  int D = pick_D(p, prec);
-  RTE_TRY(ensure_tasks(p, D));
-  RTE_TRY(ensure_partial(p, prec));
+  const WaveShape shape = op_shape(p, prec);
+  RTE_TRY(ensure_op(p, prec, shape));
   SweepArgs a;
   fill_args(p, a, prec);
   a.src = mode == MODE_RHS ? (const void*)p->d_G.p : src;
@@ -1481,13 +1149,7 @@ int launch_T(rte_problem* p, int mode, bool f64, const void* src, bool in_f64, c
                                                    : nullptr;
   a.partial = p->d_partial.p;
   a.active = d_active;
-  if (f64) {
-    if (src64) RTE_TRY((launch_sweep_t<double, double, false>(p, D, a, st)));
-    else RTE_TRY((launch_sweep_t<double, float, false>(p, D, a, st)));
-  } else {
-    if (src64) RTE_TRY((launch_sweep_t<float, double, false>(p, D, a, st)));
-    else RTE_TRY((launch_sweep_t<float, float, false>(p, D, a, st)));
-  }
+  RTE_TRY(launch_op_sweep(p, prec, shape, src64, a, st));
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
   dim3 grid((maxn + 255) / 256, p->B);
@@ -1517,23 +1179,15 @@ int launch_T(rte_problem* p, int mode, bool f64, const void* src, bool in_f64, c
 // subtraction z - sum_t partial_t is left to the caller's kernel (the fused Arnoldi step).
 int launch_op_partials(rte_problem* p, bool f64, const void* z, bool in_f64, const int* d_active, cudaStream_t st) {
   const int prec = f64 ? PREC_F64 : PREC_F32;
-  int D = pick_D(p, prec);
-  RTE_TRY(ensure_tasks(p, D));
-  RTE_TRY(ensure_partial(p, prec));
+  const WaveShape shape = op_shape(p, prec);
+  RTE_TRY(ensure_op(p, prec, shape));
   SweepArgs a;
   fill_args(p, a, prec);
   a.src = z;
   a.sig_s = sigma_s_arg(p, f64);
   a.partial = p->d_partial.p;
   a.active = d_active;
-  if (f64) {
-    if (in_f64) RTE_TRY((launch_sweep_t<double, double, false>(p, D, a, st)));
-    else RTE_TRY((launch_sweep_t<double, float, false>(p, D, a, st)));
-  } else {
-    if (in_f64) RTE_TRY((launch_sweep_t<float, double, false>(p, D, a, st)));
-    else RTE_TRY((launch_sweep_t<float, float, false>(p, D, a, st)));
-  }
-  return RTE_OK;
+  return launch_op_sweep(p, prec, shape, in_f64, a, st);
 }
 
 // A~ z (mode OP) with caller-provided task list and partial-sum storage: allocates nothing.  D must be
@@ -1550,7 +1204,8 @@ int launch_op_external(rte_problem* p, bool f64, const void* z, void* w, const S
   a.udir = p->d_udir.p;
   a.tasks = tasks;
   a.ntasks = ntasks;
-  a.linv = f64 ? (const void*)p->d_linv64.p : (const void*)p->d_linv32.p;
+  if (p->dim == 1) a.linv = f64 ? (const void*)p->d_linv64.p : (const void*)p->d_linv32.p;
+  else a.linv = f64 ? (const void*)p->d_modal64.p : (const void*)p->d_rot32.p;
   a.inflow_mask = p->inflow_mask;
   a.tasks_per_inst = tasks_per_inst;
   a.ndir = p->ndir;
@@ -1561,8 +1216,8 @@ int launch_op_external(rte_problem* p, bool f64, const void* z, void* w, const S
   a.src = z;
   a.sig_s = sigma_s_arg(p, f64);
   a.partial = partial;
-  if (f64) RTE_TRY((launch_sweep_t<double, double, false>(p, D, a, st)));
-  else RTE_TRY((launch_sweep_t<float, float, false>(p, D, a, st)));
+  const int prec = f64 ? PREC_F64 : PREC_F32;
+  RTE_TRY(launch_op_sweep(p, prec, p->dim == 2 ? wave_shape_for(p, prec, D) : WaveShape{1, 1, 1}, f64, a, st));
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
   dim3 grid((maxn + 255) / 256, p->B);
@@ -1587,7 +1242,7 @@ int launch_angular(rte_problem* p, bool f64, const void* src, int with_bc, void*
   RTE_TRY(ensure_tasks(p, D));
   RTE_TRY(ensure_partial(p, prec));
   SweepArgs a;
-  fill_args(p, a, prec);
+  fill_args(p, a, prec, false);
   a.src = src;
   a.with_bc = with_bc ? 1 : 0;
   a.partial = p->d_partial.p;
@@ -1656,11 +1311,6 @@ int rte_apply_op(rte_problem_t p, int dtype, const void* z, void* w, void* strea
 int rte_problem_set_sweep_variant(rte_problem_t p, int variant, int directions_per_warp, int tasks_per_run) {
   RTE_ARG(p, "null handle");
   RTE_ARG(tasks_per_run >= 0 && tasks_per_run <= 64, "tasks_per_run must be in [0, 64]");
-  if (tasks_per_run != p->pin_run) {
-    // runs are rebuilt with the new length
-    p->pin_run = tasks_per_run;
-    for (int d = 0; d < 17; ++d) p->nruns_by_D[d] = 0;
-  }
   if (variant < 0) {
     p->pin_var = -1;
     p->pin_D = 0;
