@@ -55,20 +55,31 @@ __device__ double block_sum(double v, double* sh) {
   return sh[32];
 }
 
-// Norms accumulate in FP64 whatever the vector type (one launch per restart, not per iteration).
+// Norms accumulate in FP64 whatever the vector type.  Grid (pieces, B): piece x of an instance's dofs; with one piece the
+// norm itself, else the piece's sum of squares, which k_norm_sum adds up in a fixed order.  One block per instance reads
+// 262,144 dofs in 240 us (the latency of one SM); 64 pieces and their sum take 12.
 template <typename TV>
 __global__ void k_norm(const TV* x, const InstInfo* inst, const int* active, double* out) {
   __shared__ double sh[33];
-  const int b = blockIdx.x;
+  const int b = blockIdx.y, np = gridDim.x;
   if (active && !active[b]) return;
   const InstInfo in = inst[b];
   double s = 0.0;
-  for (int i = threadIdx.x; i < in.ndof; i += blockDim.x) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < in.ndof; i += np * blockDim.x) {
     double v = (double)x[in.off + i];
     s += v * v;
   }
   s = block_sum(s, sh);
-  if (threadIdx.x == 0) out[b] = sqrt(s);
+  if (threadIdx.x == 0) out[(size_t)b * np + blockIdx.x] = np == 1 ? sqrt(s) : s;
+}
+
+__global__ void k_norm_sum(const double* part, int np, const int* active, double* out) {
+  const int b = blockIdx.x, lane = threadIdx.x;
+  if (active && !active[b]) return;
+  double s = 0.0;
+  for (int i = lane; i < np; i += 32) s += part[(size_t)b * np + i];
+  s = warp_sum(s);
+  if (lane == 0) out[b] = sqrt(s);
 }
 
 __global__ void k_linf(const double* x, const InstInfo* inst, double* out) {
@@ -501,11 +512,13 @@ __global__ void __launch_bounds__(256) k_arnoldi_coop(ArnArgs<TP, TV> A) {
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int r = r0 + warp + 8 * q;
+        if (r >= j) break;   // uniform for the warp; the loads above stay unconditional, the arithmetic (FP64) does not
         const TV lr = sl[min(m + 1 + r, 2 * m + 1)];
         TV s = 0;
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
           const int k = lane + 32 * p;
+          if (32 * p >= r) break;
           const bool tri = r < j && k < r;
           s += tri ? tv[q][p] * sl[k] : TV(0);
           cacc[p] += tri ? lr * tv[q][p] : TV(0);
@@ -764,10 +777,13 @@ __global__ void __launch_bounds__(256) k_arnoldi_coop(ArnArgs<TP, TV> A) {
 // h = T a; norm, Givens and flags) runs once per instance, in phases of its own between grid-wide
 // barriers (five phases, four barriers), and the preconditioner is a separate launch.  Compared with
 // k_arnoldi_coop this adds barriers but does not repeat any reduction, which is the better trade
-// once the chunks of the batch fill the GPU several times over.
+// once the chunks of the batch fill the GPU several times over.  Every block takes one run of consecutive chunks and adds
+// up the dot products of those that belong to one instance before it writes them, so the per-instance sums run over a
+// few dozen pieces instead of a thousand chunks (16 instances of 256^2: 260 -> 171 us an iteration, of which the Krylov
+// basis read twice and the partial fluxes are 90 us at the copy bandwidth).
 template <typename TP, typename TV>
 __global__ void __launch_bounds__(256) k_arnoldi_wide(
-    int B, const int2* items, int nitems, const InstInfo* inst, int* active, const TP* partial, int ntask,
+    int B, const int2* items, const int* item0, int nitems, const InstInfo* inst, int* active, const TP* partial, int ntask,
     const TV* z, TV* V, long long ntot, int j, int m, int nchunk, TV* part, TV* npart, TV* Tm, int ldT,
     double* H, double* Hraw, double* w0, double* cs, double* sn, double* g, int* brk, const double* bnorm,
     const double* rtol_p, int* iters_left, double* est, int* flag, int* kcols, double* hnorm, int* active0) {
@@ -781,9 +797,22 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
   //     a_k = v_k . w (k <= j), g_k = v_k . v_j (k < j), w . w.  w and v_j are staged in shared memory
   //     and warp q owns k = q, q + 8, ...: its reductions are independent of the other warps'.
   __shared__ TV wsh[256], vjsh[256];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+  const int per = (nitems + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int it0 = min(nitems, (int)blockIdx.x * per), it1 = min(nitems, it0 + per);
+  // pieces of an instance's chunk sums: one per block that holds chunks of it, stored at the piece's first chunk
+  auto pieces = [&](int b, int nch, auto&& at) {   // this lane's share: at(chunk where a piece is stored)
+    const int first = item0[b], k0 = first / per, k1 = (first + nch - 1) / per;
+    for (int k = k0 + lane; k <= k1; k += 32) at(max(0, k * per - first));
+  };
+  int start = it0;   // first chunk of the current piece
+  for (int it = it0; it < it1; ++it) {
     const int b = items[it].x, ch = items[it].y;
+    const bool fresh = it == it0 || items[it - 1].x != b, done = it + 1 == it1 || items[it + 1].x != b;
+    if (fresh) start = ch;
     if (!active[b]) continue;
+    if (fresh) {
+      for (int t = threadIdx.x; t < nslot; t += blockDim.x) red[t] = 0;
+    }
     const InstInfo in = inst[b];
     const int i0 = ch * 256;
     const int i = i0 + threadIdx.x;
@@ -815,8 +844,8 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
       a = warp_sum_t(a);
       gg = warp_sum_t(gg);
       if (lane == 0) {
-        red[kk] = a;
-        if (kk < j) red[m + 1 + kk] = gg;
+        red[kk] += a;
+        if (kk < j) red[m + 1 + kk] += gg;
       }
     }
     if (warp == 7) {
@@ -824,30 +853,33 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
 #pragma unroll
       for (int e = 0; e < 8; ++e) ww += wsh[lane + 32 * e] * wsh[lane + 32 * e];
       ww = warp_sum_t(ww);
-      if (lane == 0) red[2 * m + 2] = ww;
+      if (lane == 0) red[2 * m + 2] += ww;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < nslot; t += blockDim.x) {
-      const bool used = t <= j || (t >= m + 1 && t < m + 1 + j) || t == 2 * m + 2;
-      if (used) part[((size_t)b * nslot + t) * nchunk + ch] = red[t];
+    if (done) {
+      for (int t = threadIdx.x; t < nslot; t += blockDim.x) {
+        const bool used = t <= j || (t >= m + 1 && t < m + 1 + j) || t == 2 * m + 2;
+        if (used) part[((size_t)b * nslot + t) * nchunk + start] = red[t];
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
   grid.sync();
   // P1: per instance: sum the chunk partials, grow T = (I + L)^{-1} by the new row, h = T a
   for (int b = blockIdx.x; b < B; b += gridDim.x) {
     if (!active[b]) continue;
     const int nch = (inst[b].ndof + 255) / 256;
-    for (int t = threadIdx.x; t < nslot; t += blockDim.x) {
-      const bool used = t <= j || (t >= m + 1 && t < m + 1 + j) || t == 2 * m + 2;
-      if (!used) continue;
+    for (int u = warp; u < 2 * j + 2; u += 8) {   // used slots a_0 .. a_j, l_0 .. l_{j-1}, w.w; lanes over the pieces
+      const int t = u <= j ? u : (u < 2 * j + 1 ? m + 1 + (u - j - 1) : 2 * m + 2);
       const TV* pp = part + ((size_t)b * nslot + t) * nchunk;
       TV acc = 0;
-#pragma unroll 16
-      for (int c = 0; c < nch; ++c) acc += pp[c];
-      if (t <= j) as[t] = acc;
-      else if (t < m + 1 + j) ls[t - m - 1] = acc;
-      else w0[b] = sqrt((double)acc);
+      pieces(b, nch, [&](int c) { acc += pp[c]; });
+      acc = warp_sum_t(acc);
+      if (lane == 0) {
+        if (t <= j) as[t] = acc;
+        else if (t < m + 1 + j) ls[t - m - 1] = acc;
+        else w0[b] = sqrt((double)acc);
+      }
     }
     __syncthreads();
     TV* Tb = Tm + (size_t)b * (m + 1) * ldT;
@@ -873,31 +905,39 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
   }
   grid.sync();
   // P2: w -= sum_k h_k v_k over the chunk, partial ||w||^2
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+  TV s2 = 0;   // this thread's share of the piece's ||w||^2
+  for (int it = it0; it < it1; ++it) {
     const int b = items[it].x, ch = items[it].y;
+    const bool fresh = it == it0 || items[it - 1].x != b, done = it + 1 == it1 || items[it + 1].x != b;
+    if (fresh) start = ch;
     if (!active[b]) continue;
     const InstInfo in = inst[b];
-    const double* h = H + ((size_t)b * m + j) * (m + 1);
-    for (int t = threadIdx.x; t <= j; t += blockDim.x) hsv[t] = (TV)h[t];
-    __syncthreads();
+    if (fresh) {
+      const double* h = H + ((size_t)b * m + j) * (m + 1);
+      __syncthreads();
+      for (int t = threadIdx.x; t <= j; t += blockDim.x) hsv[t] = (TV)h[t];
+      __syncthreads();
+      s2 = 0;
+    }
     const int i = ch * 256 + threadIdx.x;
-    TV s2 = 0;
     if (i < in.ndof) {
       TV wi = V[(size_t)(j + 1) * ntot + in.off + i];
 #pragma unroll 16
       for (int kk = 0; kk <= j; ++kk) wi -= hsv[kk] * V[(size_t)kk * ntot + in.off + i];
       V[(size_t)(j + 1) * ntot + in.off + i] = wi;
-      s2 = wi * wi;
+      s2 += wi * wi;
     }
-    s2 = warp_sum_t(s2);
-    if (lane == 0) red[warp] = s2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      TV tot = 0;
-      for (int w = 0; w < 8; ++w) tot += red[w];
-      npart[(size_t)b * nchunk + ch] = tot;
+    if (done) {
+      s2 = warp_sum_t(s2);
+      __syncthreads();
+      if (lane == 0) red[warp] = s2;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        TV tot = 0;
+        for (int w = 0; w < 8; ++w) tot += red[w];
+        npart[(size_t)b * nchunk + start] = tot;
+      }
     }
-    __syncthreads();
   }
   grid.sync();
   // P3: per instance: h_{j+1,j} = ||w||, breakdown test, Givens rotation, stopping flags
@@ -918,7 +958,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
     if (warp == 0) {
       const int nch = (inst[b].ndof + 255) / 256;
       TV acc = 0;
-      for (int cc = lane; cc < nch; cc += 32) acc += npart[(size_t)b * nchunk + cc];
+      pieces(b, nch, [&](int c) { acc += npart[(size_t)b * nchunk + c]; });
       acc = warp_sum_t(acc);
       if (lane == 0) red[0] = acc;
     }
@@ -966,7 +1006,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
   }
   grid.sync();
   // P4: v_{j+1} = w / h_{j+1,j}
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+  for (int it = it0; it < it1; ++it) {
     const int b = items[it].x, ch = items[it].y;
     if (!active0[b] || brk[b]) continue;
     const InstInfo in = inst[b];
@@ -1083,6 +1123,7 @@ struct Ws {
   // fused iteration kernels: vector chunks (instance, 256-dof chunk), per-instance ROM data, and the
   // co-resident grid sizes of the cooperative launches
   DevBuf<int2> items;
+  DevBuf<int> item0;            // [B] first item of each instance
   int nitems = 0;
   DevBuf<RomInstDev> rominst;
   DevBuf<double> rpart, rc;
@@ -1096,7 +1137,7 @@ struct Ws {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second.exec);
     graphs.clear();
   }
-  DevBuf<double> bnorm, beta, est, nrm;
+  DevBuf<double> bnorm, beta, est, nrm, norm_part;
   DevBuf<int> active, brk, flag, kcols, iters_left, list;
   DevBuf<double> rom_y, rom_c;
   // learned ROMSAD slot: per-instance flag and coefficients c_hat / beta (FP64 and FP32)
@@ -1136,13 +1177,17 @@ struct Ws {
     RTE_TRY(Lt.alloc((size_t)B * (m + 1) * (m + 1)));
     {
       std::vector<int2> it;
+      std::vector<int> first(p->B);
       for (int b = 0; b < p->B; ++b) {
+        first[b] = (int)it.size();
         const int nb = (int)((p->off[b + 1] - p->off[b] + 255) / 256);
         for (int c = 0; c < nb; ++c) it.push_back(make_int2(b, c));
       }
       nitems = (int)it.size();
       RTE_TRY(items.alloc(it.size()));
       RTE_CHECK_CUDA(cudaMemcpy(items.p, it.data(), it.size() * sizeof(int2), cudaMemcpyHostToDevice));
+      RTE_TRY(item0.alloc(B));
+      RTE_CHECK_CUDA(cudaMemcpy(item0.p, first.data(), B * sizeof(int), cudaMemcpyHostToDevice));
       RTE_TRY(rominst.alloc(B));
       RTE_TRY(rpart.alloc((size_t)B * nchunk * 64));
       RTE_TRY(rc.alloc((size_t)B * 64));
@@ -1185,6 +1230,7 @@ struct Ws {
     RTE_TRY(ro.alloc(ntot));
     RTE_TRY(d.alloc(ntot));
     RTE_TRY(bnorm.alloc(B));
+    RTE_TRY(norm_part.alloc((size_t)B * 64));
     RTE_TRY(beta.alloc(B));
     RTE_TRY(est.alloc(B));
     RTE_TRY(nrm.alloc(B));
@@ -1232,6 +1278,20 @@ static dim3 vec_grid(rte_problem* p) {
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
   return dim3((maxn + 255) / 256, p->B);
+}
+
+// out[b] = ||x_b||_2 of the active instances
+template <typename TV>
+static int launch_norm(rte_problem* p, Ws& W, const TV* x, const int* active, double* out, cudaStream_t st) {
+  const int np = std::min(64, std::max(1, W.nchunk / 16));   // at least 4096 dofs a piece
+  k_norm<<<dim3(np, p->B), 512, 0, st>>>(x, p->d_inst.p, active, np == 1 ? out : W.norm_part.p);
+  count_launch();
+  if (np > 1) {
+    k_norm_sum<<<p->B, 32, 0, st>>>(W.norm_part.p, np, active, out);
+    count_launch();
+  }
+  RTE_CHECK_CUDA(cudaGetLastError());
+  return RTE_OK;
 }
 
 // Per-instance outcome of one inner (or FP64) FGMRES run.
@@ -1290,8 +1350,7 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
   std::vector<double> hb(B), hbn(B);
   // ||rhs||
   RTE_CHECK_CUDA(cudaMemcpyAsync(W.active.p, act.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-  k_norm<<<B, 512, 0, st>>>(rhs, p->d_inst.p, W.active.p, W.bnorm.p);
-  count_launch();
+  RTE_TRY(launch_norm(p, W, rhs, W.active.p, W.bnorm.p, st));
   // r0
   if (zero_guess) {
     k_copy_active<<<vg, 256, 0, st>>>(rb, rhs, p->d_inst.p, W.active.p);
@@ -1311,8 +1370,7 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
   while (true) {
     // beta = ||r||
     RTE_CHECK_CUDA(cudaMemcpyAsync(W.active.p, act.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-    k_norm<<<B, 512, 0, st>>>(rb, p->d_inst.p, W.active.p, W.beta.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, W, rb, W.active.p, W.beta.p, st));
     RTE_CHECK_CUDA(cudaMemcpyAsync(hb.data(), W.beta.p, B * 8, cudaMemcpyDeviceToHost, st));
     RTE_CHECK_CUDA(cudaStreamSynchronize(st));
     int nact = 0;
@@ -1439,7 +1497,8 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
           int* kc_p = W.kcols.p;
           double* hn_p = W.hnorm.p;
           int* a0_p = W.active0.p;
-          void* args[] = {&Bv, &it_p, &nit, &inst_p, &act_p, &part_p, &ntask, &z_p, &V_p, &nt, &jj, &mm, &nch,
+          const int* i0_p = W.item0.p;
+          void* args[] = {&Bv, &it_p, &i0_p, &nit, &inst_p, &act_p, &part_p, &ntask, &z_p, &V_p, &nt, &jj, &mm, &nch,
                           &dp_p, &np_p, &Lt_p, &ldT, &H_p, &Hr_p, &w0_p, &cs_p, &sn_p, &g_p, &brk_p, &bn_p, &rt_p,
                           &il_p, &est_p, &fl_p, &kc_p, &hn_p, &a0_p};
           RTE_CHECK_CUDA(cudaLaunchCooperativeKernel((const void*)k_arnoldi_wide<TP, TV>,
@@ -1595,8 +1654,7 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
     for (int b = 0; b < B; ++b) act[b] = mask[b];
     // check-sweep instances: the loop head computes beta and stops them if within 2 rtol
     if (true_check) {
-      k_norm<<<B, 512, 0, st>>>(rb, p->d_inst.p, W.active.p, W.nrm.p);
-      count_launch();
+      RTE_TRY(launch_norm(p, W, rb, W.active.p, W.nrm.p, st));
       std::vector<double> hn(B);
       RTE_CHECK_CUDA(cudaMemcpyAsync(hn.data(), W.nrm.p, B * 8, cudaMemcpyDeviceToHost, st));
       RTE_CHECK_CUDA(cudaStreamSynchronize(st));
@@ -1823,8 +1881,7 @@ extern "C" int fgmres_solve(rte_problem_t p, const romsad_t* roms, const fgmres_
     // can raise the residual in fast ones.)
     std::vector<int> all1(B, 1);
     RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, all1.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-    k_norm<<<B, 512, 0, st>>>(x, p->d_inst.p, ws->active.p, ws->nrm.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, *ws, x, ws->active.p, ws->nrm.p, st));
     std::vector<double> hx(B);
     RTE_CHECK_CUDA(cudaMemcpyAsync(hx.data(), ws->nrm.p, B * 8, cudaMemcpyDeviceToHost, st));
     RTE_CHECK_CUDA(cudaStreamSynchronize(st));
@@ -1850,8 +1907,7 @@ extern "C" int fgmres_solve(rte_problem_t p, const romsad_t* roms, const fgmres_
   if (o->learned_slot && roms && !warm) {
     std::vector<int> all1(B, 1);
     RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, all1.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-    k_norm<<<B, 512, 0, st>>>(ws->bt.p, p->d_inst.p, ws->active.p, ws->beta.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, *ws, ws->bt.p, ws->active.p, ws->beta.p, st));
     std::vector<double> hb(B), cs((size_t)B * 64, 0.0);
     RTE_CHECK_CUDA(cudaMemcpyAsync(hb.data(), ws->beta.p, B * 8, cudaMemcpyDeviceToHost, st));
     std::vector<std::pair<romsad_t, int>> groups;
@@ -1958,14 +2014,12 @@ extern "C" int fgmres_solve(rte_problem_t p, const romsad_t* roms, const fgmres_
     const double kPredict = 0.5;
     std::vector<double> hb(B), hr(B), hprev(B, 0.0);
     RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, act.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-    k_norm<<<B, 512, 0, st>>>(ws->bt.p, p->d_inst.p, ws->active.p, ws->nrm.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, *ws, ws->bt.p, ws->active.p, ws->nrm.p, st));
     RTE_CHECK_CUDA(cudaMemcpyAsync(hb.data(), ws->nrm.p, B * 8, cudaMemcpyDeviceToHost, st));
     RTE_CHECK_CUDA(cudaStreamSynchronize(st));
     auto read_norms = [&]() -> int {
       RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, act.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-      k_norm<<<B, 512, 0, st>>>(ro, p->d_inst.p, ws->active.p, ws->nrm.p);
-      count_launch();
+      RTE_TRY(launch_norm(p, *ws, ro, ws->active.p, ws->nrm.p, st));
       RTE_CHECK_CUDA(cudaMemcpyAsync(hr.data(), ws->nrm.p, B * 8, cudaMemcpyDeviceToHost, st));
       RTE_CHECK_CUDA(cudaStreamSynchronize(st));
       return RTE_OK;
@@ -2113,10 +2167,8 @@ extern "C" int fgmres_solve(rte_problem_t p, const romsad_t* roms, const fgmres_
     const double* rfin = o->mode != RTE_MODE_FP64 ? ws->ro.p : ws->r.p;
     std::vector<int> all1(B, 1);
     RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, all1.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-    k_norm<<<B, 512, 0, st>>>(rfin, p->d_inst.p, ws->active.p, ws->nrm.p);
-    count_launch();
-    k_norm<<<B, 512, 0, st>>>(ws->bt.p, p->d_inst.p, ws->active.p, ws->beta.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, *ws, rfin, ws->active.p, ws->nrm.p, st));
+    RTE_TRY(launch_norm(p, *ws, ws->bt.p, ws->active.p, ws->beta.p, st));
     k_linf<<<B, 512, 0, st>>>(rfin, p->d_inst.p, ws->est.p);
     count_launch();
     std::vector<double> hn(B), hb(B), hl(B);
@@ -2226,8 +2278,7 @@ extern "C" int si_solve(rte_problem_t p, const romsad_t* roms, const fgmres_opts
   RTE_TRY(launch_T(p, MODE_RHS, true, nullptr, true, nullptr, ws->bt.p, true, nullptr, st));
   std::vector<int> act(B, 1), sub(B, 0);
   RTE_CHECK_CUDA(cudaMemcpyAsync(ws->active.p, act.data(), B * sizeof(int), cudaMemcpyHostToDevice, st));
-  k_norm<<<B, 512, 0, st>>>(ws->bt.p, p->d_inst.p, ws->active.p, ws->bnorm.p);
-  count_launch();
+  RTE_TRY(launch_norm(p, *ws, ws->bt.p, ws->active.p, ws->bnorm.p, st));
   if (phi0) {
     RTE_CHECK_CUDA(cudaMemcpyAsync(x, phi0, p->ntot * 8, cudaMemcpyDeviceToDevice, st));
   } else {
@@ -2249,8 +2300,7 @@ extern "C" int si_solve(rte_problem_t p, const romsad_t* roms, const fgmres_opts
           ++S[b].sweeps_fp64;
         }
     }
-    k_norm<<<B, 512, 0, st>>>(ws->r.p, p->d_inst.p, ws->active.p, ws->nrm.p);
-    count_launch();
+    RTE_TRY(launch_norm(p, *ws, ws->r.p, ws->active.p, ws->nrm.p, st));
     k_linf<<<B, 512, 0, st>>>(ws->r.p, p->d_inst.p, ws->est.p);
     count_launch();
     std::vector<double> hl(B);

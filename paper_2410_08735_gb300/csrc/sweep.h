@@ -12,7 +12,7 @@ struct SweepArgs {
   const UDir* udir;
   const SweepTask* tasks;
   int ntasks;
-  const void* linv;     // compute type: cell inverses (sweep.cu) or wavefront tables (wavefront.cu)
+  const void* linv;     // compute type: cell inverses (sweep.cu), or the tables launch_wave puts here
   const void* sig_s;    // compute type, [B][R]; null: no Sigma_s scaling of the input
   const void* src;      // input type, scalar vector
   int with_bc;

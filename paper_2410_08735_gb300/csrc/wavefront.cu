@@ -273,6 +273,55 @@ struct Modal {
   }
 };
 
+// The Legendre basis itself: no transforms, sixteen table entries (the cell inverses), 32 D + 4 operations a cell against
+// 24 D + 30.  FP64 tasks of one or two directions, which do not pay for the eigenbasis's transforms (26 x (64 x 22), 28
+// directions in quadrants of 8 and 6, D = 1: 271 us in the eigenbasis, 190 us here).
+template <typename T>
+struct Legendre {
+  static constexpr int TW = 16;
+  static constexpr int NC = 5;   // alpha, beta, sqrt3 alpha, sqrt3 beta, omega
+  __device__ static T factor(int k, double fx, double fy) {
+    return (T)(((k & 1) ? fx : 1.0) * ((k & 2) ? fy : 1.0));
+  }
+  __device__ __forceinline__ static void to_basis(const T* t, T* S) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) S[e] = t[e];
+  }
+  __device__ __forceinline__ static void from_basis(const T* c, T* s) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] = c[e];
+  }
+  __device__ static void boundary(double g, T* t) {
+    t[0] = (T)g;
+    t[1] = (T)0;
+  }
+  __device__ static void constants(double al, double be, double w, T* c) {
+    const double s3 = 1.7320508075688772;
+    c[0] = (T)al;
+    c[1] = (T)be;
+    c[2] = (T)(s3 * al);
+    c[3] = (T)(s3 * be);
+    c[4] = (T)w;
+  }
+  template <typename V>
+  __device__ __forceinline__ static void cell(const V* S, V* X, V* Y, const V* m, const V* c, V* acc, bool zero) {
+    const T a = c[0].x, b = c[1].x, a3 = c[2].x, b3 = c[3].x, w = c[4].x, s3 = (T)1.7320508075688772;
+    const T x0 = X[0].x, x1 = X[1].x, y0 = Y[0].x, y1 = Y[1].x;
+    const T r[4] = {S[0].x + a * x0 + b * y0, S[1].x - a3 * x0 + b * y1, S[2].x + a * x1 - b3 * y0,
+                    S[3].x - a3 * x1 - b3 * y1};
+    T q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      q[i] = m[4 * i].x * r[0] + m[4 * i + 1].x * r[1] + m[4 * i + 2].x * r[2] + m[4 * i + 3].x * r[3];
+      acc[i].x = zero ? w * q[i] : acc[i].x + w * q[i];
+    }
+    X[0].x = q[0] + s3 * q[1];
+    X[1].x = q[2] + s3 * q[3];
+    Y[0].x = q[0] + s3 * q[2];
+    Y[1].x = q[1] + s3 * q[3];
+  }
+};
+
 // Unevaluated sums of two doubles, for the tables alone (two-sum and two-product as in dfloat.cuh)
 struct Dd {
   double h, l;
@@ -582,10 +631,14 @@ static void mesh_max(const rte_problem* p, int* nx, int* ny) {
   }
 }
 
+// FP64 tasks of one or two directions run in the Legendre basis
+static bool legendre(int prec, int D) { return prec == PREC_F64 && D <= 2; }
+
 size_t wave_smem(const rte_problem* p, int prec, WaveShape s) {
   int nx, ny;
   mesh_max(p, &nx, &ny);
-  const int tw = prec == PREC_F32 ? Rot<float>::TW : Modal<double>::TW, nc = prec == PREC_F32 ? Rot<float>::NC : Modal<double>::NC;
+  const int tw = prec == PREC_F32 ? Rot<float>::TW : (legendre(prec, s.D) ? Legendre<double>::TW : Modal<double>::TW);
+  const int nc = prec == PREC_F32 ? Rot<float>::NC : Modal<double>::NC;
   const int bytes = prec == PREC_F32 ? 4 : 8;
   const size_t elems = (size_t)(p->R + 1) * table_stride(4 + s.D * tw, bytes) + ((s.D * nc + 3) & ~3) +
                        ((size_t)nx + (s.W - 1) * kRing) * s.D * 2;
@@ -628,8 +681,8 @@ bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
 // step, one step taking the pipe cycles of all of them or the latency of one alone, whichever is longer.  Per warp and
 // step, measured: FP32 10 D + 40 cycles of the load/store data pipe (tables, shuffles; 13 D + 30 with two rows a lane),
 // the pipe that fills up first, of which single-warp tasks reach 0.65 and wider ones 0.75, 50 D + 300 alone (1750 with
-// two rows); FP64 19 cycles of the SM's FP64 unit for each of 24 D + 30 instructions (5 % more a
-// direction above 4), 70 alone; double-float 320 D + 264 instructions, 0.85 a cycle and SM quarter, 0.7 alone.  The partial fluxes, written and read once, are
+// two rows); FP64 19 cycles of the SM's FP64 unit for each of 24 D + 30 instructions (32 D + 4 in
+// the Legendre basis; 5 % more a direction above 4), 70 alone; double-float 320 D + 264 instructions, 0.85 a cycle and SM quarter, 0.7 alone.  The partial fluxes, written and read once, are
 // added at the copy bandwidth.
 static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, const std::vector<int>& order) {
   const int SK = 4, per_sm = 65536 / (shape_regs(prec, s.D, s.rpl) * 32);
@@ -642,8 +695,9 @@ static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, co
     pipe = (s.rpl == 2 ? 13.0 * s.D + 30.0 : 10.0 * s.D + 40.0) / (s.W == 1 ? 0.65 : 0.75);
     alone = s.rpl == 2 ? 1750.0 : 50.0 * s.D + 300.0;
   } else if (prec == PREC_F64) {
-    pipe = 19.0 * (1.0 + 0.05 * std::max(0, s.D - 4)) * (24.0 * s.D + 30.0);
-    alone = 70.0 * (24.0 * s.D + 30.0);
+    const double instr = legendre(prec, s.D) ? 32.0 * s.D + 4.0 : 24.0 * s.D + 30.0;
+    pipe = 19.0 * (1.0 + 0.05 * std::max(0, s.D - 4)) * instr;
+    alone = 70.0 * instr;
   } else {
     pipe = (320.0 * s.D + 264.0) / 3.4;   // of warps in multiples of four
     alone = (320.0 * s.D + 264.0) / 0.7;
@@ -762,8 +816,8 @@ template <bool BC>
 static int launch_f64(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t st) {
   using A = Modal<double>;
   switch (s.D) {
-    case 1: return launch_one<double, double, A, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 2: return launch_one<double, double, A, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st);
+    case 1: return launch_one<double, double, Legendre<double>, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st);
+    case 2: return launch_one<double, double, Legendre<double>, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st);
     case 3: return launch_one<double, double, A, 1, 3, 1, 4, BC, 2>(a, s.W, smem, st);
     case 4: return launch_one<double, double, A, 1, 4, 1, 4, BC, 1>(a, s.W, smem, st);
     case 8: return launch_one<double, double, A, 1, 8, 1, 4, BC, 1>(a, s.W, smem, st);
@@ -783,7 +837,11 @@ static int launch_df(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t 
   return RTE_ERR_UNSUPPORTED;
 }
 
-int launch_wave(const rte_problem* p, int prec, WaveShape s, bool in64, const SweepArgs& a, cudaStream_t st) {
+int launch_wave(const rte_problem* p, int prec, WaveShape s, bool in64, const SweepArgs& args, cudaStream_t st) {
+  SweepArgs a = args;
+  if (prec == PREC_F32) a.linv = p->d_rot32.p;
+  else if (prec == PREC_DF) a.linv = p->d_modal_df.p;
+  else a.linv = legendre(prec, s.D) ? p->d_linv64.p : p->d_modal64.p;
   if (!wave_shape_ok(p, prec, s)) {
     set_error("sweep: shared-memory table too large for this mesh/region count");
     return RTE_ERR_UNSUPPORTED;
