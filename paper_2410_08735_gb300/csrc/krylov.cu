@@ -773,15 +773,50 @@ __global__ void __launch_bounds__(256) k_arnoldi_coop(ArnArgs<TP, TV> A) {
   }
 }
 
+// four consecutive dofs of a vector, `left` of them in the piece; VEC: every instance's size and offset is a multiple of
+// four, so that a thread's four are loaded and stored at once
+template <bool VEC, typename T>
+__device__ __forceinline__ void tile_load(const T* p, int left, T* x) {
+  if constexpr (VEC) {
+    load4(p, x[0], x[1], x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < left) x[e] = p[e];
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void tile_store(float* p, int left, const float* x) {
+  if constexpr (VEC) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < left) p[e] = x[e];
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void tile_store(double* p, int left, const double* x) {
+  if constexpr (VEC) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < left) p[e] = x[e];
+  }
+}
+
 // Arnoldi step for large batches: the per-instance work (sums of the chunk partials, the T update and
 // h = T a; norm, Givens and flags) runs once per instance, in phases of its own between grid-wide
 // barriers (five phases, four barriers), and the preconditioner is a separate launch.  Compared with
 // k_arnoldi_coop this adds barriers but does not repeat any reduction, which is the better trade
 // once the chunks of the batch fill the GPU several times over.  Every block takes one run of consecutive chunks and adds
 // up the dot products of those that belong to one instance before it writes them, so the per-instance sums run over a
-// few dozen pieces instead of a thousand chunks (16 instances of 256^2: 260 -> 171 us an iteration, of which the Krylov
-// basis read twice and the partial fluxes are 90 us at the copy bandwidth).
-template <typename TP, typename TV>
+// few dozen pieces instead of a thousand chunks; a block takes 1024 dofs at a time, four a thread in one 16-byte access.
+// Bound by memory latency, then by HBM: 16 instances of 256^2, ten Krylov vectors on average, 260 us a launch with single
+// chunks and 4-byte accesses, 239 with pieces alone, 155 now; the bytes (the basis twice, the partial fluxes) take 90.
+template <typename TP, typename TV, bool VEC>
 __global__ void __launch_bounds__(256) k_arnoldi_wide(
     int B, const int2* items, const int* item0, int nitems, const InstInfo* inst, int* active, const TP* partial, int ntask,
     const TV* z, TV* V, long long ntot, int j, int m, int nchunk, TV* part, TV* npart, TV* Tm, int ldT,
@@ -792,78 +827,100 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nslot = 2 * m + 3;
   __shared__ TV red[260];
+  constexpr int TILE = 1024;   // dofs a block takes at a time, four consecutive ones a thread
   __shared__ TV as[130], ls[130], css[128], sns[128], hsv[130];
-  // P0: w = z - sum_t partial_t (the A~ z of this iteration) into V[j+1], then the chunk's partial dots
-  //     a_k = v_k . w (k <= j), g_k = v_k . v_j (k < j), w . w.  w and v_j are staged in shared memory
-  //     and warp q owns k = q, q + 8, ...: its reductions are independent of the other warps'.
-  __shared__ TV wsh[256], vjsh[256];
+  // P0: w = z - sum_t partial_t (the A~ z of this iteration) into V[j+1], then the partial dots a_k = v_k . w (k <= j),
+  //     g_k = v_k . v_j (k < j), w . w.  w and v_j are staged in shared memory and warp q owns k = q, q + 8, ...: its
+  //     reductions are independent of the other warps'.
+  __shared__ __align__(16) TV wsh[TILE], vjsh[TILE];
   const int per = (nitems + (int)gridDim.x - 1) / (int)gridDim.x;
   const int it0 = min(nitems, (int)blockIdx.x * per), it1 = min(nitems, it0 + per);
-  // pieces of an instance's chunk sums: one per block that holds chunks of it, stored at the piece's first chunk
-  auto pieces = [&](int b, int nch, auto&& at) {   // this lane's share: at(chunk where a piece is stored)
+  // the pieces of the block's run, one per instance it meets: f(instance, its first chunk, dof range)
+  auto for_pieces = [&](auto&& f) {
+    for (int it = it0; it < it1;) {
+      const int b = items[it].x, ch = items[it].y, nd = inst[b].ndof;
+      const int n = min(it1 - it, (nd + 255) / 256 - ch);
+      f(b, ch, ch * 256, min(nd, (ch + n) * 256));
+      it += n;
+    }
+  };
+  // where an instance's pieces are stored (at their first chunks): this lane's share of them
+  auto stored = [&](int b, int nch, auto&& at) {
     const int first = item0[b], k0 = first / per, k1 = (first + nch - 1) / per;
     for (int k = k0 + lane; k <= k1; k += 32) at(max(0, k * per - first));
   };
-  int start = it0;   // first chunk of the current piece
-  for (int it = it0; it < it1; ++it) {
-    const int b = items[it].x, ch = items[it].y;
-    const bool fresh = it == it0 || items[it - 1].x != b, done = it + 1 == it1 || items[it + 1].x != b;
-    if (fresh) start = ch;
-    if (!active[b]) continue;
-    if (fresh) {
-      for (int t = threadIdx.x; t < nslot; t += blockDim.x) red[t] = 0;
-    }
+  for_pieces([&](int b, int ch, int d0, int d1) {
+    if (!active[b]) return;
     const InstInfo in = inst[b];
-    const int i0 = ch * 256;
-    const int i = i0 + threadIdx.x;
-    const bool ok = i < in.ndof;
-    TV wi = 0;
-    if (ok) {
-      const TP* pp = partial + (size_t)ntask * in.off;
-      TP s = 0;
+    for (int t = threadIdx.x; t < nslot; t += blockDim.x) red[t] = 0;
+    for (int base = d0; base < d1; base += TILE) {
+      const int i = base + 4 * threadIdx.x, left = d1 - i;
+      TV wi[4] = {0, 0, 0, 0}, vj[4] = {0, 0, 0, 0};
+      if (left > 0) {
+        const TP* pp = partial + (size_t)ntask * in.off + i;
+        TP s[4] = {0, 0, 0, 0};
 #pragma unroll 8
-      for (int t = 0; t < ntask; ++t) s += pp[(size_t)t * in.ndof + i];
-      wi = z[in.off + i] - (TV)s;
-      V[(size_t)(j + 1) * ntot + in.off + i] = wi;
-    }
-    wsh[threadIdx.x] = wi;
-    vjsh[threadIdx.x] = ok ? V[(size_t)j * ntot + in.off + i] : TV(0);
-    __syncthreads();
-    const int nvalid = min(256, in.ndof - i0);
-#pragma unroll 4
-    for (int kk = warp; kk <= j; kk += 8) {
-      const TV* vk = V + (size_t)kk * ntot + in.off + i0;
-      TV a = 0, gg = 0;
+        for (int t = 0; t < ntask; ++t) {
+          TP x[4];
+          tile_load<VEC>(pp + (size_t)t * in.ndof, left, x);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int ii = lane + 32 * e;
-        const TV x = vk[min(ii, nvalid - 1)];   // surplus lanes meet zeros in wsh / vjsh
-        a += x * wsh[ii];
-        gg += x * vjsh[ii];
-      }
-      a = warp_sum_t(a);
-      gg = warp_sum_t(gg);
-      if (lane == 0) {
-        red[kk] += a;
-        if (kk < j) red[m + 1 + kk] += gg;
-      }
-    }
-    if (warp == 7) {
-      TV ww = 0;
+          for (int e = 0; e < 4; ++e) s[e] += x[e];
+        }
+        tile_load<VEC>(z + in.off + i, left, wi);
+        tile_load<VEC>(V + (size_t)j * ntot + in.off + i, left, vj);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) ww += wsh[lane + 32 * e] * wsh[lane + 32 * e];
-      ww = warp_sum_t(ww);
-      if (lane == 0) red[2 * m + 2] += ww;
-    }
-    __syncthreads();
-    if (done) {
-      for (int t = threadIdx.x; t < nslot; t += blockDim.x) {
-        const bool used = t <= j || (t >= m + 1 && t < m + 1 + j) || t == 2 * m + 2;
-        if (used) part[((size_t)b * nslot + t) * nchunk + start] = red[t];
+        for (int e = 0; e < 4; ++e) wi[e] = e < left ? wi[e] - (TV)s[e] : TV(0);
+        tile_store<VEC>(V + (size_t)(j + 1) * ntot + in.off + i, left, wi);
+      }
+      __syncthreads();   // the previous tile's dots are done
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        wsh[4 * threadIdx.x + e] = wi[e];
+        vjsh[4 * threadIdx.x + e] = vj[e];
       }
       __syncthreads();
+      for (int kk = warp; kk <= j; kk += 8) {
+        const TV* vk = V + (size_t)kk * ntot + in.off + base;
+        TV x[TILE / 128][4];
+#pragma unroll
+        for (int h = 0; h < TILE / 128; ++h) {   // all loads of the row first
+          const int o = 4 * lane + 128 * h;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[h][e] = TV(0);
+          if (base + o < d1) tile_load<VEC>(vk + o, d1 - base - o, x[h]);
+        }
+        TV a = 0, gg = 0;
+#pragma unroll
+        for (int h = 0; h < TILE / 128; ++h) {
+          const int o = 4 * lane + 128 * h;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            a += x[h][e] * wsh[o + e];
+            gg += x[h][e] * vjsh[o + e];
+          }
+        }
+        a = warp_sum_t(a);
+        gg = warp_sum_t(gg);
+        if (lane == 0) {
+          red[kk] += a;
+          if (kk < j) red[m + 1 + kk] += gg;
+        }
+      }
+      if (warp == 7) {
+        TV ww = 0;
+#pragma unroll 8
+        for (int e = 0; e < TILE / 32; ++e) ww += wsh[lane + 32 * e] * wsh[lane + 32 * e];
+        ww = warp_sum_t(ww);
+        if (lane == 0) red[2 * m + 2] += ww;
+      }
     }
-  }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nslot; t += blockDim.x) {
+      const bool used = t <= j || (t >= m + 1 && t < m + 1 + j) || t == 2 * m + 2;
+      if (used) part[((size_t)b * nslot + t) * nchunk + ch] = red[t];
+    }
+    __syncthreads();
+  });
   grid.sync();
   // P1: per instance: sum the chunk partials, grow T = (I + L)^{-1} by the new row, h = T a
   for (int b = blockIdx.x; b < B; b += gridDim.x) {
@@ -873,7 +930,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
       const int t = u <= j ? u : (u < 2 * j + 1 ? m + 1 + (u - j - 1) : 2 * m + 2);
       const TV* pp = part + ((size_t)b * nslot + t) * nchunk;
       TV acc = 0;
-      pieces(b, nch, [&](int c) { acc += pp[c]; });
+      stored(b, nch, [&](int c) { acc += pp[c]; });
       acc = warp_sum_t(acc);
       if (lane == 0) {
         if (t <= j) as[t] = acc;
@@ -904,41 +961,41 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
     __syncthreads();
   }
   grid.sync();
-  // P2: w -= sum_k h_k v_k over the chunk, partial ||w||^2
-  TV s2 = 0;   // this thread's share of the piece's ||w||^2
-  for (int it = it0; it < it1; ++it) {
-    const int b = items[it].x, ch = items[it].y;
-    const bool fresh = it == it0 || items[it - 1].x != b, done = it + 1 == it1 || items[it + 1].x != b;
-    if (fresh) start = ch;
-    if (!active[b]) continue;
+  // P2: w -= sum_k h_k v_k over the block's pieces, partial ||w||^2
+  for_pieces([&](int b, int ch, int d0, int d1) {
+    if (!active[b]) return;
     const InstInfo in = inst[b];
-    if (fresh) {
-      const double* h = H + ((size_t)b * m + j) * (m + 1);
-      __syncthreads();
-      for (int t = threadIdx.x; t <= j; t += blockDim.x) hsv[t] = (TV)h[t];
-      __syncthreads();
-      s2 = 0;
-    }
-    const int i = ch * 256 + threadIdx.x;
-    if (i < in.ndof) {
-      TV wi = V[(size_t)(j + 1) * ntot + in.off + i];
-#pragma unroll 16
-      for (int kk = 0; kk <= j; ++kk) wi -= hsv[kk] * V[(size_t)kk * ntot + in.off + i];
-      V[(size_t)(j + 1) * ntot + in.off + i] = wi;
-      s2 += wi * wi;
-    }
-    if (done) {
-      s2 = warp_sum_t(s2);
-      __syncthreads();
-      if (lane == 0) red[warp] = s2;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        TV tot = 0;
-        for (int w = 0; w < 8; ++w) tot += red[w];
-        npart[(size_t)b * nchunk + start] = tot;
+    const double* h = H + ((size_t)b * m + j) * (m + 1);
+    for (int t = threadIdx.x; t <= j; t += blockDim.x) hsv[t] = (TV)h[t];
+    __syncthreads();
+    TV s2 = 0;
+    for (int i = d0 + 4 * threadIdx.x; i < d1; i += TILE) {
+      const int left = d1 - i;
+      TV* vw = V + (size_t)(j + 1) * ntot + in.off + i;
+      TV wi[4] = {0, 0, 0, 0};
+      tile_load<VEC>(vw, left, wi);
+#pragma unroll 8
+      for (int kk = 0; kk <= j; ++kk) {
+        TV x[4] = {0, 0, 0, 0};
+        tile_load<VEC>(V + (size_t)kk * ntot + in.off + i, left, x);
+        const TV hk = hsv[kk];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) wi[e] -= hk * x[e];
       }
+      tile_store<VEC>(vw, left, wi);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s2 += e < left ? wi[e] * wi[e] : TV(0);
     }
-  }
+    s2 = warp_sum_t(s2);
+    if (lane == 0) red[warp] = s2;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      TV tot = 0;
+      for (int q = 0; q < 8; ++q) tot += red[q];
+      npart[(size_t)b * nchunk + ch] = tot;
+    }
+    __syncthreads();
+  });
   grid.sync();
   // P3: per instance: h_{j+1,j} = ||w||, breakdown test, Givens rotation, stopping flags
   for (int b = blockIdx.x; b < B; b += gridDim.x) {
@@ -958,7 +1015,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
     if (warp == 0) {
       const int nch = (inst[b].ndof + 255) / 256;
       TV acc = 0;
-      pieces(b, nch, [&](int c) { acc += npart[(size_t)b * nchunk + c]; });
+      stored(b, nch, [&](int c) { acc += npart[(size_t)b * nchunk + c]; });
       acc = warp_sum_t(acc);
       if (lane == 0) red[0] = acc;
     }
@@ -1006,13 +1063,19 @@ __global__ void __launch_bounds__(256) k_arnoldi_wide(
   }
   grid.sync();
   // P4: v_{j+1} = w / h_{j+1,j}
-  for (int it = it0; it < it1; ++it) {
-    const int b = items[it].x, ch = items[it].y;
-    if (!active0[b] || brk[b]) continue;
+  for_pieces([&](int b, int ch, int d0, int d1) {
+    if (!active0[b] || brk[b]) return;
     const InstInfo in = inst[b];
-    const int i = ch * 256 + threadIdx.x;
-    if (i < in.ndof) V[(size_t)(j + 1) * ntot + in.off + i] *= (TV)(1.0 / hnorm[b]);
-  }
+    const TV s = (TV)(1.0 / hnorm[b]);
+    for (int i = d0 + 4 * threadIdx.x; i < d1; i += TILE) {
+      TV* vw = V + (size_t)(j + 1) * ntot + in.off + i;
+      TV wi[4] = {0, 0, 0, 0};
+      tile_load<VEC>(vw, d1 - i, wi);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) wi[e] *= s;
+      tile_store<VEC>(vw, d1 - i, wi);
+    }
+  });
 }
 
 
@@ -1131,6 +1194,7 @@ struct Ws {
   // latency-bound problems (all chunks resident at once, few chunks per instance) take the fused
   // two-barrier Arnoldi step; larger batches the multi-phase one (k_arnoldi_wide)
   bool fused = true;
+  bool wide_vec = false;        // k_arnoldi_wide: sizes and offsets of all instances are multiples of four
   std::vector<romsad_t> plan_rom;
   std::vector<std::vector<int>> plan_ids;
   void drop_graphs() {
@@ -1209,11 +1273,16 @@ struct Ws {
       RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_arnoldi_coop<float, float>, 256, 0));
       grid_post32 = std::min(want, std::max(1, occ) * nsm);
       fused = nitems <= std::min(grid_post32, grid_post64) && nchunk <= 64;
-      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_arnoldi_wide<double, double>, 256, 0));
-      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_arnoldi_wide<float, double>, 256, 0));
+      wide_vec = true;
+      for (int b = 0; b <= p->B; ++b) wide_vec = wide_vec && p->off[b] % 4 == 0;
+      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &o1, wide_vec ? k_arnoldi_wide<double, double, true> : k_arnoldi_wide<double, double, false>, 256, 0));
+      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &o2, wide_vec ? k_arnoldi_wide<float, double, true> : k_arnoldi_wide<float, double, false>, 256, 0));
       occ = std::min(o1, o2);
       grid_wide64 = std::min(want, std::max(1, occ) * nsm);
-      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_arnoldi_wide<float, float>, 256, 0));
+      RTE_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &occ, wide_vec ? k_arnoldi_wide<float, float, true> : k_arnoldi_wide<float, float, false>, 256, 0));
       grid_wide32 = std::min(want, std::max(1, occ) * nsm);
     }
     RTE_TRY(part.alloc((size_t)B * nchunk * (2 * m + 3)));
@@ -1501,7 +1570,8 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
           void* args[] = {&Bv, &it_p, &i0_p, &nit, &inst_p, &act_p, &part_p, &ntask, &z_p, &V_p, &nt, &jj, &mm, &nch,
                           &dp_p, &np_p, &Lt_p, &ldT, &H_p, &Hr_p, &w0_p, &cs_p, &sn_p, &g_p, &brk_p, &bn_p, &rt_p,
                           &il_p, &est_p, &fl_p, &kc_p, &hn_p, &a0_p};
-          RTE_CHECK_CUDA(cudaLaunchCooperativeKernel((const void*)k_arnoldi_wide<TP, TV>,
+          const void* wide = W.wide_vec ? (const void*)k_arnoldi_wide<TP, TV, true> : (const void*)k_arnoldi_wide<TP, TV, false>;
+          RTE_CHECK_CUDA(cudaLaunchCooperativeKernel(wide,
                                                      dim3(f64 ? W.grid_wide64 : W.grid_wide32), dim3(256), args, 0,
                                                      s));
           count_launch();
