@@ -34,7 +34,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "internal.h"
+#include "sweep.h"
 
 namespace rte {
 
@@ -46,13 +46,15 @@ constexpr int kThreads = 512;         // per block of the V-cycle cluster
 constexpr int kCluster = 8;           // blocks per instance in the V-cycle
 constexpr int kClusterVerts = 2048;   // vertex levels at least this large are split over the cluster
 constexpr int kSetupThreads = 256;
+constexpr int kWideCells = 1024;      // set-up: levels with at least as many cells get a launch of their own
 constexpr float kSqrt3 = 1.7320508075688772f;
 
 struct DsaInst {
   int nx, ny;                  // DG mesh (cells)
   int L;                       // vertex levels 1..L (L = coarsest)
   float hx, hy;
-  long long o_sgs, o_sga, o_binv, o_kinv, o_b0, o_x0, o_t, o_r0;
+  int per_cell;                // coefficients of level 0 and 1: 1 = one set per cell, 0 = one per class (below)
+  long long o_sgs, o_sga, o_binv, o_kinv, o_r0;
   int ncx[kMaxLevels + 1], ncy[kMaxLevels + 1];
   long long o_E[kMaxLevels + 1], o_dinv[kMaxLevels + 1], o_u[kMaxLevels + 1], o_b[kMaxLevels + 1],
       o_r[kMaxLevels + 1];
@@ -204,10 +206,16 @@ __device__ __forceinline__ float ldv(const float* p) {
   else return *p;
 }
 
-// y = A_l u at vertex (ix, iy) of a level with ncx x ncy cells and element matrices E [cells][4][4]
-template <bool CG>
-__device__ float vertex_apply(const float* E, const float* u, int ncx, int ncy, int ix, int iy) {
+// y = A_l u at vertex (ix, iy) of a level with ncx x ncy cells and element matrices E + at(cx, cy)
+template <bool CG, typename F>
+__device__ __forceinline__ float vertex_apply(const float* E, F&& at, const float* u, int ncx, int ncy, int ix, int iy) {
   const int nvx = ncx + 1;
+  float U[3][3];   // the vertex and its neighbours, each loaded once (clamped at the edges: no cell reads those)
+#pragma unroll
+  for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+      U[dy][dx] = ldv<CG>(u + min(max(iy + dy - 1, 0), ncy) * nvx + min(max(ix + dx - 1, 0), ncx));
   float y = 0.f;
 #pragma unroll
   for (int sy = 0; sy < 2; ++sy) {
@@ -217,16 +225,26 @@ __device__ float vertex_apply(const float* E, const float* u, int ncx, int ncy, 
     for (int sx = 0; sx < 2; ++sx) {
       const int cx = ix - 1 + sx;
       if (cx < 0 || cx >= ncx) continue;
-      const int qv = (ix - cx) + 2 * (iy - cy);
+      const int qv = (1 - sx) + 2 * (1 - sy);
       float e[4];
-      load4(E + ((size_t)(cy * ncx + cx) * 16 + qv * 4), e);
-      const int v0 = cy * nvx + cx;
-      y += e[0] * ldv<CG>(u + v0) + e[1] * ldv<CG>(u + v0 + 1) + e[2] * ldv<CG>(u + v0 + nvx) +
-           e[3] * ldv<CG>(u + v0 + nvx + 1);
+      load4(E + at(cx, cy) + qv * 4, e);
+      y += e[0] * U[sy][sx] + e[1] * U[sy][sx + 1] + e[2] * U[sy + 1][sx] + e[3] * U[sy + 1][sx + 1];
     }
   }
   return y;
 }
+
+// i -> (i % n, i / n) for i < count: a multiplication where count n < 2^32 makes it exact, a division otherwise
+struct Split {
+  int n;
+  unsigned m;
+  __device__ Split(int n_, int count)
+      : n(n_), m(n_ > 1 && (unsigned long long)count * n_ < (1ull << 32) ? 0xffffffffu / (unsigned)n_ + 1u : 0u) {}
+  __device__ __forceinline__ void operator()(int i, int& x, int& y) const {
+    y = m ? (int)__umulhi((unsigned)i, m) : i / n;
+    x = i - y * n;
+  }
+};
 
 // B_d^{-1} of one cell (4 dofs) from its sigma_t
 __device__ __forceinline__ void binv_of(float st, int d, const DsaConst& k, const float* hs, float* out) {
@@ -240,18 +258,42 @@ __device__ __forceinline__ void binv_of(float st, int d, const DsaConst& k, cons
   }
 }
 
+// Classes of cells.  With cross sections constant on rx x ry equal blocks of cells, a cell's coefficients (sigma, B_d^{-1},
+// K_cc^{-1}, level-1 element matrix) follow from its region and from which of its four neighbours lie in another region or
+// outside: 16 classes per region, class = code_x(ix) + code_y(iy) with the edge bits of both axes.  Meshes with so many
+// regions that this saves little, and cross-section profiles, keep one set per cell: code_x = ix, code_y = iy nx.
+__device__ __forceinline__ int edge_bits(int i, int c) { return (i == 0 ? 1 : 0) + (i == c - 1 ? 2 : 0); }
+__device__ __forceinline__ int code_x(const DsaInst& di, int ix, int rx) {
+  const int c = di.nx / rx;
+  return di.per_cell ? ix : (ix / c) * 16 + edge_bits(ix % c, c) * 4;
+}
+__device__ __forceinline__ int code_y(const DsaInst& di, int iy, int rx, int ry) {
+  const int c = di.ny / ry;
+  return di.per_cell ? iy * di.nx : (iy / c) * rx * 16 + edge_bits(iy % c, c);
+}
+// a cell of class k, or -1: bits 1 and 2 both set only where the block is one cell wide, and none only from three on
+__device__ __forceinline__ int class_cell(const DsaInst& di, int k, int rx, int ry) {
+  if (di.per_cell) return k;
+  const int cx = di.nx / rx, cy = di.ny / ry, reg = k >> 4, ex = (k >> 2) & 3, ey = k & 3;
+  const int ix = ex == 0 ? 1 : (ex == 2 ? cx - 1 : 0), iy = ey == 0 ? 1 : (ey == 2 ? cy - 1 : 0);
+  if (ix >= cx || iy >= cy || edge_bits(ix, cx) != ex || edge_bits(iy, cy) != ey) return -1;
+  return ((reg / rx) * cy + iy) * di.nx + (reg % rx) * cx + ix;
+}
+
 // ----------------------------------------------------------------------------------------------- set-up
-// Per cell, every instance at once (grid [cells / kSetupThreads, B]): cross sections, B_d^{-1}, the
+// Per class of cells, every instance at once (grid [classes / kSetupThreads, B]): cross sections, B_d^{-1}, the
 // inverted 4x4 diagonal block of K and the level-1 element matrix.  Neighbours' B^{-1} are recomputed
-// from their sigma_t, so cells are independent.
+// from their sigma_t, so classes are independent.
 __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_cells(const DsaInst* dinfo, float* base,
                                                                    const double* sig_s, const double* sig_t, int R,
                                                                    int rx, int ry, DsaConst k) {
   const int b = blockIdx.y;
   const DsaInst& di = dinfo[b];
-  const int nx = di.nx, ny = di.ny, nc = nx * ny;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nc) return;
+  const int nx = di.nx, ny = di.ny;
+  const int cls = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cls >= (di.per_cell ? nx * ny : 16 * rx * ry)) return;
+  const int c = class_cell(di, cls, rx, ry);
+  if (c < 0) return;
   const int cxr = nx / rx, cyr = ny / ry;
   const float hs[2] = {di.hx, di.hy};
   auto st_of = [&](int cell) {
@@ -263,13 +305,13 @@ __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_cells(const DsaInst
   const float ss = (float)sig_s[(size_t)b * R + reg];
   const float st = (float)sig_t[(size_t)b * R + reg];
   const float sa = st - ss;
-  base[di.o_sgs + c] = ss;
-  base[di.o_sga + c] = sa;
+  base[di.o_sgs + cls] = ss;
+  base[di.o_sga + cls] = sa;
   float bc[2][4];
   binv_of(st, 0, k, hs, bc[0]);
   binv_of(st, 1, k, hs, bc[1]);
   for (int d = 0; d < 2; ++d)
-    for (int q = 0; q < 4; ++q) base[di.o_binv + (size_t)c * 8 + d * 4 + q] = bc[d][q];
+    for (int q = 0; q < 4; ++q) base[di.o_binv + (size_t)cls * 8 + d * 4 + q] = bc[d][q];
   const Axis ax[2] = {Axis(di.hx), Axis(di.hy)};
   const float zero4[4] = {0.f, 0.f, 0.f, 0.f};
   // diagonal block of K, column by column: K e_col restricted to this cell
@@ -316,7 +358,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_cells(const DsaInst
       for (int q = 0; q < 4; ++q) Kc[r * 4 + q] -= f * Kc[p * 4 + q];
     }
   }
-  for (int q = 0; q < 16; ++q) base[di.o_kinv + (size_t)c * 16 + q] = Kc[q];
+  for (int q = 0; q < 16; ++q) base[di.o_kinv + (size_t)cls * 16 + q] = Kc[q];
   // element matrix: P^T (sigma_a + sum_e kappa_e J_e) P + sum_d 3 mu2_d^2 (G_d P)^T B_d^{-1} (G_d P)
   float Pq[4][4], M[4][4], G[2][4][4];
   for (int q = 0; q < 4; ++q) {
@@ -339,69 +381,82 @@ __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_cells(const DsaInst
         const float f = 3.f * k.mu2[d] * k.mu2[d];
         for (int kk = 0; kk < 4; ++kk) s += f * G[d][q][kk] * bc[d][kk] * G[d][q2][kk];
       }
-      E1[(size_t)c * 16 + q * 4 + q2] = s;
+      E1[(size_t)cls * 16 + q * 4 + q2] = s;
     }
 }
 
-// Per instance (one block): coarse element matrices, inverse diagonals and the dense inverse of the
-// coarsest level.
-__global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_levels(const DsaInst* dinfo, float* base) {
+// offset of the element matrix of cell (cx, cy) of level l
+__device__ __forceinline__ size_t elem(const DsaInst& di, int l, int cx, int cy, int rx, int ry) {
+  return 16 * (size_t)(l == 1 ? code_x(di, cx, rx) + code_y(di, cy, rx, ry) : cy * di.ncx[l] + cx);
+}
+
+// element matrices of level l >= 2 (sum over the 4 children of I^T E_child I) and inverse diagonals of level l - 1, by
+// the threads t0, t0 + tn, ... of an instance
+__device__ void setup_level(const DsaInst& di, float* base, int l, int t0, int tn, int rx, int ry) {
+  const int ncx = di.ncx[l], ncy = di.ncy[l];
+  const float* Ef = base + di.o_E[l - 1];
+  float* Ec = base + di.o_E[l];
+  for (int cc = t0; cc < ncx * ncy; cc += tn) {
+    const int CX = cc % ncx, CY = cc / ncx;
+    float acc[16];
+    for (int q = 0; q < 16; ++q) acc[q] = 0.f;
+    for (int s = 0; s < 4; ++s) {
+      const int sx = s & 1, sy = s >> 1;
+      const float* e = Ef + elem(di, l - 1, 2 * CX + sx, 2 * CY + sy, rx, ry);
+      // I[child corner][coarse corner] = w(Vx, (sx+vx)/2) w(Vy, (sy+vy)/2), w(0,t) = 1-t, w(1,t) = t
+      float I[4][4];
+      for (int qc = 0; qc < 4; ++qc) {
+        const float tx = 0.5f * (sx + (qc & 1)), ty = 0.5f * (sy + (qc >> 1));
+        for (int Q = 0; Q < 4; ++Q) I[qc][Q] = ((Q & 1) ? tx : 1.f - tx) * ((Q >> 1) ? ty : 1.f - ty);
+      }
+      float EI[4][4];
+      for (int r = 0; r < 4; ++r)
+        for (int Q = 0; Q < 4; ++Q) {
+          float s2 = 0.f;
+          for (int q = 0; q < 4; ++q) s2 += e[r * 4 + q] * I[q][Q];
+          EI[r][Q] = s2;
+        }
+      for (int P = 0; P < 4; ++P)
+        for (int Q = 0; Q < 4; ++Q) {
+          float s2 = 0.f;
+          for (int r = 0; r < 4; ++r) s2 += I[r][P] * EI[r][Q];
+          acc[P * 4 + Q] += s2;
+        }
+    }
+    for (int q = 0; q < 16; ++q) Ec[(size_t)cc * 16 + q] = acc[q];
+  }
+  const int fx = di.ncx[l - 1], fy = di.ncy[l - 1], nvx = fx + 1, nv = nvx * (fy + 1);
+  float* dinv = base + di.o_dinv[l - 1];
+  for (int v = t0; v < nv; v += tn) {
+    const int ix = v % nvx, iy = v / nvx;
+    float s = 0.f;
+    for (int sy = 0; sy < 2; ++sy)
+      for (int sx = 0; sx < 2; ++sx) {
+        const int cx = ix - 1 + sx, cy = iy - 1 + sy;
+        if (cx < 0 || cx >= fx || cy < 0 || cy >= fy) continue;
+        s += Ef[elem(di, l - 1, cx, cy, rx, ry) + ((ix - cx) + 2 * (iy - cy)) * 5];
+      }
+    dinv[v] = 1.f / s;
+  }
+}
+
+// One level of every instance, grid [blocks, B]: the levels with many cells, which one block per instance took 1010 us
+// for at 16 x 256^2.
+__global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_level(const DsaInst* dinfo, float* base, int l, int rx,
+                                                                   int ry) {
+  const DsaInst& di = dinfo[blockIdx.y];
+  if (l <= di.L) setup_level(di, base, l, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, rx, ry);
+}
+
+// Per instance (one block): the levels from l0 on and the dense inverse of the coarsest.
+__global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_levels(const DsaInst* dinfo, float* base, int l0, int rx,
+                                                                    int ry) {
   __shared__ float A[kMaxCoarse * kMaxCoarse];
   const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
   const DsaInst& di = dinfo[b];
-  // coarse element matrices: sum over the 4 children of I^T E_child I
-  for (int l = 2; l <= di.L; ++l) {
-    const int ncx = di.ncx[l], ncy = di.ncy[l], fcx = di.ncx[l - 1];
-    const float* Ef = base + di.o_E[l - 1];
-    float* Ec = base + di.o_E[l];
-    for (int cc = tid; cc < ncx * ncy; cc += nth) {
-      const int CX = cc % ncx, CY = cc / ncx;
-      float acc[16];
-      for (int q = 0; q < 16; ++q) acc[q] = 0.f;
-      for (int s = 0; s < 4; ++s) {
-        const int sx = s & 1, sy = s >> 1;
-        const float* e = Ef + (size_t)((2 * CY + sy) * fcx + 2 * CX + sx) * 16;
-        // I[child corner][coarse corner] = w(Vx, (sx+vx)/2) w(Vy, (sy+vy)/2), w(0,t) = 1-t, w(1,t) = t
-        float I[4][4];
-        for (int qc = 0; qc < 4; ++qc) {
-          const float tx = 0.5f * (sx + (qc & 1)), ty = 0.5f * (sy + (qc >> 1));
-          for (int Q = 0; Q < 4; ++Q) I[qc][Q] = ((Q & 1) ? tx : 1.f - tx) * ((Q >> 1) ? ty : 1.f - ty);
-        }
-        float EI[4][4];
-        for (int r = 0; r < 4; ++r)
-          for (int Q = 0; Q < 4; ++Q) {
-            float s2 = 0.f;
-            for (int q = 0; q < 4; ++q) s2 += e[r * 4 + q] * I[q][Q];
-            EI[r][Q] = s2;
-          }
-        for (int P = 0; P < 4; ++P)
-          for (int Q = 0; Q < 4; ++Q) {
-            float s2 = 0.f;
-            for (int r = 0; r < 4; ++r) s2 += I[r][P] * EI[r][Q];
-            acc[P * 4 + Q] += s2;
-          }
-      }
-      for (int q = 0; q < 16; ++q) Ec[(size_t)cc * 16 + q] = acc[q];
-    }
+  for (int l = l0; l <= di.L; ++l) {
+    setup_level(di, base, l, tid, nth, rx, ry);
     __syncthreads();
-  }
-  // inverse diagonals of the vertex levels above the coarsest
-  for (int l = 1; l < di.L; ++l) {
-    const int ncx = di.ncx[l], ncy = di.ncy[l], nvx = ncx + 1, nv = nvx * (ncy + 1);
-    const float* E = base + di.o_E[l];
-    float* dinv = base + di.o_dinv[l];
-    for (int v = tid; v < nv; v += nth) {
-      const int ix = v % nvx, iy = v / nvx;
-      float s = 0.f;
-      for (int sy = 0; sy < 2; ++sy)
-        for (int sx = 0; sx < 2; ++sx) {
-          const int cx = ix - 1 + sx, cy = iy - 1 + sy;
-          if (cx < 0 || cx >= ncx || cy < 0 || cy >= ncy) continue;
-          const int qv = (ix - cx) + 2 * (iy - cy);
-          s += E[(size_t)(cy * ncx + cx) * 16 + qv * 5];
-        }
-      dinv[v] = 1.f / s;
-    }
   }
   // dense inverse of the coarsest level (Gauss-Jordan in shared memory, one row per thread)
   const int l = di.L, ncx = di.ncx[l], ncy = di.ncy[l], nvx = ncx + 1, n = nvx * (ncy + 1);
@@ -415,7 +470,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_levels(const DsaIns
         for (int cx = max(ix, jx) - 1; cx <= min(ix, jx); ++cx) {
           if (cx < 0 || cx >= ncx || cy < 0 || cy >= ncy) continue;
           const int qi = (ix - cx) + 2 * (iy - cy), qj = (jx - cx) + 2 * (jy - cy);
-          s += E[(size_t)(cy * ncx + cx) * 16 + qi * 4 + qj];
+          s += E[elem(di, l, cx, cy, rx, ry) + qi * 4 + qj];
         }
     A[idx] = s;
   }
@@ -441,10 +496,27 @@ __global__ void __launch_bounds__(kSetupThreads) k_dsa_setup_levels(const DsaIns
 // are done by block 0 alone.
 namespace cg = cooperative_groups;
 
+// The DG stages run over tiles of 32 x 16 cells, one cell a thread.  x = omega Kcc^{-1} Sigma_s v (+ P_c w after the coarse
+// correction) of the tile and of two cells around it along each axis, and from it the fluxes B^{-1} D_C x of the tile and
+// one cell around it, stay in shared memory; nothing but r is stored between the passes over the mesh, and the coefficients
+// come from the classes' tables, which the L1 holds.  An apply used to move 800 bytes a cell (x, its source and the fluxes
+// written and read back, a 4x4 inverse and an element matrix per cell); now 115 from DRAM.  64 instances of 256^2: 783 ->
+// 602 us, no longer bound by HBM but by dependent loads and barriers (37 % of the issue slots; registers for two blocks
+// an SM).  Recomputing x at the nine cells of the stencil instead of the tile took 1119 us.
+constexpr int kTileX = 32, kTileY = kThreads / kTileX;
+__device__ __forceinline__ void load_v4(const float* p, float* x) { load4(p, x); }
+__device__ __forceinline__ void load_v4(const double* p, float* x) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+  x[0] = (float)a.x;
+  x[1] = (float)a.y;
+  x[2] = (float)b.x;
+  x[3] = (float)b.y;
+}
+
 template <typename TV>
-__global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, const DsaInst* dinfo, float* base,
-                                                         DsaConst k, const TV* v, TV* z, const int* active,
-                                                         const int* only) {
+__global__ void __launch_bounds__(kThreads, 2) k_dsa_vcycle(const InstInfo* inst, const DsaInst* dinfo, float* base,
+                                                         DsaConst k, int rx, int ry, const TV* v, TV* z,
+                                                         const int* active, const int* only) {
   cg::cluster_group cl = cg::this_cluster();
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int b = blockIdx.x / CS, tid = threadIdx.x, nth = blockDim.x;
@@ -452,6 +524,7 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
   if (only && !only[b]) return;
   const int gt = rank * nth + tid, gn = CS * nth;
   __shared__ float Pc[16];
+  extern __shared__ int codes[];      // class codes of the columns [nx] and rows [ny]
   const DsaInst& di = dinfo[b];
   const InstInfo in = inst[b];
   const int nx = di.nx, ny = di.ny, nc = nx * ny;
@@ -459,14 +532,15 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
   const float* sga = base + di.o_sga;
   const float* binv = base + di.o_binv;
   const float* kinv = base + di.o_kinv;
-  float* b0 = base + di.o_b0;
-  float* x0 = base + di.o_x0;
-  float* t = base + di.o_t;
   float* r0 = base + di.o_r0;
   const TV* vb = v + in.off;
   TV* zb = z + in.off;
   const Axis ax[2] = {Axis(di.hx), Axis(di.hy)};
   const float om = k.omega, omv = k.omega_v;
+  int* xc = codes;
+  int* yc = codes + nx;
+  for (int i = tid; i < nx; i += nth) xc[i] = code_x(di, i, rx);
+  for (int i = tid; i < ny; i += nth) yc[i] = code_y(di, i, rx, ry);
   if (tid < 16) Pc[tid] = pc_entry(tid >> 2, tid & 3, di.hx, di.hy);   // [k][q]
   __syncthreads();
   // first vertex level handled by block 0 alone
@@ -476,49 +550,102 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
       lsplit = l;
       break;
     }
-
-  // K x0 on cell c from x0 and t (= B^{-1} D_C x0 per axis)
-  auto Kx = [&](int c, float* out) {
-    const int ix = c % nx, iy = c / nx;
-    float xc[4];
-    load4cg(x0 + (size_t)c * 4, xc);
-    for (int q = 0; q < 4; ++q) out[q] = sga[c] * xc[q];
+  __shared__ float4 X[kTileY + 4][kTileX + 4], Tx[kTileY][kTileX + 2], Ty[kTileY + 2][kTileX];
+  // omega Kcc^{-1} Sigma_s v on a cell of class cls; bc: Sigma_s v
+  auto smooth = [&](int c, int cls, float* bc, float* x) {
+    load_v4(vb + (size_t)c * 4, bc);
+    const float sg = sgs[cls];
 #pragma unroll
-    for (int d = 0; d < 2; ++d) {
-      const Nb n = nb_of(ix, iy, nx, ny, d);
-      float xl[4], xh[4], tc[4], tl[4], th[4], tmp[4];
-      load4cg(x0 + (size_t)n.cl * 4, xl);
-      load4cg(x0 + (size_t)n.ch * 4, xh);
-      dj_cell(xc, xl, xh, n.l, n.h, d, ax[d], tmp);
+    for (int q = 0; q < 4; ++q) bc[q] *= sg;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) out[q] -= k.kappa[d] * tmp[q];
-      const float* td = t + (size_t)d * nc * 4;
-      load4cg(td + (size_t)c * 4, tc);
-      load4cg(td + (size_t)n.cl * 4, tl);
-      load4cg(td + (size_t)n.ch * 4, th);
-      dc_cell(tc, tl, th, n.l, n.h, d, ax[d], tmp);
-      const float f = 3.f * k.mu2[d] * k.mu2[d];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) out[q] -= f * tmp[q];
+    for (int r = 0; r < 4; ++r) {
+      float kr[4];
+      load4(kinv + (size_t)cls * 16 + r * 4, kr);
+      x[r] = om * (kr[0] * bc[0] + kr[1] * bc[1] + kr[2] * bc[2] + kr[3] * bc[3]);
     }
   };
-  auto stage_t = [&]() {
-    for (int c = gt; c < nc; c += gn) {
-      const int ix = c % nx, iy = c / nx;
-      float xc[4];
-      load4cg(x0 + (size_t)c * 4, xc);
-#pragma unroll
-      for (int d = 0; d < 2; ++d) {
-        const Nb n = nb_of(ix, iy, nx, ny, d);
-        float xl[4], xh[4], out[4], bi[4];
-        load4cg(x0 + (size_t)n.cl * 4, xl);
-        load4cg(x0 + (size_t)n.ch * 4, xh);
-        dc_cell(xc, xl, xh, n.l, n.h, d, ax[d], out);
-        load4(binv + (size_t)c * 8 + d * 4, bi);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) out[q] *= bi[q];
-        store4(t + ((size_t)d * nc + c) * 4, out);
+  auto put = [](float4& p, const float* x) { p = make_float4(x[0], x[1], x[2], x[3]); };
+  auto get = [](const float4& p, float* x) {
+    x[0] = p.x;
+    x[1] = p.y;
+    x[2] = p.z;
+    x[3] = p.w;
+  };
+  // for every cell of the block's tiles finish(ix, iy, Sigma_s v, x, K x); add(ix, iy, x) completes the smoothed x
+  auto for_tiles = [&](auto&& add, auto&& finish) {
+    const int tnx = (nx + kTileX - 1) / kTileX, tny = (ny + kTileY - 1) / kTileY;
+    const int lx = tid % kTileX, ly = tid / kTileX;
+    for (int tile = rank; tile < tnx * tny; tile += CS) {
+      const int ox = (tile % tnx) * kTileX, oy = (tile / tnx) * kTileY, ix = ox + lx, iy = oy + ly;
+      const bool in_mesh = ix < nx && iy < ny;
+      float bc[4] = {0.f, 0.f, 0.f, 0.f}, x0[4] = {0.f, 0.f, 0.f, 0.f};
+      if (in_mesh) {
+        smooth(iy * nx + ix, xc[ix] + yc[iy], bc, x0);
+        add(ix, iy, x0);
       }
+      put(X[ly + 2][lx + 2], x0);
+      if (tid < 4 * (kTileX + kTileY)) {   // two columns or rows on each side
+        const int g = tid - 4 * kTileY, k = g < 0 ? tid & 3 : g / kTileX;
+        const int hx = g < 0 ? (k < 2 ? k - 2 : kTileX + k - 2) : g % kTileX;
+        const int hy = g < 0 ? tid >> 2 : (k < 2 ? k - 2 : kTileY + k - 2);
+        const int jx = ox + hx, jy = oy + hy;
+        float hb[4], h0[4] = {0.f, 0.f, 0.f, 0.f};
+        if (jx >= 0 && jx < nx && jy >= 0 && jy < ny) {
+          smooth(jy * nx + jx, xc[jx] + yc[jy], hb, h0);
+          add(jx, jy, h0);
+        }
+        put(X[hy + 2][hx + 2], h0);
+      }
+      __syncthreads();
+      // t_d = B_d^{-1} D_C,d x at cell (hx, hy) of the tile
+      auto flux = [&](int hx, int hy, int d, float4& dst) {
+        const int jx = ox + hx, jy = oy + hy;
+        float t[4] = {0.f, 0.f, 0.f, 0.f};
+        if (jx >= 0 && jx < nx && jy >= 0 && jy < ny) {
+          float xm[4], xl[4], xh[4], bi[4];
+          get(X[hy + 2][hx + 2], xm);
+          get(d == 0 ? X[hy + 2][hx + 1] : X[hy + 1][hx + 2], xl);
+          get(d == 0 ? X[hy + 2][hx + 3] : X[hy + 3][hx + 2], xh);
+          dc_cell(xm, xl, xh, d == 0 ? jx > 0 : jy > 0, d == 0 ? jx < nx - 1 : jy < ny - 1, d, ax[d], t);
+          load4(binv + (size_t)(xc[jx] + yc[jy]) * 8 + d * 4, bi);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) t[q] *= bi[q];
+        }
+        put(dst, t);
+      };
+      flux(lx, ly, 0, Tx[ly][lx + 1]);
+      flux(lx, ly, 1, Ty[ly + 1][lx]);
+      if (tid < 2 * kTileY) flux((tid & 1) ? kTileX : -1, tid >> 1, 0, Tx[tid >> 1][(tid & 1) ? kTileX + 1 : 0]);
+      else if (tid < 2 * (kTileX + kTileY)) {
+        const int g = tid - 2 * kTileY, top = g / kTileX;
+        flux(g % kTileX, top ? kTileY : -1, 1, Ty[top ? kTileY + 1 : 0][g % kTileX]);
+      }
+      __syncthreads();
+      if (in_mesh) {
+        float out[4];
+        const float sa = sga[xc[ix] + yc[iy]];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) out[q] = sa * x0[q];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          const bool l = d == 0 ? ix > 0 : iy > 0, h = d == 0 ? ix < nx - 1 : iy < ny - 1;
+          float xl[4], xh[4], tc[4], tl[4], th[4], tmp[4];
+          get(d == 0 ? X[ly + 2][lx + 1] : X[ly + 1][lx + 2], xl);
+          get(d == 0 ? X[ly + 2][lx + 3] : X[ly + 3][lx + 2], xh);
+          dj_cell(x0, xl, xh, l, h, d, ax[d], tmp);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) out[q] -= k.kappa[d] * tmp[q];
+          get(d == 0 ? Tx[ly][lx + 1] : Ty[ly + 1][lx], tc);
+          get(d == 0 ? Tx[ly][lx] : Ty[ly][lx], tl);
+          get(d == 0 ? Tx[ly][lx + 2] : Ty[ly + 2][lx], th);
+          dc_cell(tc, tl, th, l, h, d, ax[d], tmp);
+          const float f = 3.f * k.mu2[d] * k.mu2[d];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) out[q] -= f * tmp[q];
+        }
+        finish(ix, iy, bc, x0, out);
+      }
+      __syncthreads();
     }
   };
   // Vertex levels.  On entry to level l, b_l and the pre-smoothed u_l = omega D^{-1} b_l are stored
@@ -535,10 +662,14 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
     float* u = base + di.o_u[l];
     const float* bl = base + di.o_b[l];
     float* rl = base + di.o_r[l];
-    if (CG || ecg)
-      for (int vv = t0; vv < nv; vv += tn) rl[vv] = __ldcg(bl + vv) - vertex_apply<true>(E, u, ncx, ncy, vv % nvx, vv / nvx);
-    else
-      for (int vv = t0; vv < nv; vv += tn) rl[vv] = bl[vv] - vertex_apply<false>(E, u, ncx, ncy, vv % nvx, vv / nvx);
+    auto el = [&](int cx, int cy) { return (size_t)(l == 1 ? xc[cx] + yc[cy] : cy * ncx + cx) * 16; };
+    const Split fine(nvx, nv);
+    for (int vv = t0; vv < nv; vv += tn) {
+      int ix, iy;
+      fine(vv, ix, iy);
+      if (CG || ecg) rl[vv] = __ldcg(bl + vv) - vertex_apply<true>(E, el, u, ncx, ncy, ix, iy);
+      else rl[vv] = bl[vv] - vertex_apply<false>(E, el, u, ncx, ncy, ix, iy);
+    }
     sync();
     // full-weighting restriction (transpose of bilinear interpolation) and pre-smoothing of level l+1
     const int Cx = di.ncx[l + 1], Cy = di.ncy[l + 1], nCx = Cx + 1, nC = nCx * (Cy + 1);
@@ -546,8 +677,10 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
     float* uc = base + di.o_u[l + 1];
     const float* dinvc = base + di.o_dinv[l + 1];
     const bool smooth_next = l + 1 < di.L;
+    const Split coarse(nCx, nC);
     for (int V = t0; V < nC; V += tn) {
-      const int I = V % nCx, J = V / nCx;
+      int I, J;
+      coarse(V, I, J);
       float s = 0.f;
       for (int dj = -1; dj <= 1; ++dj) {
         const int fy = 2 * J + dj;
@@ -576,16 +709,25 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
     const float* bl = base + di.o_b[l];
     float* rl = base + di.o_r[l];
     auto ucf = [&](int V) { return ldv<CG>(uc + V) + (ws != 0.f ? ws * dinvc[V] * ldv<CG>(rc + V) : 0.f); };
+    const Split fine(nvx, nv);
     for (int vv = t0; vv < nv; vv += tn) {
       // bilinear interpolation: the coarse neighbours of an even index coincide
-      const int ix = vv % nvx, iy = vv / nvx;
+      int ix, iy;
+      fine(vv, ix, iy);
       const int x0i = ix >> 1, y0i = iy >> 1, x1i = (ix + 1) >> 1, y1i = (iy + 1) >> 1;
       const float uo = (CG || ecg) ? __ldcg(u + vv) : u[vv];
       u[vv] = uo + 0.25f * (ucf(y0i * nCx + x0i) + ucf(y0i * nCx + x1i) + ucf(y1i * nCx + x0i) + ucf(y1i * nCx + x1i));
     }
     sync();
-    for (int vv = t0; vv < nv; vv += tn)
-      rl[vv] = ((CG || ecg) ? __ldcg(bl + vv) : bl[vv]) - vertex_apply<CG>(E, u, ncx, ncy, vv % nvx, vv / nvx);
+    auto el = [&](int cx, int cy) { return (size_t)(l == 1 ? xc[cx] + yc[cy] : cy * ncx + cx) * 16; };
+    const float* dinv = base + di.o_dinv[l];
+    for (int vv = t0; vv < nv; vv += tn) {
+      int ix, iy;
+      fine(vv, ix, iy);
+      const float r = ((CG || ecg) ? __ldcg(bl + vv) : bl[vv]) - vertex_apply<CG>(E, el, u, ncx, ncy, ix, iy);
+      // level 1: its post-smoothing is folded in here, once a vertex; the DG level then reads one value
+      rl[vv] = l == 1 ? (CG ? __ldcg(u + vv) : u[vv]) + omv * dinv[vv] * r : r;
+    }
     sync();
   };
   auto csync = [&]() { cl.sync(); };
@@ -593,41 +735,26 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
   using CgOn = std::integral_constant<bool, true>;
   using CgOff = std::integral_constant<bool, false>;
 
-  // A: b0 = Sigma_s v, x0 = omega Kcc^{-1} b0
-  for (int c = gt; c < nc; c += gn) {
-    float bc[4], xc[4];
+  // A: r0 = Sigma_s v - K x0, x0 = omega Kcc^{-1} Sigma_s v
+  for_tiles([](int, int, float*) {},
+            [&](int ix, int iy, const float* bc, const float*, float* kx) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) bc[q] = sgs[c] * (float)vb[(size_t)c * 4 + q];
-    store4(b0 + (size_t)c * 4, bc);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float kr[4];
-      load4(kinv + (size_t)c * 16 + r * 4, kr);
-      xc[r] = om * (kr[0] * bc[0] + kr[1] * bc[1] + kr[2] * bc[2] + kr[3] * bc[3]);
-    }
-    store4(x0 + (size_t)c * 4, xc);
-  }
-  cl.sync();
-  stage_t();
-  cl.sync();
-  // C: r0 = b0 - K x0
-  for (int c = gt; c < nc; c += gn) {
-    float kx[4], bc[4];
-    Kx(c, kx);
-    load4cg(b0 + (size_t)c * 4, bc);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) kx[q] = bc[q] - kx[q];
-    store4(r0 + (size_t)c * 4, kx);
-  }
+              for (int q = 0; q < 4; ++q) kx[q] = bc[q] - kx[q];
+              store4(r0 + (size_t)(iy * nx + ix) * 4, kx);
+            });
   cl.sync();
   // D: restriction to level 1, b1_v = sum over the cells around v of (P_T^T r0_T)_v
   {
     const int nvx = nx + 1, nv = nvx * (ny + 1);
     float* b1 = base + di.o_b[1];
+    const Split fine(nvx, nv);
     for (int vv = gt; vv < nv; vv += gn) {
-      const int ix = vv % nvx, iy = vv / nvx;
+      int ix, iy;
+      fine(vv, ix, iy);
       float s = 0.f;
+#pragma unroll
       for (int sy = 0; sy < 2; ++sy)
+#pragma unroll
         for (int sx = 0; sx < 2; ++sx) {
           const int cx = ix - 1 + sx, cy = iy - 1 + sy;
           if (cx < 0 || cx >= nx || cy < 0 || cy >= ny) continue;
@@ -663,46 +790,29 @@ __global__ void __launch_bounds__(kThreads) k_dsa_vcycle(const InstInfo* inst, c
   }
   cl.sync();
   for (int l = lsplit - 1; l >= 1; --l) ascend(l, gt, gn, csync, CgOn{}, true);
-  // E: x0 += P_c (u1 + omega D^{-1} r1), the post-smoothing of level 1 folded in
-  {
-    const float* u1 = base + di.o_u[1];
-    const float* r1 = base + di.o_r[1];
-    const float* d1 = base + di.o_dinv[1];
-    const float w1 = di.L > 1 ? omv : 0.f;
-    const int nvx = nx + 1;
-    auto uf = [&](int vv) { return ldg2(u1 + vv) + (w1 != 0.f ? w1 * d1[vv] * ldg2(r1 + vv) : 0.f); };
-    for (int c = gt; c < nc; c += gn) {
-      const int ix = c % nx, iy = c / nx;
-      const int v0 = iy * nvx + ix;
-      const float uq[4] = {uf(v0), uf(v0 + 1), uf(v0 + nvx), uf(v0 + nvx + 1)};
-      float xc[4];
-      load4cg(x0 + (size_t)c * 4, xc);
+  // E: z = v + x + omega Kcc^{-1} (Sigma_s v - K x), x = x0 + P_c w, w the post-smoothed correction of level 1
+  const float* w = base + (di.L > 1 ? di.o_r[1] : di.o_u[1]);
+  for_tiles(
+      [&](int ix, int iy, float* x) {
+        const float* p = w + iy * (nx + 1) + ix;
+        const float u0 = ldg2(p), u1 = ldg2(p + 1), u2 = ldg2(p + nx + 1), u3 = ldg2(p + nx + 2);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
+        for (int kk = 0; kk < 4; ++kk)
+          x[kk] += Pc[kk * 4] * u0 + Pc[kk * 4 + 1] * u1 + Pc[kk * 4 + 2] * u2 + Pc[kk * 4 + 3] * u3;
+      },
+      [&](int ix, int iy, const float* bc, const float* x0, float* kx) {
+        const int cls = xc[ix] + yc[iy];
+        const size_t c = (size_t)(iy * nx + ix) * 4;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) xc[kk] += Pc[kk * 4 + q] * uq[q];
-      store4(x0 + (size_t)c * 4, xc);
-    }
-  }
-  cl.sync();
-  stage_t();
-  cl.sync();
-  // G: z = v + x0 + omega Kcc^{-1} (b0 - K x0)
-  for (int c = gt; c < nc; c += gn) {
-    float kx[4], bc[4], xc[4];
-    Kx(c, kx);
-    load4cg(b0 + (size_t)c * 4, bc);
-    load4cg(x0 + (size_t)c * 4, xc);
+        for (int q = 0; q < 4; ++q) kx[q] = bc[q] - kx[q];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) kx[q] = bc[q] - kx[q];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float kr[4];
-      load4(kinv + (size_t)c * 16 + r * 4, kr);
-      const float x = xc[r] + om * (kr[0] * kx[0] + kr[1] * kx[1] + kr[2] * kx[2] + kr[3] * kx[3]);
-      zb[(size_t)c * 4 + r] = vb[(size_t)c * 4 + r] + (TV)x;
-    }
-  }
+        for (int r = 0; r < 4; ++r) {
+          float kr[4];
+          load4(kinv + (size_t)cls * 16 + r * 4, kr);
+          const float x = x0[r] + om * (kr[0] * kx[0] + kr[1] * kx[1] + kr[2] * kx[2] + kr[3] * kx[3]);
+          zb[c + r] = vb[c + r] + (TV)x;
+        }
+      });
 }
 
 // ------------------------------------------------------------------------------------------------ 1D slab
@@ -904,20 +1014,17 @@ int dsa_layout(rte_problem* p, std::vector<DsaInst>& out, long long& total) {
     d.hx = (float)p->inst[b].hx;
     d.hy = (float)p->inst[b].hy;
     const long long nc = (long long)d.nx * d.ny;
+    // classes where they are few next to the cells; cross-section profiles have none
+    d.per_cell = p->cellsig || 16LL * p->R * 2 > nc;
+    const long long ncls = d.per_cell ? nc : 16LL * p->R;
     d.o_sgs = o;
-    o = align4(o + nc);
+    o = align4(o + ncls);
     d.o_sga = o;
-    o = align4(o + nc);
+    o = align4(o + ncls);
     d.o_binv = o;
-    o += 8 * nc;
+    o += 8 * ncls;
     d.o_kinv = o;
-    o += 16 * nc;
-    d.o_b0 = o;
-    o += 4 * nc;
-    d.o_x0 = o;
-    o += 4 * nc;
-    d.o_t = o;
-    o += 8 * nc;
+    o += 16 * ncls;
     d.o_r0 = o;
     o += 4 * nc;
     int cx = d.nx, cy = d.ny, l = 1;
@@ -930,7 +1037,7 @@ int dsa_layout(rte_problem* p, std::vector<DsaInst>& out, long long& total) {
       d.ncy[l] = cy;
       const long long nv = (long long)(cx + 1) * (cy + 1);
       d.o_E[l] = o;
-      o += 16LL * cx * cy;
+      o += 16LL * (l == 1 ? ncls : (long long)cx * cy);
       d.o_dinv[l] = o;
       o = align4(o + nv);
       d.o_u[l] = o;
@@ -1045,15 +1152,29 @@ int dsa_prepare(rte_problem* p, int variant, cudaStream_t st) {
     RTE_CHECK_CUDA(cudaMemcpy(w->d_di.p, w->di.data(), w->di.size() * sizeof(DsaInst), cudaMemcpyHostToDevice));
   }
   const DsaConst k = dsa_constants(p, variant);
-  int max_nc = 0;
-  for (const DsaInst& d : w->di) max_nc = std::max(max_nc, d.nx * d.ny);
+  const int rx = p->cellsig ? p->nx[0] : p->rx, ry = p->cellsig ? p->ny[0] : p->ry;
+  int max_cls = 0, max_L = 0;
+  for (const DsaInst& d : w->di) {
+    max_cls = std::max(max_cls, d.per_cell ? d.nx * d.ny : 16 * p->R);
+    max_L = std::max(max_L, d.L);
+  }
   // cross-section profiles: the diffusion operator and its scattering source take the cell means (one "region"
   // per cell)
-  k_dsa_setup_cells<<<dim3((max_nc + kSetupThreads - 1) / kSetupThreads, p->B), kSetupThreads, 0, st>>>(
+  k_dsa_setup_cells<<<dim3((max_cls + kSetupThreads - 1) / kSetupThreads, p->B), kSetupThreads, 0, st>>>(
       w->d_di.p, w->data.p, p->cellsig ? p->d_sigc_s.p : p->d_sig_s.p, p->cellsig ? p->d_sigc_t.p : p->d_sig_t.p,
-      p->cellsig ? p->ncell : p->R, p->cellsig ? p->nx[0] : p->rx, p->cellsig ? p->ny[0] : p->ry, k);
+      p->cellsig ? p->ncell : p->R, rx, ry, k);
   count_launch();
-  k_dsa_setup_levels<<<p->B, kSetupThreads, 0, st>>>(w->d_di.p, w->data.p);
+  int l0 = 2;   // levels with at least kWideCells cells on some mesh: one launch each over all of the GPU
+  for (; l0 <= max_L; ++l0) {
+    int cells = 0;
+    for (const DsaInst& d : w->di)
+      if (l0 <= d.L) cells = std::max(cells, d.ncx[l0] * d.ncy[l0]);
+    if (cells < kWideCells) break;
+    k_dsa_setup_level<<<dim3((cells + kSetupThreads - 1) / kSetupThreads, p->B), kSetupThreads, 0, st>>>(
+        w->d_di.p, w->data.p, l0, rx, ry);
+    count_launch();
+  }
+  k_dsa_setup_levels<<<p->B, kSetupThreads, 0, st>>>(w->d_di.p, w->data.p, l0, rx, ry);
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
   w->lumped = k.lumped;
@@ -1088,7 +1209,12 @@ int dsa_launch(rte_problem* p, bool f64, const void* v, void* z, const int* acti
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p->B * kCluster);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
+  int codes = 0;   // class codes of the columns and rows
+  for (const DsaInst& d : w->di) codes = std::max(codes, d.nx + d.ny);
+  cfg.dynamicSmemBytes = codes * sizeof(int);
+  static std::atomic<size_t> granted[2][kMaxDevices];
+  if (f64) RTE_TRY(grant_smem(k_dsa_vcycle<double>, cfg.dynamicSmemBytes, granted[0]));
+  else RTE_TRY(grant_smem(k_dsa_vcycle<float>, cfg.dynamicSmemBytes, granted[1]));
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1097,13 +1223,14 @@ int dsa_launch(rte_problem* p, bool f64, const void* v, void* z, const int* acti
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const int rx = p->cellsig ? p->nx[0] : p->rx, ry = p->cellsig ? p->ny[0] : p->ry;
   if (f64)
     RTE_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_dsa_vcycle<double>, (const InstInfo*)p->d_inst.p,
-                                      (const DsaInst*)w->d_di.p, w->data.p, k, (const double*)v, (double*)z, active,
+                                      (const DsaInst*)w->d_di.p, w->data.p, k, rx, ry, (const double*)v, (double*)z, active,
                                       only));
   else
     RTE_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_dsa_vcycle<float>, (const InstInfo*)p->d_inst.p,
-                                      (const DsaInst*)w->d_di.p, w->data.p, k, (const float*)v, (float*)z, active,
+                                      (const DsaInst*)w->d_di.p, w->data.p, k, rx, ry, (const float*)v, (float*)z, active,
                                       only));
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
