@@ -504,16 +504,24 @@ namespace cg = cooperative_groups;
 // 602 us, no longer bound by HBM but by dependent loads and barriers (37 % of the issue slots; registers for two blocks
 // an SM).  Recomputing x at the nine cells of the stencil instead of the tile took 1119 us.
 constexpr int kTileX = 32, kTileY = kThreads / kTileX;
-__device__ __forceinline__ void load_v4(const float* p, float* x) { load4(p, x); }
-__device__ __forceinline__ void load_v4(const double* p, float* x) {
-  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-  x[0] = (float)a.x;
-  x[1] = (float)a.y;
-  x[2] = (float)b.x;
-  x[3] = (float)b.y;
+// a cell of v; VEC: v is 16-byte aligned (a caller's vector need not be)
+template <bool VEC, typename TV>
+__device__ __forceinline__ void load_v4(const TV* p, float* x) {
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = (float)p[q];
+  } else if constexpr (std::is_same<TV, float>::value) {
+    load4(p, x);
+  } else {
+    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+    x[0] = (float)a.x;
+    x[1] = (float)a.y;
+    x[2] = (float)b.x;
+    x[3] = (float)b.y;
+  }
 }
 
-template <typename TV>
+template <typename TV, bool VEC>
 __global__ void __launch_bounds__(kThreads, 2) k_dsa_vcycle(const InstInfo* inst, const DsaInst* dinfo, float* base,
                                                          DsaConst k, int rx, int ry, const TV* v, TV* z,
                                                          const int* active, const int* only) {
@@ -527,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_dsa_vcycle(const InstInfo* inst
   extern __shared__ int codes[];      // class codes of the columns [nx] and rows [ny]
   const DsaInst& di = dinfo[b];
   const InstInfo in = inst[b];
-  const int nx = di.nx, ny = di.ny, nc = nx * ny;
+  const int nx = di.nx, ny = di.ny;
   const float* sgs = base + di.o_sgs;
   const float* sga = base + di.o_sga;
   const float* binv = base + di.o_binv;
@@ -553,7 +561,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_dsa_vcycle(const InstInfo* inst
   __shared__ float4 X[kTileY + 4][kTileX + 4], Tx[kTileY][kTileX + 2], Ty[kTileY + 2][kTileX];
   // omega Kcc^{-1} Sigma_s v on a cell of class cls; bc: Sigma_s v
   auto smooth = [&](int c, int cls, float* bc, float* x) {
-    load_v4(vb + (size_t)c * 4, bc);
+    load_v4<VEC>(vb + (size_t)c * 4, bc);
     const float sg = sgs[cls];
 #pragma unroll
     for (int q = 0; q < 4; ++q) bc[q] *= sg;
@@ -1212,9 +1220,12 @@ int dsa_launch(rte_problem* p, bool f64, const void* v, void* z, const int* acti
   int codes = 0;   // class codes of the columns and rows
   for (const DsaInst& d : w->di) codes = std::max(codes, d.nx + d.ny);
   cfg.dynamicSmemBytes = codes * sizeof(int);
-  static std::atomic<size_t> granted[2][kMaxDevices];
-  if (f64) RTE_TRY(grant_smem(k_dsa_vcycle<double>, cfg.dynamicSmemBytes, granted[0]));
-  else RTE_TRY(grant_smem(k_dsa_vcycle<float>, cfg.dynamicSmemBytes, granted[1]));
+  const int vec = ((uintptr_t)v & 15) == 0, form = (f64 ? 2 : 0) + vec;
+  const void* const kern[4] = {(const void*)k_dsa_vcycle<float, false>, (const void*)k_dsa_vcycle<float, true>,
+                               (const void*)k_dsa_vcycle<double, false>, (const void*)k_dsa_vcycle<double, true>};
+  // the tiles' 30 KB count towards the 48 KB that need no grant
+  static std::atomic<size_t> granted[4][kMaxDevices];
+  if (cfg.dynamicSmemBytes > 16 * 1024) RTE_TRY(grant_smem(kern[form], cfg.dynamicSmemBytes + 32 * 1024, granted[form]));
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1224,14 +1235,12 @@ int dsa_launch(rte_problem* p, bool f64, const void* v, void* z, const int* acti
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int rx = p->cellsig ? p->nx[0] : p->rx, ry = p->cellsig ? p->ny[0] : p->ry;
-  if (f64)
-    RTE_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_dsa_vcycle<double>, (const InstInfo*)p->d_inst.p,
-                                      (const DsaInst*)w->d_di.p, w->data.p, k, rx, ry, (const double*)v, (double*)z, active,
-                                      only));
-  else
-    RTE_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_dsa_vcycle<float>, (const InstInfo*)p->d_inst.p,
-                                      (const DsaInst*)w->d_di.p, w->data.p, k, rx, ry, (const float*)v, (float*)z, active,
-                                      only));
+  const InstInfo* inst = p->d_inst.p;
+  const DsaInst* di = w->d_di.p;
+  float* data = w->data.p;
+  void* args[] = {(void*)&inst, (void*)&di, (void*)&data, (void*)&k, (void*)&rx, (void*)&ry,
+                  (void*)&v, (void*)&z, (void*)&active, (void*)&only};
+  RTE_CHECK_CUDA(cudaLaunchKernelExC(&cfg, kern[form], args));
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
   return RTE_OK;

@@ -404,11 +404,13 @@ constexpr int table_stride(int n, int bytes) { return n + (((n * bytes) / 16) % 
 // two meet every SK steps, so 32 columns are more than it can lag
 constexpr int kRing = 32;
 
-// Steps between a warp's bands: a row and one idle step, which clears the traces; and so many that what the last warp's
-// band leaves for the first warp's next one is SK + 1 steps old when it is read
+// Steps between a warp's bands: a row and one idle step, which clears the traces; so many that what the last warp's band
+// leaves for the first warp's next one is SK + 1 steps old when it is read; and so many that the next band's column c
+// is written to a ring's slot a group after the last column that shares the slot, at most (nx - 1) & ~31 further on, was
+// read, SK + 1 steps after it was written.  (The last rule asks for idle steps where nx is 1 to 15 above a multiple of 32.)
 __host__ __device__ constexpr int wave_period(int nx, int W, int SK) {
-  const int a = nx + 1, b = W * (32 + SK);
-  return a > b ? a : b;
+  const int a = nx + 1, b = W * (32 + SK), c = W > 1 ? ((nx - 1) & ~(kRing - 1)) + 2 * SK + 1 : 0;
+  return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
 __device__ __forceinline__ void group_sync(int warps) {
@@ -631,18 +633,28 @@ static void mesh_max(const rte_problem* p, int* nx, int* ny) {
   }
 }
 
-// FP64 tasks of one or two directions run in the Legendre basis
-static bool legendre(int prec, int D) { return prec == PREC_F64 && D <= 2; }
+constexpr size_t kMaxSmem = 227 * 1024;
 
-size_t wave_smem(const rte_problem* p, int prec, WaveShape s) {
+static size_t table_smem(const rte_problem* p, int prec, WaveShape s, int tw) {
   int nx, ny;
   mesh_max(p, &nx, &ny);
-  const int tw = prec == PREC_F32 ? Rot<float>::TW : (legendre(prec, s.D) ? Legendre<double>::TW : Modal<double>::TW);
   const int nc = prec == PREC_F32 ? Rot<float>::NC : Modal<double>::NC;
   const int bytes = prec == PREC_F32 ? 4 : 8;
   const size_t elems = (size_t)(p->R + 1) * table_stride(4 + s.D * tw, bytes) + ((s.D * nc + 3) & ~3) +
                        ((size_t)nx + (s.W - 1) * kRing) * s.D * 2;
   return elems * bytes;
+}
+
+// FP64 tasks of one or two directions run in the Legendre basis while its tables (sixteen entries a direction and region)
+// fit: up to about 1,300 regions with one direction, 750 with two.  The eigenbasis's four take twice as many and more.
+static bool legendre(const rte_problem* p, int prec, WaveShape s) {
+  return prec == PREC_F64 && s.D <= 2 && table_smem(p, prec, s, Legendre<double>::TW) <= kMaxSmem;
+}
+
+size_t wave_smem(const rte_problem* p, int prec, WaveShape s) {
+  return table_smem(p, prec, s, prec == PREC_F32          ? Rot<float>::TW
+                                : legendre(p, prec, s) ? Legendre<double>::TW
+                                                       : Modal<double>::TW);
 }
 
 // Registers a thread of each built shape takes (0: not built): they set how many warps an SM holds.
@@ -669,7 +681,7 @@ static int shape_regs(int prec, int D, int rpl) {
 }
 
 bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
-  if (s.W < 1 || s.W > 8 || shape_regs(prec, s.D, s.rpl) == 0 || wave_smem(p, prec, s) > 227 * 1024) return false;
+  if (s.W < 1 || s.W > 8 || shape_regs(prec, s.D, s.rpl) == 0 || wave_smem(p, prec, s) > kMaxSmem) return false;
   if (s.rpl == 2)   // the two rows of a lane share a table: they have to lie in one region in both sweep directions
     for (int b = 0; b < p->B; ++b)
       if (p->ny[b] % 2 || (p->ny[b] / p->ry) % 2) return false;
@@ -687,7 +699,7 @@ bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
 static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, const std::vector<int>& order) {
   const int SK = 4, per_sm = 65536 / (shape_regs(prec, s.D, s.rpl) * 32);
   const size_t smem = wave_smem(p, prec, s) + 1024;
-  const size_t slots = std::max(1, std::min(per_sm / s.W, (int)(227 * 1024 / smem)));
+  const size_t slots = std::max(1, std::min(per_sm / s.W, (int)(kMaxSmem / smem)));
   int chunks = 0;
   for (int q = 0; q < 4; ++q) chunks += (p->quad_start[q + 1] - p->quad_start[q] + s.D - 1) / s.D;
   double pipe, alone;
@@ -695,7 +707,7 @@ static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, co
     pipe = (s.rpl == 2 ? 13.0 * s.D + 30.0 : 10.0 * s.D + 40.0) / (s.W == 1 ? 0.65 : 0.75);
     alone = s.rpl == 2 ? 1750.0 : 50.0 * s.D + 300.0;
   } else if (prec == PREC_F64) {
-    const double instr = legendre(prec, s.D) ? 32.0 * s.D + 4.0 : 24.0 * s.D + 30.0;
+    const double instr = legendre(p, prec, s) ? 32.0 * s.D + 4.0 : 24.0 * s.D + 30.0;
     pipe = 19.0 * (1.0 + 0.05 * std::max(0, s.D - 4)) * instr;
     alone = 70.0 * instr;
   } else {
@@ -813,11 +825,16 @@ static int launch_f32(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t
 }
 
 template <bool BC>
-static int launch_f64(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t st) {
+static int launch_f64(const SweepArgs& a, WaveShape s, bool leg, size_t smem, cudaStream_t st) {
   using A = Modal<double>;
+  using Leg = Legendre<double>;
   switch (s.D) {
-    case 1: return launch_one<double, double, Legendre<double>, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 2: return launch_one<double, double, Legendre<double>, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st);
+    case 1:
+      return leg ? launch_one<double, double, Leg, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st)
+                 : launch_one<double, double, A, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st);
+    case 2:
+      return leg ? launch_one<double, double, Leg, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st)
+                 : launch_one<double, double, A, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st);
     case 3: return launch_one<double, double, A, 1, 3, 1, 4, BC, 2>(a, s.W, smem, st);
     case 4: return launch_one<double, double, A, 1, 4, 1, 4, BC, 1>(a, s.W, smem, st);
     case 8: return launch_one<double, double, A, 1, 8, 1, 4, BC, 1>(a, s.W, smem, st);
@@ -841,14 +858,15 @@ int launch_wave(const rte_problem* p, int prec, WaveShape s, bool in64, const Sw
   SweepArgs a = args;
   if (prec == PREC_F32) a.linv = p->d_rot32.p;
   else if (prec == PREC_DF) a.linv = p->d_modal_df.p;
-  else a.linv = legendre(prec, s.D) ? p->d_linv64.p : p->d_modal64.p;
+  const bool leg = legendre(p, prec, s);
+  if (prec == PREC_F64) a.linv = leg ? p->d_linv64.p : p->d_modal64.p;
   if (!wave_shape_ok(p, prec, s)) {
     set_error("sweep: shared-memory table too large for this mesh/region count");
     return RTE_ERR_UNSUPPORTED;
   }
   const size_t smem = wave_smem(p, prec, s);
   if (prec == PREC_F64)
-    return a.with_bc ? launch_f64<true>(a, s, smem, st) : launch_f64<false>(a, s, smem, st);
+    return a.with_bc ? launch_f64<true>(a, s, leg, smem, st) : launch_f64<false>(a, s, leg, smem, st);
   if (prec == PREC_DF) return launch_df(a, s, smem, st);
   return in64 ? launch_f32<double>(a, s, smem, st) : launch_f32<float>(a, s, smem, st);
 }

@@ -55,3 +55,52 @@ def test_operator_sweeps_match_oracle(name):
         assert rel(host["t64"][b], OT.T_apply(op, zb)) < 1e-13, b
         assert rel(host["b64"][b], rhs) < 1e-13, b
         assert rel(host["b32"][b], rhs) < 2e-5, b
+
+
+@pytest.mark.parametrize("D", [1, 2])
+def test_columns_that_share_a_trace_slot_across_bands(D):
+    """Two warps per task and rows a little longer than a multiple of 32: the next band's first columns take the slots
+    of the last ones, which the other warp still has to read."""
+    torch = torch_cuda()
+    B = lib()
+    from oracle import transport as OT
+    spec = spec2d([97, 73, 100, 129, 96], [130, 160, 100, 97, 128], n_polar=2, n_azim=8, rx=1, ry=1)
+    rs = np.random.RandomState(D)
+    ss, sa = np.exp(rs.uniform(0.0, np.log(3.0), (5, 1))), rs.uniform(0.0, 0.1, (5, 1))
+    gp = B.Problem(spec, ss, sa)
+    gp.set_sweep_variant(2, D)
+    ops = oracle_problems(spec, ss, sa)
+    z = rs.standard_normal(gp.n_dof)
+    w64, w32 = torch.empty(gp.n_dof, dtype=torch.float64, device="cuda"), torch.empty(gp.n_dof, device="cuda")
+    wdf = torch.empty_like(w64)
+    gp.apply_op(to_dev(z), w64)
+    gp.apply_op(to_dev(z), wdf, double_float=True)
+    gp.apply_op(to_dev(z, torch.float32), w32)
+    for b, op in enumerate(ops):
+        zb = split(z, gp.offsets)[b]
+        ref, ref32 = OT.Atilde_apply(op, zb), OT.Atilde_apply(op, zb.astype(np.float32).astype(np.float64))
+        assert rel(split(w64.cpu().numpy(), gp.offsets)[b], ref) < 1e-13, b
+        assert rel(split(wdf.cpu().numpy(), gp.offsets)[b], ref) < 1e-12, b
+        assert rel(split(w32.cpu().numpy().astype(np.float64), gp.offsets)[b], ref32) < 2e-5, b
+
+
+@pytest.mark.parametrize("n,D", [(40, 1), (28, 2)])
+def test_regions_beyond_the_legendre_tables(n, D):
+    """A region per cell, more than the sixteen-entry tables of D directions hold in shared memory: FP64 applies with a
+    task of D directions, chosen and without allocations."""
+    torch = torch_cuda()
+    B = lib()
+    from oracle import transport as OT
+    spec = spec2d([n], [n], n_polar=2, n_azim=4 * D, rx=n, ry=n)
+    rs = np.random.RandomState(n)
+    ss, sa = np.exp(rs.uniform(0.0, np.log(300.0), (1, n * n))), rs.uniform(0.0, 0.5, (1, n * n))
+    op = oracle_problems(spec, ss, sa)[0]
+    z = rs.standard_normal(4 * n * n)
+    ref = OT.Atilde_apply(op, z)
+    for how in ("pinned", "noalloc", "chosen"):
+        gp = B.Problem(spec, ss, sa)
+        w = torch.empty(gp.n_dof, dtype=torch.float64, device="cuda")
+        if how == "pinned":
+            gp.set_sweep_variant(0, D)
+        (gp.apply_op_noalloc if how == "noalloc" else gp.apply_op)(to_dev(z), w)
+        assert rel(w.cpu().numpy(), ref) < 1e-13, how
