@@ -1182,6 +1182,7 @@ struct Ws {
     int launches;
   };
   std::unordered_map<int, Graph> graphs;
+  const void* graph_partial = nullptr;   // the problem's partial-flux buffer that the graphs write and read
   std::vector<RomPlan> plans;   // persistent across solves (same ROM groups -> same buffers)
   // fused iteration kernels: vector chunks (instance, 256-dof chunk), per-instance ROM data, and the
   // co-resident grid sizes of the cooperative launches
@@ -1200,6 +1201,12 @@ struct Ws {
   void drop_graphs() {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second.exec);
     graphs.clear();
+  }
+  // before a run: the problem's partial-flux buffer grows with the task count of whatever sweep it is asked for (a
+  // pinned shape, another precision), and the graphs captured before hold the freed one
+  void check_graphs(const rte_problem* p) {
+    if (graph_partial != p->d_partial.p) drop_graphs();
+    graph_partial = p->d_partial.p;
   }
   DevBuf<double> bnorm, beta, est, nrm, norm_part;
   DevBuf<int> active, brk, flag, kcols, iters_left, list;
@@ -1384,6 +1391,7 @@ static int run_fgmres_t(SolveCtx& C, const TV* rhs, TV* x, bool zero_guess, cons
   static_assert(f64 || !sw64, "FP64 sweeps need FP64 vectors");
   rte_problem* p = C.p;
   Ws& W = *C.ws;
+  W.check_graphs(p);
   if (C.rec && !(f64 && sw64)) {
     set_error("run_fgmres: the first-cycle record needs an FP64 solve");
     return RTE_ERR_UNSUPPORTED;

@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(128) k_sweep2d(SweepArgs a) {
   const T bndy = (a.inflow_mask & (sy > 0 ? 4 : 8)) ? (T)gtr : (T)0;
   const bool sig_s = a.sig_s != nullptr;
   const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
-  T* part = reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
+  T* part = ANG ? nullptr
+                : reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
   T* psi = ANG ? reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off : nullptr;
   // angular output: element offsets (within the instance) of the blocks each of the task's directions
   // is stored to (its unique block, or the one or two N_Omega blocks it stands for), read once here
@@ -292,10 +293,12 @@ __global__ void __launch_bounds__(128) k_sweep2d(SweepArgs a) {
         tx1[d] = p2 + S3 * p3;
         ty0[d] = p0 + S3 * p2;
         ty1[d] = p1 + S3 * p3;
-        acc0 += wg[d] * p0;
-        acc1 += wg[d] * p1;
-        acc2 += wg[d] * p2;
-        acc3 += wg[d] * p3;
+        if (!ANG) {
+          acc0 += wg[d] * p0;
+          acc1 += wg[d] * p1;
+          acc2 += wg[d] * p2;
+          acc3 += wg[d] * p3;
+        }
         if (lane == 31 && band + 1 < nbands) {
           ybuf[(d * nx + col) * 2] = ty0[d];
           ybuf[(d * nx + col) * 2 + 1] = ty1[d];
@@ -305,10 +308,12 @@ __global__ void __launch_bounds__(128) k_sweep2d(SweepArgs a) {
           Vec4<T>::store(ring + d * 32 + (col & 7) * 4, p0, q1, q2, q3);
         }
       }
-      acc1 = sx > 0 ? acc1 : -acc1;
-      acc2 = sy > 0 ? acc2 : -acc2;
-      acc3 = (sx * sy) > 0 ? acc3 : -acc3;
-      Vec4<T>::store(part + 4 * c, acc0, acc1, acc2, acc3);
+      if (!ANG) {
+        acc1 = sx > 0 ? acc1 : -acc1;
+        acc2 = sy > 0 ? acc2 : -acc2;
+        acc3 = (sx * sy) > 0 ? acc3 : -acc3;
+        Vec4<T>::store(part + 4 * c, acc0, acc1, acc2, acc3);
+      }
     }
     if (ANG) {
       // lanes that completed an aligned 8-cell row segment (or their row) hand it to the warp: lanes
@@ -380,18 +385,13 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
     for (int e = threadIdx.x; e < R; e += blockDim.x) sgs[e] = reinterpret_cast<const T*>(a.sig_s)[(size_t)tk.b * R + e];
   const int cx = nx / a.rx, cy = ny / a.ry;
   for (int e = threadIdx.x; e < nx; e += blockDim.x) xreg[e] = e / cx;
-  T al[D], be[D], wg[D], wg1[D], wg2[D], wg3[D];
+  T al[D], be[D];
   const int sx = a.udir[tk.u0].sx, sy = a.udir[tk.u0].sy;
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const UDir u = a.udir[tk.u0 + d];
     al[d] = (T)(u.ax / in.hx);
     be[d] = (T)(u.ay / in.hy);
-    wg[d] = (T)u.w;
-    // quadrature weights with the reflection signs of the odd modes folded in
-    wg1[d] = sx > 0 ? wg[d] : -wg[d];
-    wg2[d] = sy > 0 ? wg[d] : -wg[d];
-    wg3[d] = sx * sy > 0 ? wg[d] : -wg[d];
   }
   // inflow traces of the constant g on the task's inflow faces (x face by the sign of Omega_x, y face by that of
   // Omega_y), zero on faces without inflow
@@ -400,7 +400,6 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
   const T bndy = (a.inflow_mask & (sy > 0 ? 4 : 8)) ? (T)gtr : (T)0;
   const bool sig_s = a.sig_s != nullptr;
   const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
-  T* part = reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
   T* psi = ANG ? reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off : nullptr;
   // angular output: element offsets (within the instance) of the blocks each of the task's directions
   // is stored to (its unique block, or the one or two N_Omega blocks it stands for), read once here
@@ -492,7 +491,6 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
         s1 = sx > 0 ? s1 : -s1;
         s2 = sy > 0 ? s2 : -s2;
         s3 = (sx * sy) > 0 ? s3 : -s3;
-        T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
           const T ax = al[d], by = be[d];
@@ -514,10 +512,6 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
           tx1[d] = p2 + S3 * p3;
           ty0[d] = p0 + S3 * p2;
           ty1[d] = p1 + S3 * p3;
-          acc0 += wg[d] * p0;
-          acc1 += wg1[d] * p1;
-          acc2 += wg2[d] * p2;
-          acc3 += wg3[d] * p3;
           if (lane == 31 && band + 1 < nb) {
             T* yb = ybuf + (size_t)band * D * nx * 2;
             yb[(d * nx + col) * 2] = ty0[d];
@@ -528,7 +522,6 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
             Vec4<T>::store(ring + d * 32 + (col & 7) * 4, p0, q1, q2, q3);
           }
         }
-        Vec4<T>::store(part + 4 * c, acc0, acc1, acc2, acc3);
       }
       if (ANG) {
         // lanes that completed an aligned 8-cell segment (or their row) hand it to the warp: lanes
@@ -597,7 +590,8 @@ __global__ void __launch_bounds__(128) k_sweep1d(SweepArgs a) {
   const T* linv = reinterpret_cast<const T*>(a.linv) + ((size_t)tk.b * a.nu + tk.u0) * R * 4;
   const T* sig_s = a.sig_s ? reinterpret_cast<const T*>(a.sig_s) + (size_t)tk.b * R : nullptr;
   const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
-  T* part = reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
+  T* part = ANG ? nullptr
+                : reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
   T* psi = ANG ? reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off +
                      (size_t)(a.psi_unique ? tk.u0 : u.dup[0]) * in.ndof
                 : nullptr;
@@ -643,9 +637,8 @@ __global__ void __launch_bounds__(128) k_sweep1d(SweepArgs a) {
     const T p0 = L[0] * r0 + L[1] * r1, p1 = L[2] * r0 + L[3] * r1;
     tx = p0 + S3 * p1;
     const T q1 = u.sx > 0 ? p1 : -p1;
-    part[2 * ix] = wg * p0;
-    part[2 * ix + 1] = wg * q1;
     if (ANG) { psi[2 * ix] = p0; psi[2 * ix + 1] = q1; }
+    else { part[2 * ix] = wg * p0; part[2 * ix + 1] = wg * q1; }
   }
 }
 
@@ -1043,9 +1036,10 @@ int autotune(rte_problem* p, int prec, bool ang, const void* src, void* psi, cud
   if (!ang && !p->cellsig) {
     for (const WaveShape& s : wave_shapes(p, prec, prec == PREC_F32 ? 4 : 2)) cands.push_back({s.D, -1, s});
   } else {
-    // partials for the largest candidate task count (D = 1)
-    RTE_TRY(ensure_tasks(p, 1));
-    RTE_TRY(ensure_partial(p, prec));
+    if (!ang) {   // partials for the largest candidate task count (D = 1)
+      RTE_TRY(ensure_tasks(p, 1));
+      RTE_TRY(ensure_partial(p, prec));
+    }
     for (int var = 0; var < 2; ++var) {
       if (p->cellsig && var != 1) continue;   // cross-section profiles: the warp-per-task kernel only
       if (var == 0 && max_bands(p) > 8) continue;
@@ -1274,13 +1268,11 @@ int launch_angular(rte_problem* p, bool f64, const void* src, int with_bc, void*
   const int prec = f64 ? PREC_F64 : PREC_F32;
   if (p->force_D == 0) RTE_TRY(autotune(p, prec, true, src, psi, st, scale_sigma_s, unique_layout));
   int D = pick_D(p, prec, true);
-  RTE_TRY(ensure_tasks(p, D));
-  RTE_TRY(ensure_partial(p, prec));
+  RTE_TRY(ensure_tasks(p, D));   // psi is the only output: no partial fluxes
   SweepArgs a;
   fill_args(p, a, prec);
   a.src = src;
   a.with_bc = with_bc ? 1 : 0;
-  a.partial = p->d_partial.p;
   a.psi = psi;
   a.psi_unique = unique_layout ? 1 : 0;
   if (scale_sigma_s) a.sig_s = sigma_s_arg(p, f64);
