@@ -144,13 +144,11 @@ struct rte_problem {
   rte::DevBuf<double> d_G;                    // [ntot] source moments
   rte::DevBuf<double> d_linv64;               // [B][nu][R][nd*nd]
   rte::DevBuf<float> d_linv32;
-  rte::DevBuf<float> d_linv_df;               // 1D: the same as double-float pairs (hi, lo) [..][2]
-  // 2D operator sweeps (wavefront.cu): cell tables per (instance, unique direction, region), [8] FP32, [4] FP64 and
-  // [4][2] double-float pairs
-  rte::DevBuf<float> d_rot32, d_modal_df;
-  rte::DevBuf<double> d_modal64;
+  rte::DevBuf<float> d_linv_df;               // as double-float pairs (hi, lo): 1D all entries, 2D the nine distinct ones
+                                              // [10][2] in scaled modes (wavefront.cu)
+  rte::DevBuf<float> d_rot32;                 // 2D: FP32 operator tables [B][nu][R][8] (wavefront.cu)
   rte::DevBuf<float> d_sig_s_df;              // [B][R][2] sigma_s as double-float pairs
-  rte::DevBuf<float> d_xdf;                   // [ntot][2] operator input split into double-float pairs
+  rte::DevBuf<float> d_xdf;                   // [ntot][2] source of a double-float (pairs) or FP64 sweep
   // sweep scratch (grown on demand)
   rte::DevBuf<unsigned char> d_partial;       // partial scalar fluxes per task
   // task lists per directions-per-warp value D (index D), built once; stable device pointers

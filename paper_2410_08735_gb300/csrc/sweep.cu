@@ -660,6 +660,40 @@ __global__ void k_reduce(const TP* partial, int ntask, const InstInfo* inst, int
   }
 }
 
+// Sigma_s x of the operator sweeps in FP64 (DF: divided by (1, sqrt3, sqrt3, 3), the scaled modes of the double-float
+// sweeps, and split into pairs), one thread a cell.  Every task of an instance reads the result: multiplying there takes 4 of
+// a step's 32 D + 4 FP64 instructions.
+template <bool DF>
+__global__ void k_scatter_source(const double* x, const InstInfo* inst, const double* sig_s, int R, int rx, int ry,
+                                 const int* active, float4* out) {
+  const int b = blockIdx.y;
+  if (active && !active[b]) return;
+  const InstInfo in = inst[b];
+  const int cx = in.nx / rx, cy = in.ny / ry;
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < in.nx * in.ny; c += gridDim.x * blockDim.x) {
+    const int iy = c / in.nx, ix = c - iy * in.nx;
+    const double sg = sig_s[(size_t)b * R + (iy / cy) * rx + ix / cx];
+    const long long o = in.off + 4ll * c;   // dofs are 8 bytes each in either form
+    double v[4];   // one by one: a caller's vector need not be aligned
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = x[o + e];
+    if constexpr (DF) {
+      const double f[4] = {sg, sg * 0.57735026918962576451, sg * 0.57735026918962576451, sg * (1.0 / 3.0)};
+      float h[4], l[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        v[e] *= f[e];
+        h[e] = (float)v[e];
+        l[e] = (float)(v[e] - (double)h[e]);
+      }
+      out[o / 2] = make_float4(h[0], l[0], h[1], l[1]);
+      out[o / 2 + 1] = make_float4(h[2], l[2], h[3], l[3]);
+    } else {
+      Vec4<double>::store(reinterpret_cast<double*>(out) + o, sg * v[0], sg * v[1], sg * v[2], sg * v[3]);
+    }
+  }
+}
+
 // phi = sum_j omega_j psi_j from an angular vector (K3).
 template <typename T>
 __global__ void k_scalar_flux(const T* psi, const double* w, int ndir, const InstInfo* inst, T* phi) {
@@ -991,7 +1025,7 @@ static WaveShape op_shape(rte_problem* p, int prec) {
     const int nb = std::min(max_bands(p), 8);
     const WaveShape s{p->pin_D, p->pin_var == 0 ? nb : (p->pin_var == 1 ? 1 : std::min(nb, 2)), 1};
     if (wave_shape_ok(p, prec, s) || prec == PREC_F32) return s;
-    return WaveShape{4, s.W, 1};   // the wider types take at most 8 (FP64) or 4 directions a task
+    return WaveShape{4, s.W, 1};   // the wider types take at most 4 directions a task
   }
   if (p->tuned_shape[prec].D > 0) return p->tuned_shape[prec];
   if (p->rule_shape[prec].D == 0) {
@@ -1122,6 +1156,28 @@ int prepare_sweeps(rte_problem* p) {
   return p->d_partial.ensure(bytes);
 }
 
+// Sigma_s x (2D, cross sections per region) into the problem's source buffer
+template <bool DF>
+static int scatter_source(rte_problem* p, const double* x, const int* d_active, cudaStream_t st) {
+  RTE_TRY(p->d_xdf.ensure((size_t)2 * p->ntot));
+  int maxc = 0;
+  for (int b = 0; b < p->B; ++b) maxc = std::max(maxc, p->nx[b] * p->ny[b]);
+  k_scatter_source<DF><<<dim3((maxc + 255) / 256, p->B), 256, 0, st>>>(x, p->d_inst.p, p->d_sig_s.p, p->R, p->rx, p->ry,
+                                                                      d_active, reinterpret_cast<float4*>(p->d_xdf.p));
+  count_launch();
+  RTE_CHECK_CUDA(cudaGetLastError());
+  return RTE_OK;
+}
+
+// The source of an FP64 operator sweep of a region problem, multiplied by Sigma_s beforehand
+static int scattered_f64(rte_problem* p, const int* d_active, SweepArgs& a, cudaStream_t st) {
+  if (p->dim == 1 || p->cellsig || !a.sig_s) return RTE_OK;
+  RTE_TRY(scatter_source<false>(p, reinterpret_cast<const double*>(a.src), d_active, st));
+  a.src = p->d_xdf.p;
+  a.sig_s = nullptr;
+  return RTE_OK;
+}
+
 // x (FP64) -> double-float pairs, all instances
 __global__ void k_split_df(const double* x, long long n, float2* out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -1144,14 +1200,18 @@ int launch_T_df(rte_problem* p, int mode, const double* x, const double* bvec, d
   RTE_TRY(p->d_xdf.ensure((size_t)2 * p->ntot));
   const WaveShape shape = op_shape(p, PREC_DF);
   RTE_TRY(ensure_op(p, PREC_DF, shape));
-  float2* xdf = reinterpret_cast<float2*>(p->d_xdf.p);
-  k_split_df<<<(unsigned)std::min<long long>(4096, (p->ntot + 255) / 256), 256, 0, st>>>(x, p->ntot, xdf);
-  count_launch();
   SweepArgs a;
   fill_args(p, a, PREC_DF);
-  a.src = xdf;
-  a.with_bc = 0;
-  a.sig_s = p->d_sig_s_df.p;
+  if (p->dim == 1) {
+    float2* xdf = reinterpret_cast<float2*>(p->d_xdf.p);
+    k_split_df<<<(unsigned)std::min<long long>(4096, (p->ntot + 255) / 256), 256, 0, st>>>(x, p->ntot, xdf);
+    count_launch();
+    a.src = xdf;
+    a.sig_s = p->d_sig_s_df.p;
+  } else {
+    RTE_TRY(scatter_source<true>(p, x, d_active, st));
+    a.src = p->d_xdf.p;
+  }
   a.partial = p->d_partial.p;
   a.active = d_active;
   RTE_TRY(launch_op_sweep(p, PREC_DF, shape, true, a, st));
@@ -1179,6 +1239,7 @@ int launch_T(rte_problem* p, int mode, bool f64, const void* src, bool in_f64, c
                                                    : nullptr;
   a.partial = p->d_partial.p;
   a.active = d_active;
+  if (f64) RTE_TRY(scattered_f64(p, d_active, a, st));
   RTE_TRY(launch_op_sweep(p, prec, shape, src64, a, st));
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
@@ -1217,6 +1278,7 @@ int launch_op_partials(rte_problem* p, bool f64, const void* z, bool in_f64, con
   a.sig_s = sigma_s_arg(p, f64);
   a.partial = p->d_partial.p;
   a.active = d_active;
+  if (f64) RTE_TRY(scattered_f64(p, d_active, a, st));
   return launch_op_sweep(p, prec, shape, in_f64, a, st);
 }
 

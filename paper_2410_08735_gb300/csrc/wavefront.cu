@@ -14,33 +14,33 @@
 //
 // Cell algebra.  In the frame reflected so that Omega_x, Omega_y > 0 the cell block is
 // L = alpha K(x)I + beta I(x)K + sigma_t I, K = 2 I + sqrt2 N with N^2 = -I.  L^{-1} is therefore a combination of
-// 1, N_x, N_y, N_x N_y, and two bases make that cheap:
+// 1, N_x, N_y, N_x N_y, which a basis can make use of:
 //  * Rot (FP32): both axes turned by 45 degrees, x' = (x_0 + x_1, x_1 - x_0) / sqrt2, an orthogonal change of basis.
 //    There N = [[0, a], [-1/a, 0]], a^2 = 2 + sqrt3, the outflow functional is (a, 1/a) and the inflow vector
 //    -(1/a, a).  With the second component of each axis scaled by q = 1/a^2, traces in units of a, the inflow enters
 //    both components of a pair with the same weight -alpha (or -beta), the outflow is a plain sum, and L^{-1} has
 //    eight distinct entries: 8 + 16 + 4 multiply-adds and adds and 4 for the quadrature, against 9 + 16 + 4 + 4 and
-//    sixteen entries in the Legendre basis, with the same rounding errors.
-//  * Modal (FP64, double-float): the eigenbasis of N on both axes.  A real 4-vector becomes two complex numbers
-//    A (modes (i, i)) and B (modes (i, -i)) on which L is multiplication by a complex number:
-//    A = G_A (S_A + alpha X + beta Y), B = G_B (S_B + alpha conj X + beta rho Y), X' = A + conj B, Y' = A + B:
-//    24 multiply-adds and adds and four table entries.  The eigenbasis is not orthogonal (condition number 3.7): with
-//    tables rounded once the FP64 apply is as close to 64-bit reference values as in the Legendre basis (7.5e-16 against
-//    4.9e-16 to 8.1e-16), but in FP32 the error would grow 1.7x, so FP32 keeps Rot (2.1e-7 either way).
-// The source is brought to the basis, and the summed flux back, once per cell and task (about 30 operations over D
-// directions).
+//    sixteen entries in the Legendre basis.  The source is brought to the basis, and the summed flux back, once per cell
+//    and task.  The error of an apply against 64-bit values is 0.6 to 1.1 times that of the former Legendre kernels (13
+//    batches of 1 to 256 instances; 2.4e-7 against 2.2e-7 on the uneven one below): the transforms add roundings that all
+//    directions of a task share, longer tasks save some in the sum of the partial fluxes.
+//  * Legendre (FP64): no change of basis, the cell inverses that the angular sweeps use.
+//  * Scaled (double-float): the Legendre modes scaled, which saves products.
+// The eigenbasis of N (complex products, 24 operations a direction and 30 a cell for its transforms) is no better choice for
+// these two: it is not orthogonal (condition number 3.7), in double-float the error of an apply is 15 to 70 % larger, and
+// in FP64 the 32 D operations of the Legendre basis are as few for tasks of up to four directions.
 //
 // FP32 runs pairs of directions in the packed multiply-add (fma.rn.f32x2): half the issue slots at the same rate.
 //
 // Bounds and measurements (one operator apply with the sum of its partial fluxes, GB300; before: Legendre basis, sixteen
 // table entries per direction and region, D <= 8, one warp per task or per band).  FP32, 64 x 256^2, 192 directions,
-// 8 x 8 regions: 2.08 -> 0.98 ms (D = 12, W = 2; 63 % of the load/store data pipe, 47 % of the FMA pipe); 256 instances
-// on 32^2, 64^2 and 128^2, 128 directions: 0.672 -> 0.331 ms (D = 8, two rows a lane: each table and shuffle serves two
-// cells); one 64^2 instance: 36.8 -> 28.8 us (latency of 131 steps).  FP64 is bound by the FP64 unit (19 SM cycles a warp
-// instruction), so by instructions per cell and direction: 7.93 -> 6.73 ms on the 256 instances, 0.919 -> 0.726 ms on
-// 10 x 80^2 with CL(30, 6), where D = 3 now divides quadrants of 24 and 21 directions (before: D = 1).  Double-float is
-// bound by FP32 issue: 3.61 -> 2.00 ms on 16 x 256^2 (sums of products with one renormalisation each, and the step loop
-// not unrolled: unrolled it missed the instruction cache, 3.48 ms).
+// 8 x 8 regions: 2.08 -> 0.98 ms (D = 12, W = 2; bound by the load/store data pipe); 256 instances on 32^2, 64^2 and 128^2,
+// 128 directions: 0.672 -> 0.336 ms (D = 8, two rows a lane: each table and shuffle serves two cells); one 64^2 instance:
+// 36.3 -> 28.9 us (latency of 131 steps).  FP64 is bound by the FP64 unit, which takes 64 cycles of an SM quarter for a warp
+// instruction, whatever the number of lanes, and 76 with all four quarters busy: so by instructions per step.
+// 7.92 -> 6.74 ms on the 256 instances (D = 4), 0.919 -> 0.527 ms on 10 x 80^2 with CL(30, 6) (D = 1).  Double-float is bound
+// by FP32 issue: 3.61 -> 2.01 ms on 16 x 256^2 (D = 4, W = 4; the step loop not unrolled: unrolled it missed the instruction
+// cache, 3.48 ms).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -127,62 +127,76 @@ template <typename T>
 __device__ __forceinline__ Dv<T, 1> up1(Dv<T, 1> v) { return Dv<T, 1>{up1(v.x)}; }
 __device__ __forceinline__ F2 up1(F2 v) { return F2{up1(v.x), up1(v.y)}; }
 
+// v or -v: the sign bit times a mask (0 or 1 << 31), which takes no floating-point instruction
+__device__ __forceinline__ float flip(float v, unsigned m) { return __uint_as_float(__float_as_uint(v) ^ m); }
+__device__ __forceinline__ double flip(double v, unsigned m) {
+  return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
+}
+__device__ __forceinline__ dfloat flip(dfloat v, unsigned m) { return dfloat(flip(v.hi, m), flip(v.lo, m)); }
+
 // ------------------------------------------------------------------------------------------- cell algebras
-// Sums of products.  FP64: multiply-adds.  Double-float: the high parts go through two-sums, what these miss and the
-// low parts are added up on the side, and one renormalisation ends the sum (the compensated dot product of Ogita, Rump
-// and Oishi, SIAM J. Sci. Comput. 26, 2005): 12 operations a term against 18 for a product and a sum of pairs.
-template <typename T>
-struct Sum {
-  T v;
-  __device__ __forceinline__ explicit Sum(T a) : v(a) {}
-  __device__ __forceinline__ Sum(T a, T b) : v(a * b) {}
-  __device__ __forceinline__ Sum add(T a, T b) const { return Sum(v + a * b); }
-  __device__ __forceinline__ Sum sub(T a, T b) const { return Sum(v - a * b); }
-  __device__ __forceinline__ T get() const { return v; }
-};
-template <>
-struct Sum<dfloat> {
+// Sums of products of double-floats: the high parts go through two-sums, what these miss and the low parts are added up
+// on the side, and one renormalisation ends the sum (the compensated dot product of Ogita, Rump and Oishi, SIAM J. Sci.
+// Comput. 26, 2005): 12 operations a term against 18 for a product and a sum of pairs.
+struct DfSum {
   float s, e;
-  __device__ __forceinline__ explicit Sum(dfloat a) : s(a.hi), e(a.lo) {}
-  __device__ __forceinline__ Sum(dfloat a, dfloat b) {
+  __device__ __forceinline__ explicit DfSum(dfloat a) : s(a.hi), e(a.lo) {}
+  __device__ __forceinline__ DfSum(dfloat a, dfloat b) {   // a b
     s = __fmul_rn(a.hi, b.hi);
     e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -s)));
   }
-  __device__ __forceinline__ Sum add(dfloat a, dfloat b) const {
-    Sum r(a, b);
-    const float t = __fadd_rn(s, r.s), bb = __fsub_rn(t, s);
-    const float er = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(r.s, bb));
-    r.s = t;
-    r.e = __fadd_rn(e, __fadd_rn(er, r.e));
+  __device__ __forceinline__ DfSum operator-() const {
+    DfSum r = *this;
+    r.s = -s;
+    r.e = -e;
     return r;
   }
-  __device__ __forceinline__ Sum sub(dfloat a, dfloat b) const { return add(dfloat(-a.hi, -a.lo), b); }
+  __device__ __forceinline__ DfSum operator+(DfSum b) const {
+    DfSum r = *this;
+    r.s = __fadd_rn(s, b.s);
+    const float bb = __fsub_rn(r.s, s);
+    const float er = __fadd_rn(__fsub_rn(s, __fsub_rn(r.s, bb)), __fsub_rn(b.s, bb));
+    r.e = __fadd_rn(e, __fadd_rn(er, b.e));
+    return r;
+  }
+  __device__ __forceinline__ dfloat raw() const { return dfloat(s, e); }   // not renormalised: for further sums only
   __device__ __forceinline__ dfloat get() const { return df_renorm(s, e); }
 };
 
 template <typename T>
 struct Rot {
-  static constexpr int TW = 8;   // table entries per direction and region
+  // table entries per direction and region, source factors per region, elements before the entries
+  static constexpr int TW = 8, FW = 4, HD = 4;
   static constexpr int NC = 3;   // constants per direction: -alpha, -beta, omega
   static constexpr double A2 = 3.7320508075688772935, Q = 0.26794919243112270647;
   // factors of the source's four Legendre components before to_basis, for reflection signs fx, fy
   __device__ static T factor(int k, double fx, double fy) {
     return (T)(0.5 * ((k & 1) ? fx : 1.0) * ((k & 2) ? fy : 1.0));
   }
+  __device__ __forceinline__ static void source(const T* q, const T* f, const unsigned*, T* S) {
+    T t[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[e] = q[e] * f[e];
+    to_basis(t, S);
+  }
+  // The transforms' rounding errors are shared by all directions of a task, so both are written for few roundings at the
+  // size of the leading component: the higher modes are added up first and meet it in one multiply-add (to), the scalings
+  // are part of the sums (from).  Against sums of pairs and separate products: 4 to 8 % less error of an apply.
   __device__ __forceinline__ static void to_basis(const T* t, T* S) {
-    const T u = t[0] + t[3], d = t[3] - t[0], e = t[1] + t[2], f = t[1] - t[2];
-    S[0] = u + e;
-    S[1] = (T)Q * (d + f);
-    S[2] = (T)Q * (d - f);
-    S[3] = (T)(Q * Q) * (u - e);
+    const T e = t[1] + t[2], f = t[1] - t[2];
+    S[0] = t[0] + (t[3] + e);
+    S[1] = fmaf((T)-Q, t[0], (T)Q * (t[3] + f));
+    S[2] = fmaf((T)-Q, t[0], (T)Q * (t[3] - f));
+    S[3] = fmaf((T)(Q * Q), t[0], (T)(Q * Q) * (t[3] - e));
   }
   __device__ __forceinline__ static void from_basis(const T* c, T* s) {
-    const T e0 = (T)0.5 * c[0], e1 = (T)(0.5 * A2) * c[1], e2 = (T)(0.5 * A2) * c[2], e3 = (T)(0.5 * A2 * A2) * c[3];
-    const T u = e0 + e3, v = e1 + e2, w = e0 - e3, z = e1 - e2;
-    s[0] = u - v;
-    s[1] = w + z;
-    s[2] = w - z;
-    s[3] = u + v;
+    constexpr T a = (T)(0.5 * A2), b = (T)(0.5 * A2 * A2);
+    const T h = (T)0.5 * c[0], v = c[1] + c[2], z = c[1] - c[2];
+    const T u = fmaf(b, c[3], h), w = fmaf(-b, c[3], h);
+    s[0] = fmaf(-a, v, u);
+    s[1] = fmaf(a, z, w);
+    s[2] = fmaf(-a, z, w);
+    s[3] = fmaf(a, v, u);
   }
   __device__ static void boundary(double g, T* t) {   // traces of a constant g: g / (sqrt2 a) (1, -q)
     const double v = g * 0.70710678118654752440 / 1.9318516525781365735;
@@ -215,77 +229,17 @@ struct Rot {
   }
 };
 
-// Constants of the eigenbasis: u = (1, mu), mu = -(1 + i sqrt2) / sqrt3, the left eigenvector of K to 2 + i sqrt2; both
-// axes scaled by c / 2 = (1 + 2 i sqrt2) / 2, which makes both outflow functionals (1, 1); sources divided by
-// kappa = c (2 + i sqrt2) / 2 = -1 + 5 i / sqrt2, which makes the x-inflow weights alpha; rho = conj(kappa) / kappa.
-template <typename T>
-struct Modal {
-  static constexpr int TW = 4;
-  static constexpr int NC = 5;   // alpha, beta, beta Re rho, beta Im rho, omega
-  __device__ static T factor(int k, double fx, double fy) {
-    return (T)(((k & 1) ? fx : 1.0) * ((k & 2) ? fy : 1.0));
-  }
-  __device__ __forceinline__ static void to_basis(const T* t, T* S) {
-    const T e = t[0] + t[3];
-    S[0] = (T)0.5 * (t[0] - t[3]);
-    S[1] = Sum<T>((T)0.35355339059327376220, e).add((T)(-0.61237243569579452455), t[1] + t[2]).get();
-    S[2] = Sum<T>((T)(-1.0 / 6.0), e).add((T)(-0.38490017945975050967), t[1]).add((T)0.57735026918962576451, t[2]).get();
-    S[3] = Sum<T>((T)(-0.58925565098878960367), e).add((T)0.47628967220784018576, t[1])
-               .add((T)0.20412414523193150818, t[2]).get();
-  }
-  // (Re A, R, Im X', Im Y') -> Legendre components, from A = (c/2)^2 (u (x) u) p, B = |c/2|^2 (u (x) conj u) p
-  __device__ __forceinline__ static void from_basis(const T* c, T* s) {
-    const T z = c[2] + c[3], d = c[3] - c[2];
-    s[0] = Sum<T>((T)(-2.0 / 9.0), c[0]).add((T)(1.0 / 3.0), c[1]).add((T)0.15713484026367723, z).get();
-    s[3] = Sum<T>((T)(-2.0 / 27.0), c[0]).add((T)(1.0 / 3.0), c[1]).add((T)(-0.10475656017578482), z).get();
-    const T f = Sum<T>((T)0.12830005981991683, c[0]).add((T)0.19245008972987526, c[1]).add((T)0.04536092116265145, z).get();
-    const T h = (T)0.13608276348795434 * d;
-    s[1] = f - h;
-    s[2] = f + h;
-  }
-  __device__ static void boundary(double g, T* t) {
-    t[0] = (T)(0.5 * g);
-    t[1] = (T)(1.4142135623730950488 * g);
-  }
-  __device__ static void constants(double al, double be, double w, T* c) {
-    c[0] = (T)al;
-    c[1] = (T)be;
-    c[2] = (T)(-23.0 * be / 27.0);
-    c[3] = (T)(0.52378280087892411 * be);
-    c[4] = (T)w;
-  }
-  template <typename V>
-  __device__ __forceinline__ static void cell(const V* S, V* X, V* Y, const V* m, const V* c, V* acc, bool zero) {
-    const T a = c[0].x, b = c[1].x, b1 = c[2].x, b2 = c[3].x, w = c[4].x;
-    const T x0 = X[0].x, x1 = X[1].x, y0 = Y[0].x, y1 = Y[1].x;
-    const T ar = Sum<T>(S[0].x).add(a, x0).add(b, y0).get(), ai = Sum<T>(S[1].x).add(a, x1).add(b, y1).get();
-    const T br = Sum<T>(S[2].x).add(a, x0).add(b1, y0).sub(b2, y1).get();
-    const T bi = Sum<T>(S[3].x).sub(a, x1).add(b1, y1).add(b2, y0).get();
-    const T Ar = Sum<T>(m[0].x, ar).sub(m[1].x, ai).get(), Ai = Sum<T>(m[0].x, ai).add(m[1].x, ar).get();
-    const T R = Sum<T>(Ar).add(m[2].x, br).sub(m[3].x, bi).get(), Bi = Sum<T>(m[2].x, bi).add(m[3].x, br).get();
-    X[0].x = Y[0].x = R;
-    X[1].x = Ai - Bi;
-    Y[1].x = Ai + Bi;
-    acc[0].x = zero ? w * Ar : Sum<T>(acc[0].x).add(w, Ar).get();
-    acc[1].x = zero ? w * R : Sum<T>(acc[1].x).add(w, R).get();
-    acc[2].x = zero ? w * X[1].x : Sum<T>(acc[2].x).add(w, X[1].x).get();
-    acc[3].x = zero ? w * Y[1].x : Sum<T>(acc[3].x).add(w, Y[1].x).get();
-  }
-};
-
-// The Legendre basis itself: no transforms, sixteen table entries (the cell inverses), 32 D + 4 operations a cell against
-// 24 D + 30.  FP64 tasks of one or two directions, which do not pay for the eigenbasis's transforms (26 x (64 x 22), 28
-// directions in quadrants of 8 and 6, D = 1: 271 us in the eigenbasis, 190 us here).
-template <typename T>
+// The Legendre basis itself (FP64): the sixteen entries of the cell inverses, 32 D operations a cell.  SIG: the kernel
+// multiplies the source by Sigma_s (4 more); else it comes multiplied, or unscaled where there is no Sigma_s.
+template <typename T, bool SIG>
 struct Legendre {
-  static constexpr int TW = 16;
+  static constexpr int TW = 16, FW = SIG ? 1 : 0, HD = 2;   // the factor is padded to 16 bytes
   static constexpr int NC = 5;   // alpha, beta, sqrt3 alpha, sqrt3 beta, omega
-  __device__ static T factor(int k, double fx, double fy) {
-    return (T)(((k & 1) ? fx : 1.0) * ((k & 2) ? fy : 1.0));
-  }
-  __device__ __forceinline__ static void to_basis(const T* t, T* S) {
+  __device__ static T factor(int, double, double) { return (T)1; }
+  // neg: sign bits of the four components in the reflected frame
+  __device__ __forceinline__ static void source(const T* q, const T* f, const unsigned* neg, T* S) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) S[e] = t[e];
+    for (int e = 0; e < 4; ++e) S[e] = flip(SIG ? q[e] * f[0] : q[e], neg[e]);
   }
   __device__ __forceinline__ static void from_basis(const T* c, T* s) {
 #pragma unroll
@@ -322,33 +276,67 @@ struct Legendre {
   }
 };
 
-// Unevaluated sums of two doubles, for the tables alone (two-sum and two-product as in dfloat.cuh)
-struct Dd {
-  double h, l;
+// Scaled Legendre modes (double-float): P = (1, sqrt3, sqrt3, 3) p, sources divided by the same, second traces times
+// sqrt3.  Outflows become plain sums and each product of a trace enters two components: 356 operations a cell and direction
+// against 400 in the Legendre basis, with the same rounding errors (in the eigenbasis of N 318 and transforms, and errors
+// 15 to 70 % larger).  The scalings cost nothing: they are part of the tables, the quadrature weights and the pass that
+// splits the source into pairs, which also multiplies it by Sigma_s.
+// As a combination of 1, N_x, N_y, N_x N_y, N = [[-1, sqrt3], [-sqrt3, 1]] / sqrt2, a cell inverse has nine distinct entries:
+// its diagonal d0 .. d3, +-u0, +-u1 between the x-modes, +-v0, +-v1 between the y-modes, and +-w.
+struct Scaled {
+  using T = dfloat;
+  static constexpr int TW = 10, FW = 0, HD = 0;   // nine entries and a spare one, for 16-byte boundaries
+  static constexpr int NC = 8;   // alpha, alpha / 3, beta, beta / 3, omega / (1, sqrt3, sqrt3, 3)
+  __device__ static double scale(int k) { return k == 0 ? 1.0 : (k == 3 ? 3.0 : 1.7320508075688772); }
+  __device__ static T factor(int, double, double) { return (T)0; }
+  __device__ __forceinline__ static void source(const T* q, const T*, const unsigned* neg, T* S) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) S[e] = flip(q[e], neg[e]);
+  }
+  __device__ __forceinline__ static void from_basis(const T* c, T* s) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] = df_renorm(c[e].hi, c[e].lo);
+  }
+  __device__ static void boundary(double g, T* t) {
+    t[0] = (T)g;
+    t[1] = (T)0;
+  }
+  __device__ static void constants(double al, double be, double w, T* c) {
+    c[0] = (T)al;
+    c[1] = (T)(al / 3.0);
+    c[2] = (T)be;
+    c[3] = (T)(be / 3.0);
+    for (int k = 0; k < 4; ++k) c[4 + k] = (T)(w / scale(k));
+  }
+  template <typename V>
+  __device__ __forceinline__ static void cell(const V* S, V* X, V* Y, const V* m, const V* c, V* acc, bool zero) {
+    const DfSum x0(c[0].x, X[0].x), x1(c[1].x, X[1].x), y0(c[2].x, Y[0].x), y1(c[3].x, Y[1].x);
+    const T r0 = (DfSum(S[0].x) + x0 + y0).get(), r1 = (DfSum(S[1].x) + -x0 + y1).get();
+    const T r2 = (DfSum(S[2].x) + x1 + -y0).get(), r3 = (DfSum(S[3].x) + -x1 + -y1).get();
+    auto dot = [](T m0, T a0, T m1, T a1, T m2, T a2, T m3, T a3) {
+      return (DfSum(m0, a0) + DfSum(m1, a1) + DfSum(m2, a2) + DfSum(m3, a3)).get();
+    };
+    const T d0 = m[0].x, d1 = m[1].x, d2 = m[2].x, d3 = m[3].x, u0 = m[4].x, u1 = m[5].x, v0 = m[6].x, v1 = m[7].x, w = m[8].x;
+    const T q[4] = {dot(d0, r0, u0, r1, v0, r2, w, r3), dot(-u0, r0, d1, r1, -w, r2, v1, r3),
+                    dot(-v0, r0, -w, r1, d2, r2, u1, r3), dot(w, r0, -v1, r1, -u1, r2, d3, r3)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const DfSum wq(c[4 + i].x, q[i]);
+      acc[i].x = zero ? wq.raw() : (DfSum(acc[i].x) + wq).raw();   // renormalised once, in from_basis
+    }
+    X[0].x = (DfSum(q[0]) + DfSum(q[1])).get();
+    X[1].x = (DfSum(q[2]) + DfSum(q[3])).get();
+    Y[0].x = (DfSum(q[0]) + DfSum(q[2])).get();
+    Y[1].x = (DfSum(q[1]) + DfSum(q[3])).get();
+  }
 };
-__device__ Dd dd_sum(double a, double b) {
-  const double s = __dadd_rn(a, b), t = __dsub_rn(s, a);
-  return Dd{s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, t)), __dsub_rn(b, t))};
-}
-__device__ Dd dd_add(Dd a, Dd b) {
-  const Dd s = dd_sum(a.h, b.h);
-  return dd_sum(s.h, __dadd_rn(s.l, __dadd_rn(a.l, b.l)));
-}
-__device__ Dd dd_mul(Dd a, Dd b) {
-  const double p = __dmul_rn(a.h, b.h);
-  return dd_sum(p, __fma_rn(a.l, b.h, __fma_rn(a.h, b.l, __fma_rn(a.h, b.h, -p))));
-}
-__device__ double dd_div(Dd a, Dd b) {   // a / b to double
-  const double q = __ddiv_rn(a.h, b.h);
-  const Dd p = dd_mul(Dd{q, 0.0}, b), r = dd_add(a, Dd{-p.h, -p.l});
-  return __dadd_rn(q, __ddiv_rn(r.h, b.h));
-}
 
-// Tables per (instance, unique direction, region): Rot FP32 [8], Modal FP64 [4] and double-float [4] pairs.
+// FP32 tables [8] per (instance, unique direction, region).
 // l_1 = c_0 + i sqrt2 (alpha + beta), l_2 = c_0 + i sqrt2 (alpha - beta), c_0 = 2 (alpha + beta) + sigma_t, are the
-// eigenvalues of L on (i, i) and (i, -i); L^{-1} = g + g_x N_x + g_y N_y + g_xy N_x N_y follows from 1 / l_1, 1 / l_2.
+// eigenvalues of L on the products of eigenvectors of N; L^{-1} = g + g_x N_x + g_y N_y + g_xy N_x N_y follows from
+// 1 / l_1, 1 / l_2.
 __global__ void k_wave_tables(int B, int nu, int R, const InstInfo* inst, const UDir* ud, const double* sig_t,
-                              float* rot, double* modal, float* modal_df) {
+                              float* rot) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (tid >= (long long)B * nu * R) return;
   const int r = (int)(tid % R), u = (int)((tid / R) % nu), b = (int)(tid / ((long long)R * nu));
@@ -364,27 +352,12 @@ __global__ void k_wave_tables(int B, int nu, int R, const InstInfo* inst, const 
   const double a3 = 7.2097685201075047693, b3 = 1.0 / a3;
   const double t[8] = {g, gx * a3, -gx * b3, gy * a3, -gy * b3, gxy * a3 * a3, -gxy, gxy * b3 * b3};
   for (int k = 0; k < 8; ++k) rot[tid * 8 + k] = (float)t[k];
-  // G = kappa / l, rounded once: what the rounding of the tables loses adds up along a ray
-  const Dd s2d{1.4142135623730951, -9.667293313452913e-17}, kid{3.5355339059327378, -1.3066003037380717e-16};
-  const Dd sum = dd_sum(al, be), dif = dd_sum(al, -be);
-  const Dd c0d = dd_add(Dd{2.0 * sum.h, 2.0 * sum.l}, Dd{sg, 0.0});
-  const Dd i1d = dd_mul(s2d, sum), i2d = dd_mul(s2d, dif);
-  const Dd n1d = dd_add(dd_mul(c0d, c0d), dd_mul(i1d, i1d)), n2d = dd_add(dd_mul(c0d, c0d), dd_mul(i2d, i2d));
-  const Dd nc{-c0d.h, -c0d.l};
-  const double m[4] = {dd_div(dd_add(dd_mul(kid, i1d), nc), n1d), dd_div(dd_add(dd_mul(kid, c0d), i1d), n1d),
-                       dd_div(dd_add(dd_mul(kid, i2d), nc), n2d), dd_div(dd_add(dd_mul(kid, c0d), i2d), n2d)};
-  for (int k = 0; k < 4; ++k) {
-    modal[tid * 4 + k] = m[k];
-    const float h = (float)m[k];
-    modal_df[2 * (tid * 4 + k)] = h;
-    modal_df[2 * (tid * 4 + k) + 1] = (float)(m[k] - (double)h);
-  }
 }
 
 int build_wave_tables(rte_problem* p) {
   const long long n = (long long)p->B * p->nu * p->R;
   k_wave_tables<<<(unsigned)((n + 127) / 128), 128>>>(p->B, p->nu, p->R, p->d_inst.p, p->d_udir.p, p->d_sig_t.p,
-                                                      p->d_rot32.p, p->d_modal64.p, p->d_modal_df.p);
+                                                      p->d_rot32.p);
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
   return RTE_OK;
@@ -402,14 +375,14 @@ constexpr int table_stride(int n, int bytes) { return n + (((n * bytes) / 16) % 
 
 // Columns a trace buffer between neighbouring warps keeps: the reader follows SK + 1 steps behind the writer, and the
 // two meet every SK steps, so 32 columns are more than it can lag
-constexpr int kRing = 32;
+constexpr int kRingCols = 32;
 
 // Steps between a warp's bands: a row and one idle step, which clears the traces; so many that what the last warp's band
 // leaves for the first warp's next one is SK + 1 steps old when it is read; and so many that the next band's column c
 // is written to a ring's slot a group after the last column that shares the slot, at most (nx - 1) & ~31 further on, was
 // read, SK + 1 steps after it was written.  (The last rule asks for idle steps where nx is 1 to 15 above a multiple of 32.)
 __host__ __device__ constexpr int wave_period(int nx, int W, int SK) {
-  const int a = nx + 1, b = W * (32 + SK), c = W > 1 ? ((nx - 1) & ~(kRing - 1)) + 2 * SK + 1 : 0;
+  const int a = nx + 1, b = W * (32 + SK), c = W > 1 ? ((nx - 1) & ~(kRingCols - 1)) + 2 * SK + 1 : 0;
   return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
@@ -419,12 +392,13 @@ __device__ __forceinline__ void group_sync(int warps) {
 }
 
 // BC: non-zero inflow on the x-faces (the right-hand side).  MINB: resident CTAs of 256 threads that the registers have
-// to allow.
-template <typename T, typename TI, typename ALG, int VW, int NV, int RPL, int PF, bool BC, int MINB>
+// to allow.  GT: the tables stay in global memory (problems with more regions than shared memory holds).
+template <typename T, typename TI, typename ALG, int VW, int NV, int RPL, int PF, bool BC, int MINB, bool GT>
 __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
   using V = Dv<T, VW>;
-  constexpr int D = VW * NV, TW = ALG::TW, NC = ALG::NC, SK = PF;
-  constexpr int RS = table_stride(4 + D * TW, sizeof(T));
+  constexpr int D = VW * NV, TW = ALG::TW, FW = ALG::FW, NC = ALG::NC, SK = PF;
+  constexpr int HD = ALG::HD, RS = table_stride(HD + D * TW, sizeof(T));
+  static_assert(!GT || VW == 1, "global tables are read one direction at a time");
   const SweepTask tk = a.tasks[blockIdx.x];
   if (a.active && !a.active[tk.b]) return;   // uniform for the CTA
   const InstInfo in = a.inst[tk.b];
@@ -433,24 +407,28 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
   const int nb = (ny + 32 * RPL - 1) / (32 * RPL);
   const int W = min((int)(blockDim.x >> 5), nb);   // warps that have a band
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tab = reinterpret_cast<T*>(smem_raw);          // [R + 1][RS]: source factors [4], cell tables [NV][TW][VW]
-  T* cst = tab + (size_t)(R + 1) * RS;              // [NV][NC][VW], padded to 4
+  T* tab = reinterpret_cast<T*>(smem_raw);          // [R + 1][RS]: [HD], cell tables [NV][TW][VW]; source factors [FW]
+  T* cst = tab + (GT ? 0 : (size_t)(R + 1) * RS);   // [NV][NC][VW], padded to 4
   T* yfull = cst + ((NV * NC * VW + 3) & ~3);       // [nx][NV][2][VW] from the last warp's band to the first warp's next
-  T* yring = yfull + (size_t)nx * D * 2;            // [W - 1][kRing][NV][2][VW] from a warp's band to the next warp's
+  T* yring = yfull + (size_t)nx * D * 2;            // [W - 1][kRingCols][NV][2][VW] from a warp's band to the next warp's
+  float4* sring = reinterpret_cast<float4*>(yring + (size_t)(W - 1) * kRingCols * D * 2);   // double-float: [W][PF][2][32]
   const UDir u0 = a.udir[tk.u0];
   const int sx = u0.sx, sy = u0.sy;
   // Stage the tables.  Directions beyond the task's own are zero (they carry no flux); so is the whole table R, which
   // lanes outside the mesh read: their traces become zero, the vacuum inflow of the row they enter next.
-  for (int e = threadIdx.x; e < (R + 1) * D * TW; e += blockDim.x) {
-    const int k = e % TW, r = (e / TW) % (R + 1), d = e / (TW * (R + 1));
-    tab[r * RS + 4 + ((d / VW) * TW + k) * VW + d % VW] =
-        r < R && d < ndir ? reinterpret_cast<const T*>(a.linv)[(((size_t)tk.b * a.nu + tk.u0 + d) * R + r) * TW + k]
-                          : (T)0;
-  }
-  for (int e = threadIdx.x; e < (R + 1) * 4; e += blockDim.x) {
-    const int r = e >> 2;
-    const T f = r < R ? ALG::factor(e & 3, (double)sx, (double)sy) : (T)0;
-    tab[r * RS + (e & 3)] = a.sig_s && r < R ? f * reinterpret_cast<const T*>(a.sig_s)[(size_t)tk.b * R + r] : f;
+  const T* lin = reinterpret_cast<const T*>(a.linv) + ((size_t)tk.b * a.nu + tk.u0) * R * TW;
+  const T* sgr = a.sig_s ? reinterpret_cast<const T*>(a.sig_s) + (size_t)tk.b * R : nullptr;
+  if constexpr (!GT) {
+    for (int e = threadIdx.x; e < (R + 1) * D * TW; e += blockDim.x) {
+      const int k = e % TW, r = (e / TW) % (R + 1), d = e / (TW * (R + 1));
+      tab[r * RS + HD + ((d / VW) * TW + k) * VW + d % VW] = r < R && d < ndir ? lin[((size_t)d * R + r) * TW + k] : (T)0;
+    }
+    if constexpr (FW > 0)
+      for (int e = threadIdx.x; e < (R + 1) * FW; e += blockDim.x) {
+        const int r = e / FW;
+        const T f = r < R ? ALG::factor(e % FW, (double)sx, (double)sy) : (T)0;
+        tab[r * RS + e % FW] = sgr && r < R ? f * sgr[r] : f;
+      }
   }
   for (int d = threadIdx.x; d < D; d += blockDim.x) {
     T c[NC];
@@ -469,49 +447,71 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
   ALG::boundary((a.inflow_mask & (sx > 0 ? 1 : 2)) ? gtr : 0.0, bx);
   ALG::boundary((a.inflow_mask & (sy > 0 ? 4 : 8)) ? gtr : 0.0, by);
   for (int e = threadIdx.x; e < nx * D * 2; e += blockDim.x) yfull[e] = by[(e / VW) & 1];
+  if constexpr (std::is_same<T, dfloat>::value)   // lanes without a cell read their slots too
+    for (int e = threadIdx.x; e < W * PF * 64; e += blockDim.x) sring[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   if (warp >= W) return;
   const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
   T* part = reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
   constexpr int YC = D * 2;   // elements per column of a trace buffer
-  const T* yin = warp == 0 ? yfull : yring + (size_t)(warp - 1) * kRing * YC;
-  T* yout = warp == W - 1 ? yfull : yring + (size_t)warp * kRing * YC;
+  const T* yin = warp == 0 ? yfull : yring + (size_t)(warp - 1) * kRingCols * YC;
+  T* yout = warp == W - 1 ? yfull : yring + (size_t)warp * kRingCols * YC;
   const unsigned yin_s = (unsigned)__cvta_generic_to_shared(yin);
-  const int min_ = warp == 0 ? -1 : kRing - 1, mout = warp == W - 1 ? -1 : kRing - 1;
+  const int min_ = warp == 0 ? -1 : kRingCols - 1, mout = warp == W - 1 ? -1 : kRingCols - 1;
   const int cx = nx / a.rx, cy = ny / a.ry, dx = sx > 0 ? 1 : -1;
   const int P = wave_period(nx, W, SK);
   const int last = (nb - 1) / W;
   const int nsteps = last * P + (nb - 1 - last * W) * (32 + SK) + 31 + nx;
   const unsigned mx = 0xffffffffu / (unsigned)cx + 1u, my = 0xffffffffu / (unsigned)cy + 1u;   // i / c = mulhi(i, m); c = 1: see div
   auto div = [](int i, unsigned m) { return m ? (int)__umulhi((unsigned)i, m) : i; };
-  const int rdx = sx > 0 ? RS : -RS, rowstep = 32 * RPL * W, dy = sy > 0 ? nx : -nx;
+  constexpr int RI = GT ? 1 : RS;   // table index per region
+  const int rdx = sx > 0 ? RI : -RI, rowstep = 32 * RPL * W, dy = sy > 0 ? nx : -nx;
   auto cell0 = [&](int row) { return (sy > 0 ? row : ny - 1 - row) * nx + (sx > 0 ? 0 : nx - 1); };
   auto reg0 = [&](int row) {   // table of the row's first cell
     const int rr = div(row, my);
-    return ((sy > 0 ? rr : a.ry - 1 - rr) * a.rx + (sx > 0 ? 0 : a.rx - 1)) * RS;
+    return ((sy > 0 ? rr : a.ry - 1 - rr) * a.rx + (sx > 0 ? 0 : a.rx - 1)) * RI;
   };
   int row = 32 * RPL * warp + RPL * lane, col = -((32 + SK) * warp + lane);
   int cell = cell0(row), reg = reg0(row);
   int prow = row, pcol = col, pcell = cell;   // source prefetch, PF steps ahead
-  auto fetch = [&](TI* dst) {
+  // A double-float step is hundreds of instructions: unrolled, a group would not fit the instruction cache.  Its sources
+  // then cannot rotate through registers (moving one waits for its load): they go to a ring in shared memory instead.
+  constexpr bool kRing = std::is_same<T, dfloat>::value;
+  auto fetch = [&](TI* dst, unsigned slot) {
 #pragma unroll
     for (int r = 0; r < RPL; ++r)
-      if ((unsigned)pcol < (unsigned)nx && prow + r < ny)
-        Vec4<TI>::load(src + 4 * (long long)(pcell + dx * pcol + r * dy), dst[4 * r], dst[4 * r + 1], dst[4 * r + 2],
-                       dst[4 * r + 3]);
+      if ((unsigned)pcol < (unsigned)nx && prow + r < ny) {
+        const TI* from = src + 4 * (long long)(pcell + dx * pcol + r * dy);
+        if constexpr (kRing) {
+          asm volatile("cp.async.cg.shared.global [%0], [%2], 16; cp.async.cg.shared.global [%1], [%3], 16;" ::"r"(slot),
+                       "r"(slot + 512), "l"(from), "l"(from + 2)
+                       : "memory");
+        } else {
+          Vec4<TI>::load(from, dst[4 * r], dst[4 * r + 1], dst[4 * r + 2], dst[4 * r + 3]);
+        }
+      }
+    if constexpr (kRing) asm volatile("cp.async.commit_group;" ::: "memory");
     ++pcol;
     const bool wrap = pcol == P;
     pcol = wrap ? 0 : pcol;
     prow = wrap ? prow + rowstep : prow;
     pcell = wrap ? pcell + (sy > 0 ? rowstep * nx : -rowstep * nx) : pcell;
   };
-  TI q[PF][4 * RPL];
+  const unsigned ring = (unsigned)__cvta_generic_to_shared(sring) + (warp * PF * 64 + lane) * 16;   // this lane's slots
+  TI q[kRing ? 1 : PF][4 * RPL];
+  if constexpr (kRing) {
+    static_assert(!kRing || (RPL == 1 && sizeof(TI) == 8), "a slot holds one cell");
+#pragma unroll 1
+    for (int k = 0; k < PF - 1; ++k) fetch(nullptr, ring + k * 1024);
+  } else {
 #pragma unroll
-  for (int k = 0; k < PF; ++k) {
+    for (int k = 0; k < PF; ++k) {
 #pragma unroll
-    for (int e = 0; e < 4 * RPL; ++e) q[k][e] = TI(0);
-    fetch(q[k]);
+      for (int e = 0; e < 4 * RPL; ++e) q[k][e] = TI(0);
+      fetch(q[k], 0);
+    }
   }
+  const unsigned neg[4] = {0u, sx > 0 ? 0u : 1u << 31, sy > 0 ? 0u : 1u << 31, sx * sy > 0 ? 0u : 1u << 31};
   // direction constants: in registers in FP32, re-read from shared memory where a value takes two registers
   constexpr bool kRegConst = sizeof(T) == 4;
   V creg[kRegConst ? NV : 1][NC];
@@ -531,14 +531,13 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
     }
   const bool first = lane == 0, tail = lane == 31;
   using BlkY = Blk<V, 2>;
-  // A double-float step is over a thousand instructions: unrolled, a group would not fit the instruction cache
-  constexpr int UNR = std::is_same<T, dfloat>::value ? 1 : PF;
+  constexpr int UNR = kRing ? 1 : PF;
   for (int s0 = 0; s0 < nsteps; s0 += PF) {
 #pragma unroll UNR
     for (int k0 = 0; k0 < PF; ++k0) {
-      const int kk = UNR == 1 ? 0 : k0;
+      const int kk = kRing ? 0 : k0;
       const bool act = (unsigned)col < (unsigned)nx && row < ny;
-      const int ro = act ? reg + rdx * div(col, mx) : R * RS;
+      const int ro = act ? reg + rdx * div(col, mx) : (GT ? 0 : R * RS);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Y[v][0] = up1(Y[v][0]);
@@ -549,69 +548,97 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) load_traces(take, at + v * 2 * VW * (int)sizeof(T), Y[v]);
       }
-      if constexpr (BC) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-#pragma unroll
-          for (int e = 0; e < 2; ++e)
-#pragma unroll
-            for (int r = 0; r < RPL; ++r)
-              if (col == 0) X[r][v][e] = V::all(bx[e]);
+      if constexpr (kRing) {   // the slot of the step before takes the source three steps ahead
+        fetch(nullptr, ring + ((k0 + PF - 1) % PF) * 1024);
+        asm volatile("cp.async.wait_group %0;" ::"n"(PF - 1) : "memory");
       }
-      const Blk<T, 4> sg = *reinterpret_cast<const Blk<T, 4>*>(tab + ro);
-      V S[RPL][4], acc[RPL][4];
+      {
+        if constexpr (BC) {
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) {
-        T t[4], Sr[4];
+          for (int v = 0; v < NV; ++v)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) t[e] = (T)q[kk][4 * r + e] * sg.v[e];
-        ALG::to_basis(t, Sr);
+            for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) S[r][e] = V::all(Sr[e]);
-      }
-      if constexpr (UNR == 1) {
+              for (int r = 0; r < RPL; ++r)
+                if (col == 0) X[r][v][e] = V::all(bx[e]);
+        }
+        constexpr int FB = FW > 0 ? FW : 1;
+        Blk<T, FB> sg;
+        if constexpr (FW > 0) {
+          if constexpr (GT) sg.v[0] = sgr ? sgr[ro] : (T)1;
+          else sg = *reinterpret_cast<const Blk<T, FB>*>(tab + ro);
+        }
+        V S[RPL][4], acc[RPL][4];
 #pragma unroll
-        for (int k = 0; k + 1 < PF; ++k)
+        for (int r = 0; r < RPL; ++r) {
+          T t[4], Sr[4];
 #pragma unroll
-          for (int e = 0; e < 4 * RPL; ++e) q[k][e] = q[k + 1][e];
-        fetch(q[PF - 1]);
-      } else {
-        fetch(q[kk]);
-      }
+          for (int e = 0; e < 4; ++e) t[e] = (T)q[kk][4 * r + e];
+          if constexpr (kRing) {
+            const float4* sl = sring + (warp * PF + k0) * 64 + lane;
+            const float4 v0 = sl[0], v1 = sl[32];
+            t[0] = dfloat(v0.x, v0.y);
+            t[1] = dfloat(v0.z, v0.w);
+            t[2] = dfloat(v1.x, v1.y);
+            t[3] = dfloat(v1.z, v1.w);
+          }
+          ALG::source(t, sg.v, neg, Sr);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const Blk<V, TW> m = *reinterpret_cast<const Blk<V, TW>*>(tab + ro + 4 + v * TW * VW);
-        if constexpr (kRegConst) {
+          for (int e = 0; e < 4; ++e) S[r][e] = V::all(Sr[e]);
+        }
+        if constexpr (!kRing) fetch(q[kk], 0);
 #pragma unroll
-          for (int r = 0; r < RPL; ++r) ALG::cell(S[r], X[r][v], Y[v], m.v, creg[v], acc[r], v == 0);
-        } else {
+        for (int v = 0; v < NV; ++v) {
+          using BlkM = Blk<V, TW>;
+          BlkM m;
+          if constexpr (GT) m = *reinterpret_cast<const BlkM*>(lin + ((size_t)min(v, ndir - 1) * R + ro) * TW);
+          else m = *reinterpret_cast<const BlkM*>(tab + ro + HD + v * TW * VW);
           V c[NC];
 #pragma unroll
-          for (int e = 0; e < NC; ++e) c[e] = *reinterpret_cast<const V*>(cst + (v * NC + e) * VW);
+          for (int e = 0; e < NC; ++e) {
+            if constexpr (kRegConst) c[e] = creg[v][e];
+            else c[e] = *reinterpret_cast<const V*>(cst + (v * NC + e) * VW);
+          }
 #pragma unroll
           for (int r = 0; r < RPL; ++r) ALG::cell(S[r], X[r][v], Y[v], m.v, c, acc[r], v == 0);
         }
-      }
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) {
-        T c4[4], o[4];
+        for (int r = 0; r < RPL; ++r) {
+          T c4[4], o[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) c4[e] = acc[r][e].sum();
-        ALG::from_basis(c4, o);
-        o[1] = sx > 0 ? o[1] : -o[1];
-        o[2] = sy > 0 ? o[2] : -o[2];
-        o[3] = sx * sy > 0 ? o[3] : -o[3];
-        if (act && (RPL == 1 || row + r < ny))
-          Vec4<T>::store(part + 4 * (long long)(cell + dx * col + r * dy), o[0], o[1], o[2], o[3]);
-      }
-      if (tail && act) {
+          for (int e = 0; e < 4; ++e) c4[e] = acc[r][e].sum();
+          ALG::from_basis(c4, o);
+          if constexpr (sizeof(T) == 4) {   // a select with a negated operand; in FP64 the negation would be an instruction
+            o[1] = sx > 0 ? o[1] : -o[1];
+            o[2] = sy > 0 ? o[2] : -o[2];
+            o[3] = sx * sy > 0 ? o[3] : -o[3];
+          } else {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          BlkY y;
-          y.v[0] = Y[v][0];
-          y.v[1] = Y[v][1];
-          *reinterpret_cast<BlkY*>(yout + (col & mout) * YC + v * 2 * VW) = y;
+            for (int e = 1; e < 4; ++e) o[e] = flip(o[e], neg[e]);
+          }
+          if (act && (RPL == 1 || row + r < ny))
+            Vec4<T>::store(part + 4 * (long long)(cell + dx * col + r * dy), o[0], o[1], o[2], o[3]);
         }
+        if (tail && act) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            BlkY y;
+            y.v[0] = Y[v][0];
+            y.v[1] = Y[v][1];
+            *reinterpret_cast<BlkY*>(yout + (col & mout) * YC + v * 2 * VW) = y;
+          }
+        }
+      }
+      // lanes without a cell hand on the vacuum inflow of the row they enter next (else the zero table sees to that)
+      if (GT && !act) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            Y[v][e] = V::all((T)0);
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) X[r][v][e] = V::all((T)0);
+          }
       }
       ++col;
       const bool wrap = col == P;
@@ -622,6 +649,7 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
     }
     group_sync(W);
   }
+  if constexpr (kRing) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // ------------------------------------------------------------------------------------------------- launch
@@ -635,53 +663,124 @@ static void mesh_max(const rte_problem* p, int* nx, int* ny) {
 
 constexpr size_t kMaxSmem = 227 * 1024;
 
-static size_t table_smem(const rte_problem* p, int prec, WaveShape s, int tw) {
+// Shared memory of a CTA.  tables: with the region tables, else with these left in global memory.
+static size_t shape_smem(const rte_problem* p, int prec, WaveShape s, bool tables) {
+  using F = Rot<float>;
+  using W = Legendre<double, true>;
   int nx, ny;
   mesh_max(p, &nx, &ny);
-  const int nc = prec == PREC_F32 ? Rot<float>::NC : Modal<double>::NC;
-  const int bytes = prec == PREC_F32 ? 4 : 8;
-  const size_t elems = (size_t)(p->R + 1) * table_stride(4 + s.D * tw, bytes) + ((s.D * nc + 3) & ~3) +
-                       ((size_t)nx + (s.W - 1) * kRing) * s.D * 2;
-  return elems * bytes;
+  const bool f32 = prec == PREC_F32;
+  const int nc = f32 ? F::NC : (prec == PREC_F64 ? W::NC : Scaled::NC);
+  const int rs = f32 ? table_stride(F::HD + s.D * F::TW, 4)
+                     : (prec == PREC_F64 ? table_stride(W::HD + s.D * W::TW, 8) : table_stride(s.D * Scaled::TW, 8));
+  const size_t elems = (tables ? (size_t)(p->R + 1) * rs : 0) + ((s.D * nc + 3) & ~3) +
+                       ((size_t)nx + (s.W - 1) * kRingCols) * s.D * 2;
+  return elems * (f32 ? 4 : 8) + (prec == PREC_DF ? (size_t)s.W * 4 * 1024 : 0);   // and the ring of sources
 }
 
-// FP64 tasks of one or two directions run in the Legendre basis while its tables (sixteen entries a direction and region)
-// fit: up to about 1,300 regions with one direction, 750 with two.  The eigenbasis's four take twice as many and more.
-static bool legendre(const rte_problem* p, int prec, WaveShape s) {
-  return prec == PREC_F64 && s.D <= 2 && table_smem(p, prec, s, Legendre<double>::TW) <= kMaxSmem;
+// FP64 and double-float tables (144 and 80 bytes a region with one direction) stay in global memory where shared memory
+// does not hold them: 1,600 and 2,800 regions and more with one direction, 430 and 670 with four.
+static bool global_tables(const rte_problem* p, int prec, WaveShape s) {
+  return prec != PREC_F32 && shape_smem(p, prec, s, true) > kMaxSmem;
 }
 
 size_t wave_smem(const rte_problem* p, int prec, WaveShape s) {
-  return table_smem(p, prec, s, prec == PREC_F32          ? Rot<float>::TW
-                                : legendre(p, prec, s) ? Legendre<double>::TW
-                                                       : Modal<double>::TW);
+  return shape_smem(p, prec, s, !global_tables(p, prec, s));
 }
 
-// Registers a thread of each built shape takes (0: not built): they set how many warps an SM holds.
-static int shape_regs(int prec, int D, int rpl) {
-  if (prec == PREC_F32) {
-    if (rpl == 2) return D == 8 ? 208 : 0;
-    switch (D) {
-      case 1: return 96;
-      case 2: return 112;
-      case 4: case 8: return 128;
-      case 12: return 200;
-      case 16: return 224;
+template <typename T_, typename TI, typename ALG, int VW, int NV, int RPL, int PF, bool BC, int MINB, bool GT>
+struct WaveKernel {
+  static constexpr auto fn = k_wave<T_, TI, ALG, VW, NV, RPL, PF, BC, MINB, GT>;
+  static int launch(const SweepArgs& a, int W, size_t smem, cudaStream_t st) {
+    static std::atomic<size_t> granted[kMaxDevices];
+    RTE_TRY(grant_smem(fn, smem, granted));
+    fn<<<a.ntasks, W * 32, smem, st>>>(a);
+    count_launch();
+    RTE_CHECK_CUDA(cudaGetLastError());
+    return RTE_OK;
+  }
+  static int regs() {   // a thread's registers, a property of the compiled kernel
+    static std::atomic<int> n{0};
+    if (n.load() == 0) {
+      cudaFuncAttributes at;
+      if (cudaFuncGetAttributes(&at, fn) != cudaSuccess) {
+        cudaGetLastError();
+        return 128;
+      }
+      n.store((at.numRegs + 7) & ~7);
     }
-    return 0;
+    return n.load();
   }
-  if (rpl != 1) return 0;
-  switch (D) {
-    case 1: case 2: return 112;
-    case 3: return prec == PREC_F64 ? 128 : 0;
-    case 4: return 136;
-    case 8: return prec == PREC_F64 ? 168 : 0;
+};
+
+// The kernel of a shape: f(WaveKernel<...>{}), or `none` where it is not built.  FP32 sweeps of FP64 vectors are the
+// right-hand side and the inner solves with FP64 Krylov vectors.  sig: an FP64 source that is still to be multiplied by
+// Sigma_s.
+template <bool BC, typename F>
+static int with_kernel(int prec, WaveShape s, bool in64, bool sig, bool gt, int none, F&& f) {
+  const int shape = s.D * 10 + s.rpl;
+  if (prec == PREC_F32) {
+    using A = Rot<float>;
+    if (BC || in64) {
+      switch (shape) {
+        case 11: return f(WaveKernel<float, double, A, 1, 1, 1, 8, true, 2, false>{});
+        case 21: return f(WaveKernel<float, double, A, 2, 1, 1, 8, true, 2, false>{});
+        case 41: return f(WaveKernel<float, double, A, 2, 2, 1, 8, true, 2, false>{});
+        case 81: return f(WaveKernel<float, double, A, 2, 4, 1, 4, true, 2, false>{});
+        case 121: return f(WaveKernel<float, double, A, 2, 6, 1, 4, true, 1, false>{});
+        case 161: return f(WaveKernel<float, double, A, 2, 8, 1, 4, true, 1, false>{});
+        case 82: return f(WaveKernel<float, double, A, 2, 4, 2, 4, true, 1, false>{});
+      }
+    } else {
+      switch (shape) {
+        case 11: return f(WaveKernel<float, float, A, 1, 1, 1, 8, false, 2, false>{});
+        case 21: return f(WaveKernel<float, float, A, 2, 1, 1, 8, false, 2, false>{});
+        case 41: return f(WaveKernel<float, float, A, 2, 2, 1, 8, false, 2, false>{});
+        case 81: return f(WaveKernel<float, float, A, 2, 4, 1, 4, false, 2, false>{});
+        case 121: return f(WaveKernel<float, float, A, 2, 6, 1, 4, false, 1, false>{});
+        case 161: return f(WaveKernel<float, float, A, 2, 8, 1, 4, false, 1, false>{});
+        case 82: return f(WaveKernel<float, float, A, 2, 4, 2, 4, false, 1, false>{});
+      }
+    }
+  } else if (prec == PREC_F64) {
+    auto pick = [&](auto alg) {
+      using A = decltype(alg);
+      switch (shape * 2 + gt) {
+        case 22: return f(WaveKernel<double, double, A, 1, 1, 1, 4, BC, 2, false>{});
+        case 42: return f(WaveKernel<double, double, A, 1, 2, 1, 4, BC, 2, false>{});
+        case 62: return f(WaveKernel<double, double, A, 1, 3, 1, 4, BC, 2, false>{});
+        case 82: return f(WaveKernel<double, double, A, 1, 4, 1, 4, BC, 1, false>{});
+        case 23: return f(WaveKernel<double, double, A, 1, 1, 1, 4, BC, 1, true>{});
+        case 43: return f(WaveKernel<double, double, A, 1, 2, 1, 4, BC, 1, true>{});
+        case 83: return f(WaveKernel<double, double, A, 1, 4, 1, 4, BC, 1, true>{});
+      }
+      return none;
+    };
+    if constexpr (BC) return pick(Legendre<double, false>{});
+    else return sig ? pick(Legendre<double, true>{}) : pick(Legendre<double, false>{});
+  } else if (!BC) {
+    using A = Scaled;
+    switch (shape * 2 + gt) {
+      case 22: return f(WaveKernel<dfloat, dfloat, A, 1, 1, 1, 4, false, 2, false>{});
+      case 42: return f(WaveKernel<dfloat, dfloat, A, 1, 2, 1, 4, false, 2, false>{});
+      case 82: return f(WaveKernel<dfloat, dfloat, A, 1, 4, 1, 4, false, 1, false>{});
+      case 23: return f(WaveKernel<dfloat, dfloat, A, 1, 1, 1, 4, false, 1, true>{});
+    }
   }
-  return 0;
+  return none;
+}
+
+// Registers a thread of a shape takes (0: not built): they set how many warps an SM holds.
+static int shape_regs(const rte_problem* p, int prec, WaveShape s) {
+  return with_kernel<false>(prec, s, false, false, global_tables(p, prec, s), 0, [](auto k) { return decltype(k)::regs(); });
+}
+
+static bool shape_built(const rte_problem* p, int prec, WaveShape s) {
+  return with_kernel<false>(prec, s, false, false, global_tables(p, prec, s), 0, [](auto) { return 1; }) != 0;
 }
 
 bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
-  if (s.W < 1 || s.W > 8 || shape_regs(prec, s.D, s.rpl) == 0 || wave_smem(p, prec, s) > kMaxSmem) return false;
+  if (s.W < 1 || s.W > 8 || !shape_built(p, prec, s) || wave_smem(p, prec, s) > kMaxSmem) return false;
   if (s.rpl == 2)   // the two rows of a lane share a table: they have to lie in one region in both sweep directions
     for (int b = 0; b < p->B; ++b)
       if (p->ny[b] % 2 || (p->ny[b] / p->ry) % 2) return false;
@@ -697,7 +796,7 @@ bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
 // the Legendre basis; 5 % more a direction above 4), 70 alone; double-float 320 D + 264 instructions, 0.85 a cycle and SM quarter, 0.7 alone.  The partial fluxes, written and read once, are
 // added at the copy bandwidth.
 static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, const std::vector<int>& order) {
-  const int SK = 4, per_sm = 65536 / (shape_regs(prec, s.D, s.rpl) * 32);
+  const int SK = 4, per_sm = 65536 / (shape_regs(p, prec, s) * 32);
   const size_t smem = wave_smem(p, prec, s) + 1024;
   const size_t slots = std::max(1, std::min(per_sm / s.W, (int)(kMaxSmem / smem)));
   int chunks = 0;
@@ -707,12 +806,12 @@ static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, co
     pipe = (s.rpl == 2 ? 13.0 * s.D + 30.0 : 10.0 * s.D + 40.0) / (s.W == 1 ? 0.65 : 0.75);
     alone = s.rpl == 2 ? 1750.0 : 50.0 * s.D + 300.0;
   } else if (prec == PREC_F64) {
-    const double instr = legendre(p, prec, s) ? 32.0 * s.D + 4.0 : 24.0 * s.D + 30.0;
-    pipe = 19.0 * (1.0 + 0.05 * std::max(0, s.D - 4)) * instr;
+    const double instr = 32.0 * s.D;
+    pipe = 19.0 * instr;
     alone = 70.0 * instr;
   } else {
-    pipe = (320.0 * s.D + 264.0) / 3.4;   // of warps in multiples of four
-    alone = (320.0 * s.D + 264.0) / 0.7;
+    pipe = (356.0 * s.D + 160.0) / 3.4;   // of warps in multiples of four
+    alone = (356.0 * s.D + 160.0) / 0.5;
   }
   struct Run {
     double steps;
@@ -722,7 +821,8 @@ static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, co
   for (long long i = 0; i < (long long)p->B * chunks; i += sms) {
     const int b = order[i / chunks];
     const int nb = (p->ny[b] + 32 * s.rpl - 1) / (32 * s.rpl), W = std::min(s.W, nb), last = (nb - 1) / W;
-    queue.push_back({(double)last * wave_period(p->nx[b], W, SK) + (nb - 1 - last * W) * (32 + SK) + 31 + p->nx[b], W});
+    queue.push_back({(double)last * wave_period(p->nx[b], W, SK) + (nb - 1 - last * W) * (32 + SK) +
+                         31 + p->nx[b], W});
   }
   double t = 0.0;
   for (size_t next = 0; next < queue.size() || !held.empty();) {
@@ -795,80 +895,18 @@ WaveShape wave_shape_for(const rte_problem* p, int prec, int D) {
   return best;
 }
 
-template <typename T, typename TI, typename ALG, int VW, int NV, int RPL, int PF, bool BC, int MINB>
-static int launch_one(const SweepArgs& a, int W, size_t smem, cudaStream_t st) {
-  auto kern = k_wave<T, TI, ALG, VW, NV, RPL, PF, BC, MINB>;
-  static std::atomic<size_t> granted[kMaxDevices];
-  RTE_TRY(grant_smem(kern, smem, granted));
-  kern<<<a.ntasks, W * 32, smem, st>>>(a);
-  count_launch();
-  RTE_CHECK_CUDA(cudaGetLastError());
-  return RTE_OK;
-}
-
-// FP32 sweeps of FP64 vectors: the right-hand side, and the inner solves with FP64 Krylov vectors
-template <typename TI>
-static int launch_f32(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t st) {
-  using A = Rot<float>;
-  constexpr bool BC = std::is_same<TI, double>::value;
-  switch (s.D * 10 + s.rpl) {
-    case 11: return launch_one<float, TI, A, 1, 1, 1, 8, BC, 2>(a, s.W, smem, st);
-    case 21: return launch_one<float, TI, A, 2, 1, 1, 8, BC, 2>(a, s.W, smem, st);
-    case 41: return launch_one<float, TI, A, 2, 2, 1, 8, BC, 2>(a, s.W, smem, st);
-    case 81: return launch_one<float, TI, A, 2, 4, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 121: return launch_one<float, TI, A, 2, 6, 1, 4, BC, 1>(a, s.W, smem, st);
-    case 161: return launch_one<float, TI, A, 2, 8, 1, 4, BC, 1>(a, s.W, smem, st);
-    case 82: return launch_one<float, TI, A, 2, 4, 2, 4, BC, 1>(a, s.W, smem, st);
-  }
-  set_error("sweep: unsupported directions per task");
-  return RTE_ERR_UNSUPPORTED;
-}
-
-template <bool BC>
-static int launch_f64(const SweepArgs& a, WaveShape s, bool leg, size_t smem, cudaStream_t st) {
-  using A = Modal<double>;
-  using Leg = Legendre<double>;
-  switch (s.D) {
-    case 1:
-      return leg ? launch_one<double, double, Leg, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st)
-                 : launch_one<double, double, A, 1, 1, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 2:
-      return leg ? launch_one<double, double, Leg, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st)
-                 : launch_one<double, double, A, 1, 2, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 3: return launch_one<double, double, A, 1, 3, 1, 4, BC, 2>(a, s.W, smem, st);
-    case 4: return launch_one<double, double, A, 1, 4, 1, 4, BC, 1>(a, s.W, smem, st);
-    case 8: return launch_one<double, double, A, 1, 8, 1, 4, BC, 1>(a, s.W, smem, st);
-  }
-  set_error("sweep: unsupported directions per task");
-  return RTE_ERR_UNSUPPORTED;
-}
-
-static int launch_df(const SweepArgs& a, WaveShape s, size_t smem, cudaStream_t st) {
-  using A = Modal<dfloat>;
-  switch (s.D) {
-    case 1: return launch_one<dfloat, dfloat, A, 1, 1, 1, 4, false, 2>(a, s.W, smem, st);
-    case 2: return launch_one<dfloat, dfloat, A, 1, 2, 1, 4, false, 2>(a, s.W, smem, st);
-    case 4: return launch_one<dfloat, dfloat, A, 1, 4, 1, 4, false, 1>(a, s.W, smem, st);
-  }
-  set_error("sweep: unsupported directions per task");
-  return RTE_ERR_UNSUPPORTED;
-}
-
 int launch_wave(const rte_problem* p, int prec, WaveShape s, bool in64, const SweepArgs& args, cudaStream_t st) {
-  SweepArgs a = args;
-  if (prec == PREC_F32) a.linv = p->d_rot32.p;
-  else if (prec == PREC_DF) a.linv = p->d_modal_df.p;
-  const bool leg = legendre(p, prec, s);
-  if (prec == PREC_F64) a.linv = leg ? p->d_linv64.p : p->d_modal64.p;
   if (!wave_shape_ok(p, prec, s)) {
     set_error("sweep: shared-memory table too large for this mesh/region count");
     return RTE_ERR_UNSUPPORTED;
   }
+  SweepArgs a = args;
+  if (prec == PREC_F32) a.linv = p->d_rot32.p;   // else the cell inverses of the arithmetic
   const size_t smem = wave_smem(p, prec, s);
-  if (prec == PREC_F64)
-    return a.with_bc ? launch_f64<true>(a, s, leg, smem, st) : launch_f64<false>(a, s, leg, smem, st);
-  if (prec == PREC_DF) return launch_df(a, s, smem, st);
-  return in64 ? launch_f32<double>(a, s, smem, st) : launch_f32<float>(a, s, smem, st);
+  auto run = [&](auto k) { return decltype(k)::launch(a, s.W, smem, st); };
+  const bool gt = global_tables(p, prec, s);
+  return a.with_bc ? with_kernel<true>(prec, s, in64, false, gt, RTE_ERR_UNSUPPORTED, run)
+                   : with_kernel<false>(prec, s, in64, a.sig_s != nullptr, gt, RTE_ERR_UNSUPPORTED, run);
 }
 
 }  // namespace rte
