@@ -461,7 +461,8 @@ __global__ void __launch_bounds__(256, MINB) k_wave(SweepArgs a) {
   const int cx = nx / a.rx, cy = ny / a.ry, dx = sx > 0 ? 1 : -1;
   const int P = wave_period(nx, W, SK);
   const int last = (nb - 1) / W;
-  const int nsteps = last * P + (nb - 1 - last * W) * (32 + SK) + 31 + nx;
+  // up to the last column of the mesh's last row: the last band of 40 rows has 8 lanes at work, not 32
+  const int nsteps = last * P + (nb - 1 - last * W) * (32 + SK) + (ny - 1 - 32 * RPL * (nb - 1)) / RPL + nx;
   const unsigned mx = 0xffffffffu / (unsigned)cx + 1u, my = 0xffffffffu / (unsigned)cy + 1u;   // i / c = mulhi(i, m); c = 1: see div
   auto div = [](int i, unsigned m) { return m ? (int)__umulhi((unsigned)i, m) : i; };
   constexpr int RI = GT ? 1 : RS;   // table index per region
@@ -822,7 +823,7 @@ static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, co
     const int b = order[i / chunks];
     const int nb = (p->ny[b] + 32 * s.rpl - 1) / (32 * s.rpl), W = std::min(s.W, nb), last = (nb - 1) / W;
     queue.push_back({(double)last * wave_period(p->nx[b], W, SK) + (nb - 1 - last * W) * (32 + SK) +
-                         31 + p->nx[b], W});
+                         (p->ny[b] - 1 - 32 * s.rpl * (nb - 1)) / s.rpl + p->nx[b], W});
   }
   double t = 0.0;
   for (size_t next = 0; next < queue.size() || !held.empty();) {
