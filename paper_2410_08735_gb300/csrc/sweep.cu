@@ -569,7 +569,43 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
   }
 }
 
-// 1D slab (P1, 2 dofs per cell): one warp per (instance, direction).  A cell maps the trace it gets to the one it passes
+// 1D slab (P1, 2 dofs per cell): one thread per (instance, direction) marches its chain.  The fewest operations, at the
+// latency of nx dependent cells: for batches with chains enough to hide it (see slab_march).
+template <typename T, typename TI, bool ANG>
+__global__ void __launch_bounds__(128) k_march1d(SweepArgs a) {
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= a.ntasks) return;
+  const SweepTask tk = a.tasks[tid];
+  if (a.active && !a.active[tk.b]) return;
+  const InstInfo in = a.inst[tk.b];
+  const UDir u = a.udir[tk.u0];
+  const int nx = in.nx, R = a.R, cx = nx / a.rx;
+  const T al = (T)(u.ax / in.hx), wg = (T)u.w;
+  const T S3 = (T)1.7320508075688772;
+  const T* linv = reinterpret_cast<const T*>(a.linv) + ((size_t)tk.b * a.nu + tk.u0) * R * 4;
+  const T* sig_s = a.sig_s ? reinterpret_cast<const T*>(a.sig_s) + (size_t)tk.b * R : nullptr;
+  const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
+  T* out = ANG ? reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off +
+                     (size_t)(a.psi_unique ? tk.u0 : u.dup[0]) * in.ndof
+               : reinterpret_cast<T*>(a.partial) + (size_t)a.tasks_per_inst * in.off + (size_t)tk.t * in.ndof;
+  T tx = a.with_bc && (a.inflow_mask & (u.sx > 0 ? 1 : 2)) ? (T)(in.g * sqrt(in.hx)) : (T)0;
+  for (int col = 0; col < nx; ++col) {
+    const int ix = u.sx > 0 ? col : nx - 1 - col;
+    const int reg = ix / cx;
+    T s0 = (T)src[2 * ix], s1 = (T)src[2 * ix + 1];
+    if (sig_s) { s0 *= sig_s[reg]; s1 *= sig_s[reg]; }
+    s1 = u.sx > 0 ? s1 : -s1;
+    const T r0 = s0 + al * tx, r1 = s1 - S3 * al * tx;
+    const T* L = linv + reg * 4;
+    const T p0 = L[0] * r0 + L[1] * r1, p1 = L[2] * r0 + L[3] * r1;
+    tx = p0 + S3 * p1;
+    const T q1 = u.sx > 0 ? p1 : -p1;
+    out[2 * ix] = ANG ? p0 : wg * p0;
+    out[2 * ix + 1] = ANG ? q1 : wg * q1;
+  }
+}
+
+// The same for few chains: one warp per (instance, direction).  A cell maps the trace it gets to the one it passes
 // on, t' = a t + c with a = alpha e^T L^{-1} phat (the cell alone) and c = e^T L^{-1} s (its source), e = (1, sqrt3); affine
 // maps compose, so a chain of cells is a prefix product.  Each lane composes the maps of nx / 32 consecutive cells, a
 // scan over the warp gives every lane the trace that enters its cells, and a second pass over them stores the fluxes.
@@ -844,11 +880,38 @@ static int ensure_tasks(rte_problem* p, int D) {
   return RTE_OK;
 }
 
+// Slabs: whether one thread marches a chain (k_march1d) or a warp scans it (k_sweep1d), from the time each form takes, in
+// microseconds (measured with 1 to 16384 slabs of 16 to 1024 cells, 4 to 32 directions).  Marching: the latency of the
+// longest chain, or a rate per cell once the chains fill the GPU.  Scanning: a rate per chain that grows with the cells a
+// lane takes, in FP64 with its instructions, else steeply where the cells of the resident warps no longer fit the L1.
+// The forms cross at about 12,000 chains in FP64 (128 cells, 16 directions, FP64 apply, marching and scanning: 64 slabs 94
+// and 19 us, 512 slabs 99 and 72, 1024 slabs 101 and 128, 8192 slabs 510 and 969), in FP32 with 512 cells and more (1024
+// slabs, 32 directions: 269 and 438; with 128 cells scanning is faster throughout).
+static bool slab_march(rte_problem* p, int prec, bool ang) {
+  signed char& form = p->slab_form[prec][ang ? 1 : 0];
+  if (form < 0) {
+    const double lat = prec == PREC_F32 ? 0.285 : (prec == PREC_DF ? 0.70 : (ang ? 0.50 : 0.69));
+    const double rate = 1e-6 * (prec == PREC_F32 ? 15.5 : (prec == PREC_DF ? 38.0 : (ang ? 24.0 : 30.0)));
+    double longest = 0.0, cells = 0.0, scan = 0.0;
+    for (int b = 0; b < p->B; ++b) {
+      const int per = (p->nx[b] + 31) / 32;   // cells a lane
+      longest = std::max(longest, (double)p->nx[b]);
+      cells += (double)p->nx[b];
+      if (prec == PREC_F64) scan += ang ? 1.1 + 1.07 * per : 1.35 + 1.55 * per;
+      else if (prec == PREC_F32) scan += per < 4 ? 0.65 : (per < 8 ? 0.25 : (per < 16 ? 0.45 : 0.85)) * per;
+      else scan += per < 4 ? 1.0 + 0.3 * per : (per < 8 ? 1.0 : 1.65) * per;
+    }
+    form = std::max(longest * lat, cells * p->nu * rate) < 1e-3 * scan * p->nu;
+  }
+  return form != 0;
+}
+
 // Angular sweeps, sweeps with cross-section profiles, and the slab: D divides every quadrant's direction count.
 template <typename T, typename TI, bool ANG>
 static int launch_sweep_t(rte_problem* p, int D, SweepArgs& a, cudaStream_t st) {
   if (p->dim == 1) {
-    k_sweep1d<T, TI, ANG><<<(a.ntasks + 3) / 4, 128, 0, st>>>(a);
+    if (slab_march(p, prec_of<T>(), ANG)) k_march1d<T, TI, ANG><<<(a.ntasks + 127) / 128, 128, 0, st>>>(a);
+    else k_sweep1d<T, TI, ANG><<<(a.ntasks + 3) / 4, 128, 0, st>>>(a);
     count_launch();
     RTE_CHECK_CUDA(cudaGetLastError());
     return RTE_OK;
