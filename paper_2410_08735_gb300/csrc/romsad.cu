@@ -557,7 +557,7 @@ __global__ void k_lift_masked(const TP* W, int rmax, int r, const InstInfo* inst
   }
 }
 
-int RomPlan::build(romsad* rom_, rte_problem* p, const std::vector<int>& ids_, cudaStream_t st) {
+int RomPlan::build(romsad* rom_, rte_problem* p, const std::vector<int>& ids_, cudaStream_t st, bool partials) {
   rom = rom_;
   ids = ids_;
   const int n = (int)ids.size();
@@ -568,8 +568,10 @@ int RomPlan::build(romsad* rom_, rte_problem* p, const std::vector<int>& ids_, c
   RTE_TRY(piv.ensure((size_t)n * 64));
   chunk = 256;
   nchunk = (rom->N + chunk - 1) / chunk;
-  RTE_TRY(part.ensure((size_t)n * nchunk * 64));
-  RTE_TRY(c.ensure((size_t)n * 64));
+  if (partials) {
+    RTE_TRY(part.ensure((size_t)n * nchunk * 64));
+    RTE_TRY(c.ensure((size_t)n * 64));
+  }
   size_t smem = (size_t)2 * rom->r * rom->r * 8;   // 64 KiB at the largest rank (64)
   // the attribute is per device: set on the current one at every plan build (once per solve, not on the hot path)
   if (smem > 48 * 1024)
@@ -793,19 +795,20 @@ int romsad_apply(romsad_t rom, rte_problem_t p, int dtype, const void* v, void* 
   cudaStream_t st = (cudaStream_t)stream;
   std::vector<int> ids(p->B);
   for (int b = 0; b < p->B; ++b) ids[b] = b;
-  RomPlan plan;
-  RTE_TRY(plan.build(rom, p, ids, st));
+  if (dtype == RTE_F32 && p->cellsig) {
+    set_error("romsad_apply: FP32 vectors run the tensor-core products, not available with cross-section profiles");
+    return RTE_ERR_UNSUPPORTED;
+  }
+  std::unique_ptr<RomPlan> plan = rom->pool.take();
+  RTE_TRY(plan->build(rom, p, ids, st, dtype == RTE_F64));
   if (dtype == RTE_F32) {
-    if (p->cellsig) {
-      set_error("romsad_apply: FP32 vectors run the tensor-core products, not available with cross-section profiles");
-      return RTE_ERR_UNSUPPORTED;
-    }
-    RTE_TRY(rom_tc_plan_setup(plan, st));
-    RTE_TRY(rom_tc_apply(plan, p, nullptr, (const float*)v, (float*)z, st));
+    RTE_TRY(rom_tc_plan_setup(*plan, st));
+    RTE_TRY(rom_tc_apply(*plan, p, nullptr, (const float*)v, (float*)z, st));
   } else {
-    RTE_TRY(plan.apply(p, nullptr, (const double*)v, (double*)z, true, st));
+    RTE_TRY(plan->apply(p, nullptr, (const double*)v, (double*)z, true, st));
   }
   RTE_CHECK_CUDA(cudaStreamSynchronize(st));
+  rom->pool.give(std::move(plan));
   return RTE_OK;
 }
 

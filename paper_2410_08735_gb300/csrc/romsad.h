@@ -1,10 +1,53 @@
 // ROMSAD data structures shared by romsad.cu, greedy.cu and krylov.cu.
 #pragma once
 #include <cstdint>
+#include <memory>
+#include <mutex>
 
 #include "internal.h"
 
 struct rte_mlp;
+struct romsad;
+
+namespace rte {
+// ROMSAD application plan for one ROM and the instances that use it, built once per solve: the
+// reduced operators U^T A_mu U are assembled and LU-factored at build; apply() then costs one
+// projection (multi-block partial sums), two triangular solves and one lift.
+struct RomPlan {
+  romsad* rom = nullptr;
+  std::vector<int> ids;
+  DevBuf<int> d_ids, piv;
+  DevBuf<double> lu, part, c;
+  DevBuf<float> inv32;   // FP32 copy of lu (the inverses), filled by the FGMRES driver
+  DevBuf<double> WT;     // W transposed [r][N] (coalesced lift), filled by the FGMRES driver
+  DevBuf<float> WT32;
+  DevBuf<float> part32, c32;   // tensor-core path: projection partials [nchunk][n][64], coefficients [n][64]
+  int chunk = 1024, nchunk = 0;
+  // partials: with the buffers of apply() (the tensor-core path has its own)
+  int build(romsad* rom, rte_problem* p, const std::vector<int>& ids, cudaStream_t st, bool partials = true);
+  int apply(rte_problem* p, const int* d_active, const double* v, double* z, bool f64, cudaStream_t st);
+};
+
+// Plans whose buffers romsad_apply hands from one call to the next: eight cudaMalloc and cudaFree a call took longer than
+// its kernels, and a time that depended on what else was allocated.  A call owns the plan it took until its stream has been
+// waited for, so calls on several threads and streams have plans of their own; at most kKeep are kept.
+struct RomPlanPool {
+  static constexpr size_t kKeep = 4;
+  std::mutex m;
+  std::vector<std::unique_ptr<RomPlan>> free_plans;
+  std::unique_ptr<RomPlan> take() {
+    std::lock_guard<std::mutex> lock(m);
+    if (free_plans.empty()) return std::make_unique<RomPlan>();
+    std::unique_ptr<RomPlan> pl = std::move(free_plans.back());
+    free_plans.pop_back();
+    return pl;
+  }
+  void give(std::unique_ptr<RomPlan> pl) {
+    std::lock_guard<std::mutex> lock(m);
+    if (free_plans.size() < kKeep) free_plans.push_back(std::move(pl));
+  }
+};
+}  // namespace rte
 
 struct romsad {
   // mesh the ROM belongs to (must match every instance it is applied to)
@@ -37,6 +80,7 @@ struct romsad {
   int sigma_modes = 0;
   rte::DevBuf<double> F;            // [ncell][16]
   int bf16_rank = 0;                // rank the BF16 copies were made at (0: none)
+  rte::RomPlanPool pool;            // romsad_apply
 };
 
 namespace rte {
@@ -58,22 +102,6 @@ int rom_alloc_arrays(romsad* rom, int rmax, bool withU);
 // y[b][k] = (P^T Sigma_s v_b)[k] for the listed instances (FP64), y laid out [ninst][64]
 int rom_project_list(romsad* rom, rte_problem* p, const int* d_list, int ninst, const double* v, double* y,
                      cudaStream_t st);
-// ROMSAD application plan for one ROM and the instances that use it, built once per solve: the
-// reduced operators U^T A_mu U are assembled and LU-factored at build; apply() then costs one
-// projection (multi-block partial sums), two triangular solves and one lift.
-struct RomPlan {
-  romsad* rom = nullptr;
-  std::vector<int> ids;
-  DevBuf<int> d_ids, piv;
-  DevBuf<double> lu, part, c;
-  DevBuf<float> inv32;   // FP32 copy of lu (the inverses), filled by the FGMRES driver
-  DevBuf<double> WT;     // W transposed [r][N] (coalesced lift), filled by the FGMRES driver
-  DevBuf<float> WT32;
-  DevBuf<float> part32, c32;   // tensor-core path: projection partials [nchunk][n][64], coefficients [n][64]
-  int chunk = 1024, nchunk = 0;
-  int build(romsad* rom, rte_problem* p, const std::vector<int>& ids, cudaStream_t st);
-  int apply(rte_problem* p, const int* d_active, const double* v, double* z, bool f64, cudaStream_t st);
-};
 // Assemble and LU-factor U^T A_mu U for the listed instances of p (device), then
 // c = A_r^{-1} y per instance: y [ninst][r] in, c [ninst][r] out (FP64).
 int rom_small_solve(romsad* rom, rte_problem* p, const int* d_list, int ninst, const double* y, double* c,
