@@ -1086,9 +1086,11 @@ static WaveShape op_shape(rte_problem* p, int prec) {
   if (p->force_shape.D > 0) return p->force_shape;
   if (p->pin_var >= 0) {
     const int nb = std::min(max_bands(p), 8);
-    const WaveShape s{p->pin_D, p->pin_var == 0 ? nb : (p->pin_var == 1 ? 1 : std::min(nb, 2)), 1};
-    if (wave_shape_ok(p, prec, s) || prec == PREC_F32) return s;
-    return WaveShape{4, s.W, 1};   // the wider types take at most 4 directions a task
+    WaveShape s{p->pin_D, p->pin_var == 0 ? nb : (p->pin_var == 1 ? 1 : std::min(nb, 2)), 1};
+    // the wider types take at most 4 directions a task, and fewer on meshes too wide for the traces of so many
+    if (prec != PREC_F32)
+      while (s.D > 1 && !wave_shape_ok(p, prec, s)) s.D /= 2;
+    return s;
   }
   if (p->tuned_shape[prec].D > 0) return p->tuned_shape[prec];
   if (p->rule_shape[prec].D == 0) {
