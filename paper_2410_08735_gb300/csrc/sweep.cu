@@ -1373,7 +1373,13 @@ int launch_op_external(rte_problem* p, bool f64, const void* z, void* w, const S
   a.sig_s = sigma_s_arg(p, f64);
   a.partial = partial;
   const int prec = f64 ? PREC_F64 : PREC_F32;
-  RTE_TRY(launch_op_sweep(p, prec, p->dim == 2 ? wave_shape_for(p, prec, D) : WaveShape{1, 1, 1}, f64, a, st));
+  WaveShape shape{1, 1, 1};
+  if (p->dim == 2) {   // ranked once per problem and D: the estimate walks all instances
+    WaveShape& kept = p->ext_shape[prec][D];
+    if (kept.D == 0) kept = p->tuned_shape[prec].D == D ? p->tuned_shape[prec] : wave_shape_for(p, prec, D);
+    shape = kept;
+  }
+  RTE_TRY(launch_op_sweep(p, prec, shape, f64, a, st));
   int maxn = 0;
   for (int b = 0; b < p->B; ++b) maxn = std::max(maxn, (int)(p->off[b + 1] - p->off[b]));
   dim3 grid((maxn + 255) / 256, p->B);
