@@ -166,6 +166,12 @@ int rte_rhs(rte_problem_t p, int dtype, void* btilde, void* stream);
  * need meshes of at most 256 rows (RTE_ERR_INVALID_ARG otherwise).  Call it before the first solve on p: the task lists
  * and buffers of captured iteration graphs are sized then. */
 int rte_problem_set_sweep_variant(rte_problem_t p, int variant, int directions_per_warp, int tasks_per_run);
+/* Pin the launch shape of the operator applies of p in one arithmetic (no paper counterpart: a testing and tuning aid;
+ * 2D, cross sections per region): dtype RTE_F32, RTE_F64 or RTE_F64_DF, up to `directions` per task, `warps` per task
+ * (1 to 8), mesh rows per lane (1 or 2).  directions = 0 returns to the automatic choice.  A shape that is not built, or
+ * that does not fit the problem, is refused with RTE_ERR_UNSUPPORTED.  Takes precedence over a pinned variant; call it
+ * before the first solve on p. */
+int rte_problem_set_sweep_shape(rte_problem_t p, int dtype, int directions, int warps, int rows_per_lane);
 /* Allocation-free form of rte_apply_op (the paper has no counterpart; this is a deployment aid).
  * Computes the same w = z - T (Sigma_s z), but allocates no device memory: no cudaMalloc, cudaFree or
  * allocating library routine is called.  It is meant for callers that cannot allocate, for example a

@@ -160,6 +160,7 @@ _SIGS = {
     "rte_rbf_destroy": (ctypes.c_int, [ctypes.c_void_p]),
     "rte_problem_set_inflow": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)]),
     "rte_problem_set_sweep_variant": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
+    "rte_problem_set_sweep_shape": (ctypes.c_int, [ctypes.c_void_p] + 4 * [ctypes.c_int]),
     "romsad_galerkin_coefficients": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)]),
 }
 
@@ -293,9 +294,15 @@ class Problem:
         _check(load().rte_problem_set_params(self.h, _dptr(ss), _dptr(sa)), "rte_problem_set_params")
 
     def set_sweep_variant(self, variant: int, directions_per_warp: int = 1, tasks_per_run: int = 0):
-        """Pin the sweep kernel (0 band, 1 warp per task, 2 pipelined band; -1: autotuner)."""
+        """Pin the sweep kernel (0 band, 1 warp per task, 2 two warps per task; -1: autotuner)."""
         _check(load().rte_problem_set_sweep_variant(self.h, variant, directions_per_warp, tasks_per_run),
                "rte_problem_set_sweep_variant")
+
+    def set_sweep_shape(self, dtype: int, directions: int, warps: int = 1, rows_per_lane: int = 1):
+        """Pin the launch shape of the operator applies in one arithmetic (RTE_F32, RTE_F64, RTE_F64_DF); 0 directions:
+        automatic."""
+        _check(load().rte_problem_set_sweep_shape(self.h, dtype, directions, warps, rows_per_lane),
+               "rte_problem_set_sweep_shape")
 
     def set_inflow(self, g):
         """Per-instance inflow values on the problem's inflow faces: [B]."""

@@ -165,6 +165,7 @@ struct rte_problem {
   rte::WaveShape tuned_shape[3], rule_shape[3], force_shape;   // rule: the cost estimate's choice, made once
   rte::WaveShape ext_shape[2][17];            // the same for the allocation-free apply, per directions a task
   signed char slab_form[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};   // slabs: 1 march, 0 scan, chosen once (slab_march)
+  rte::WaveShape pin_shape[3];                // rte_problem_set_sweep_shape
   int pin_D = 0, pin_var = -1;                // rte_problem_set_sweep_variant (a user's pin; overrides the tuning)
   int ntasks = 0, tasks_per_inst = 0;
   rte::DevBuf<int> d_active;                  // [B] instance mask (1 = active), all 1 by default

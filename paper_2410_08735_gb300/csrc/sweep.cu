@@ -1084,6 +1084,7 @@ static int max_bands(const rte_problem* p) {
 static WaveShape op_shape(rte_problem* p, int prec) {
   if (p->dim == 1 || p->cellsig) return WaveShape{pick_D(p, prec), 1, 1};
   if (p->force_shape.D > 0) return p->force_shape;
+  if (p->pin_shape[prec].D > 0) return p->pin_shape[prec];
   if (p->pin_var >= 0) {
     const int nb = std::min(max_bands(p), 8);
     WaveShape s{p->pin_D, p->pin_var == 0 ? nb : (p->pin_var == 1 ? 1 : std::min(nb, 2)), 1};
@@ -1476,7 +1477,7 @@ int rte_problem_set_sweep_variant(rte_problem_t p, int variant, int directions_p
     p->pin_D = 0;
     return RTE_OK;
   }
-  RTE_ARG(variant <= 2, "variant must be -1, 0 (band), 1 (warp per task) or 2 (pipelined band)");
+  RTE_ARG(variant <= 2, "variant must be -1, 0 (band), 1 (warp per task) or 2 (two warps per task)");
   const int D = directions_per_warp;
   RTE_ARG(D == 1 || D == 2 || D == 4 || D == 8, "directions per warp must be 1, 2, 4 or 8");
   if (p->dim == 2) {
@@ -1487,6 +1488,24 @@ int rte_problem_set_sweep_variant(rte_problem_t p, int variant, int directions_p
   }
   p->pin_var = variant;
   p->pin_D = D;
+  return RTE_OK;
+}
+
+int rte_problem_set_sweep_shape(rte_problem_t p, int dtype, int directions, int warps, int rows_per_lane) {
+  RTE_ARG(p, "null handle");
+  RTE_ARG(dtype == RTE_F32 || dtype == RTE_F64 || dtype == RTE_F64_DF, "dtype must be RTE_F32, RTE_F64 or RTE_F64_DF");
+  const int prec = dtype == RTE_F32 ? rte::PREC_F32 : (dtype == RTE_F64 ? rte::PREC_F64 : rte::PREC_DF);
+  if (directions == 0) {
+    p->pin_shape[prec] = rte::WaveShape{};
+    return RTE_OK;
+  }
+  const rte::WaveShape s{directions, warps, rows_per_lane};
+  if (p->dim != 2 || p->cellsig || directions < 0 || directions > 16 || rows_per_lane < 1 ||
+      rows_per_lane > 2 || !rte::wave_shape_ok(p, prec, s)) {
+    rte::set_error("rte_problem_set_sweep_shape: no such operator sweep for this problem");
+    return RTE_ERR_UNSUPPORTED;
+  }
+  p->pin_shape[prec] = s;
   return RTE_OK;
 }
 
