@@ -501,8 +501,8 @@ namespace cg = cooperative_groups;
 // one cell around it, stay in shared memory; nothing but r is stored between the passes over the mesh, and the coefficients
 // come from the classes' tables, which the L1 holds.  An apply used to move 800 bytes a cell (x, its source and the fluxes
 // written and read back, a 4x4 inverse and an element matrix per cell); now 115 from DRAM.  64 instances of 256^2: 783 ->
-// 602 us, no longer bound by HBM but by dependent loads and barriers (37 % of the issue slots; registers for two blocks
-// an SM).  Recomputing x at the nine cells of the stencil instead of the tile took 1119 us.
+// 602 us, no longer bound by HBM but by dependent loads and barriers (28 % of the issue slots with 16 instances; registers
+// for two blocks an SM).  Recomputing x at the nine cells of the stencil instead of the tile took 1119 us.
 constexpr int kTileX = 32, kTileY = kThreads / kTileX;
 // a cell of v; VEC: v is 16-byte aligned (a caller's vector need not be)
 template <bool VEC, typename TV>

@@ -360,8 +360,6 @@ __global__ void __launch_bounds__(128) k_sweep2d(SweepArgs a) {
 // source prefetch is a plain +-PF offset.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
-  using TI = T;
-  constexpr bool ANG = true;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
   const int tid = blockIdx.x;
@@ -399,25 +397,23 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
   const T bndx = (a.inflow_mask & (sx > 0 ? 1 : 2)) ? (T)gtr : (T)0;
   const T bndy = (a.inflow_mask & (sy > 0 ? 4 : 8)) ? (T)gtr : (T)0;
   const bool sig_s = a.sig_s != nullptr;
-  const TI* src = reinterpret_cast<const TI*>(a.src) + in.off;
-  T* psi = ANG ? reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off : nullptr;
+  const T* src = reinterpret_cast<const T*>(a.src) + in.off;
+  T* psi = reinterpret_cast<T*>(a.psi) + (size_t)(a.psi_unique ? a.nu : a.ndir) * in.off;
   // angular output: element offsets (within the instance) of the blocks each of the task's directions
   // is stored to (its unique block, or the one or two N_Omega blocks it stands for), read once here
   // instead of from the direction table at every flush
   int ob0[D], ob1[D];
   bool dup2 = true;   // every direction stands for at most two stored blocks
-  if (ANG) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const UDir u = a.udir[tk.u0 + d];
-      if (a.psi_unique) {
-        ob0[d] = (tk.u0 + d) * in.ndof;
-        ob1[d] = -1;
-      } else {
-        ob0[d] = u.dup[0] * in.ndof;
-        ob1[d] = u.ndup > 1 ? u.dup[1] * in.ndof : -1;
-        dup2 = dup2 && u.ndup <= 2;
-      }
+  for (int d = 0; d < D; ++d) {
+    const UDir u = a.udir[tk.u0 + d];
+    if (a.psi_unique) {
+      ob0[d] = (tk.u0 + d) * in.ndof;
+      ob1[d] = -1;
+    } else {
+      ob0[d] = u.dup[0] * in.ndof;
+      ob1[d] = u.ndup > 1 ? u.dup[1] * in.ndof : -1;
+      dup2 = dup2 && u.ndup <= 2;
     }
   }
   // in a mesh whose width is a multiple of 8 the lanes that complete an 8-cell segment at step s are
@@ -439,11 +435,11 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
   for (int d = 0; d < D; ++d) { tx0[d] = tx1[d] = ty0[d] = ty1[d] = (T)0; }
   constexpr int PF = 8;
   static_assert(PF == SK, "the barrier closes each prefetch group of SK steps");
-  TI q0[PF], q1[PF], q2[PF], q3[PF];
+  T q0[PF], q1[PF], q2[PF], q3[PF];
 #pragma unroll
   for (int k = 0; k < PF; ++k) {
     const int c = col0 + k;
-    if (rowok && c >= 0 && c < nx) Vec4<TI>::load(src + 4 * cell_of(c), q0[k], q1[k], q2[k], q3[k]);
+    if (rowok && c >= 0 && c < nx) Vec4<T>::load(src + 4 * cell_of(c), q0[k], q1[k], q2[k], q3[k]);
   }
   __syncthreads();
   for (int s0 = 0; s0 < nsteps; s0 += PF) {
@@ -455,7 +451,7 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
       T s0v = (T)q0[kk], s1 = (T)q1[kk], s2 = (T)q2[kk], s3 = (T)q3[kk];
       {
         const int cn = col + PF;
-        if (rowok && cn >= 0 && cn < nx) Vec4<TI>::load(src + 4 * cell_of(cn), q0[kk], q1[kk], q2[kk], q3[kk]);
+        if (rowok && cn >= 0 && cn < nx) Vec4<T>::load(src + 4 * cell_of(cn), q0[kk], q1[kk], q2[kk], q3[kk]);
       }
       T yi0[D], yi1[D];
 #pragma unroll
@@ -517,51 +513,47 @@ __global__ void __launch_bounds__(256) k_sweep2d_bands(SweepArgs a) {
             yb[(d * nx + col) * 2] = ty0[d];
             yb[(d * nx + col) * 2 + 1] = ty1[d];
           }
-          if (ANG) {
-            const T q1 = sx > 0 ? p1 : -p1, q2 = sy > 0 ? p2 : -p2, q3 = (sx * sy) > 0 ? p3 : -p3;
-            Vec4<T>::store(ring + d * 32 + (col & 7) * 4, p0, q1, q2, q3);
-          }
+          const T q1 = sx > 0 ? p1 : -p1, q2 = sy > 0 ? p2 : -p2, q3 = (sx * sy) > 0 ? p3 : -p3;
+          Vec4<T>::store(ring + d * 32 + (col & 7) * 4, p0, q1, q2, q3);
         }
       }
-      if (ANG) {
-        // lanes that completed an aligned 8-cell segment (or their row) hand it to the warp: lanes
-        // 8k..8k+7 store the k-th completed segment, one cell each, so every store instruction writes
-        // whole 128-byte lines
-        const bool flush = act && ((col & 7) == 7 || col == nx - 1);
-        __syncwarp();
-        const int k = lane >> 3, e = lane & 7;
-        // cell of the flushing lane f's current column (its row is band * 32 + f)
-        auto cell_at = [&](int f, int colf) -> long long {
-          const int rowf = band * 32 + f;
-          const int iyf = sy > 0 ? rowf : ny - 1 - rowf;
-          return (long long)iyf * nx + (sx > 0 ? colf : nx - 1 - colf);
-        };
-        if (regular) {
-          const int f = ((s + 1) & 7) + 8 * k;
-          const bool ff = __shfl_sync(0xffffffffu, flush, f);
-          const int colf = s - (32 + SK) * band - f;
-          if (ff) {
+      // lanes that completed an aligned 8-cell segment (or their row) hand it to the warp: lanes
+      // 8k..8k+7 store the k-th completed segment, one cell each, so every store instruction writes
+      // whole 128-byte lines
+      const bool flush = act && ((col & 7) == 7 || col == nx - 1);
+      __syncwarp();
+      const int k = lane >> 3, e = lane & 7;
+      // cell of the flushing lane f's current column (its row is band * 32 + f)
+      auto cell_at = [&](int f, int colf) -> long long {
+        const int rowf = band * 32 + f;
+        const int iyf = sy > 0 ? rowf : ny - 1 - rowf;
+        return (long long)iyf * nx + (sx > 0 ? colf : nx - 1 - colf);
+      };
+      if (regular) {
+        const int f = ((s + 1) & 7) + 8 * k;
+        const bool ff = __shfl_sync(0xffffffffu, flush, f);
+        const int colf = s - (32 + SK) * band - f;
+        if (ff) {
+          const long long cf = cell_at(f, colf);
+          RTE_STORE_SEGMENT(f, cf, colf, e);
+        }
+      } else {
+        unsigned fm = __ballot_sync(0xffffffffu, flush);
+        while (fm) {
+          int fl[4], n = 0;
+          while (fm && n < 4) {
+            fl[n++] = __ffs(fm) - 1;
+            fm &= fm - 1;
+          }
+          if (k < n) {
+            const int f = fl[k];
+            const int colf = s - (32 + SK) * band - f;
             const long long cf = cell_at(f, colf);
             RTE_STORE_SEGMENT(f, cf, colf, e);
           }
-        } else {
-          unsigned fm = __ballot_sync(0xffffffffu, flush);
-          while (fm) {
-            int fl[4], n = 0;
-            while (fm && n < 4) {
-              fl[n++] = __ffs(fm) - 1;
-              fm &= fm - 1;
-            }
-            if (k < n) {
-              const int f = fl[k];
-              const int colf = s - (32 + SK) * band - f;
-              const long long cf = cell_at(f, colf);
-              RTE_STORE_SEGMENT(f, cf, colf, e);
-            }
-          }
         }
-        __syncwarp();
       }
+      __syncwarp();
       // the bands meet once per group of SK steps (PF == SK: the last step of the prefetch group)
       if (nwarps > 1 && kk == PF - 1) __syncthreads();
       else __syncwarp();

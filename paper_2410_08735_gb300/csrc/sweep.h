@@ -1,4 +1,5 @@
-// Shared by the sweep translation units (sweep.cu, wavefront.cu, slab.cu): launch arguments and vector loads.
+// Shared by the sweep translation units (sweep.cu, wavefront.cu) and dsa.cu: launch arguments, vector loads, shared-memory
+// grants.
 #pragma once
 #include <atomic>
 
@@ -12,7 +13,7 @@ struct SweepArgs {
   const UDir* udir;
   const SweepTask* tasks;
   int ntasks;
-  const void* linv;     // compute type: cell inverses (sweep.cu), or the tables launch_wave puts here
+  const void* linv;     // compute type: cell inverses, or the FP32 tables that launch_wave puts here
   const void* sig_s;    // compute type, [B][R]; null: no Sigma_s scaling of the input
   const void* src;      // input type, scalar vector
   int with_bc;

@@ -36,11 +36,12 @@
 // table entries per direction and region, D <= 8, one warp per task or per band).  FP32, 64 x 256^2, 192 directions,
 // 8 x 8 regions: 2.08 -> 0.98 ms (D = 12, W = 2; bound by the load/store data pipe); 256 instances on 32^2, 64^2 and 128^2,
 // 128 directions: 0.672 -> 0.336 ms (D = 8, two rows a lane: each table and shuffle serves two cells); one 64^2 instance:
-// 36.3 -> 28.9 us (latency of 131 steps).  FP64 is bound by the FP64 unit, which takes 64 cycles of an SM quarter for a warp
+// 36.3 -> 28.8 us (latency of 131 steps).  FP64 is bound by the FP64 unit, which takes 64 cycles of an SM quarter for a warp
 // instruction, whatever the number of lanes, and 76 with all four quarters busy: so by instructions per step.
-// 7.92 -> 6.74 ms on the 256 instances (D = 4), 0.919 -> 0.527 ms on 10 x 80^2 with CL(30, 6) (D = 1).  Double-float is bound
-// by FP32 issue: 3.61 -> 2.01 ms on 16 x 256^2 (D = 4, W = 4; the step loop not unrolled: unrolled it missed the instruction
-// cache, 3.48 ms).
+// 7.92 -> 6.75 ms on the 256 instances (D = 4), 0.919 -> 0.500 ms on 10 x 80^2 with CL(30, 6) (D = 1), one 40^2 instance
+// 154 -> 113 us.  Double-float is bound by FP32 issue: 3.61 -> 2.01 ms on 16 x 256^2 (D = 4, W = 4; the step loop not
+// unrolled: unrolled it missed the instruction cache, 3.48 ms); 2 x (160 x 186) 417 -> 177 us (238 while sources rotated
+// through registers, whose moves waited for their loads).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -793,9 +794,9 @@ bool wave_shape_ok(const rte_problem* p, int prec, WaveShape s) {
 // step, one step taking the pipe cycles of all of them or the latency of one alone, whichever is longer.  Per warp and
 // step, measured: FP32 10 D + 40 cycles of the load/store data pipe (tables, shuffles; 13 D + 30 with two rows a lane),
 // the pipe that fills up first, of which single-warp tasks reach 0.65 and wider ones 0.75, 50 D + 300 alone (1750 with
-// two rows); FP64 19 cycles of the SM's FP64 unit for each of 24 D + 30 instructions (32 D + 4 in
-// the Legendre basis; 5 % more a direction above 4), 70 alone; double-float 320 D + 264 instructions, 0.85 a cycle and SM quarter, 0.7 alone.  The partial fluxes, written and read once, are
-// added at the copy bandwidth.
+// two rows); FP64 19 cycles of the SM's FP64 unit for each of 32 D instructions, 70 alone; double-float 356 D + 160
+// instructions, 0.85 a cycle and SM quarter, 0.5 alone.  The partial fluxes, written and read once, are added at the copy
+// bandwidth.
 static double wave_cost(const rte_problem* p, int prec, WaveShape s, int sms, const std::vector<int>& order) {
   const int SK = 4, per_sm = 65536 / (shape_regs(p, prec, s) * 32);
   const size_t smem = wave_smem(p, prec, s) + 1024;
