@@ -39,9 +39,9 @@ import numpy as np  # noqa: E402
 
 import workloads as wl  # noqa: E402
 
-# Algorithmic arithmetic per cell and unique direction of the fused 2D sweep (rhs assembly, 4x4 solve with the
-# precomputed cell inverse, outflow traces, quadrature): about 42 FMA = 90 flop.
-SWEEP_FLOPS_PER_CELL_DIR = 90
+# Algorithmic arithmetic per cell and unique direction of the fused 2D sweep: the cell system is a Kronecker sum of 2x2
+# blocks, so 25 multiply-adds take a cell from its inflow to its outflow and quadrature, 50 flop.
+SWEEP_FLOPS_PER_CELL_DIR = 50
 
 METRIC = "param solves/s at 1e-8 true residual (mixed+MLP FGMRES-ROMSAD vs plain FP64 FGMRES-ROMSAD)"
 
@@ -921,8 +921,8 @@ def main():
     ndf = statistics.mean(s["sweeps_df"] for s in st_m)
     n32 = statistics.mean(s["sweeps"] for s in st_m) - n64 - ndf
     nv = statistics.mean(s["iterations"] for s in st_m)   # one preconditioner apply per iteration
-    shares = {"k_sweep2d<float> (A~ apply, FP32)": n32 * ms32, "k_sweep2d<double> (A~ apply, FP64)": n64 * ms64,
-              "k_sweep2d<dfloat> (A~ apply, double-float)": ndf * msdf, "k_dsa_vcycle (DSA V-cycle)": nv * ms_v}
+    shares = {"k_wave<float> (A~ apply, FP32)": n32 * ms32, "k_wave<double> (A~ apply, FP64)": n64 * ms64,
+              "k_wave<dfloat> (A~ apply, double-float)": ndf * msdf, "k_dsa_vcycle (DSA V-cycle)": nv * ms_v}
     per_solve_ms = 1e3 * results["mixed"][0] / args.steps
     dom = max(shares, key=shares.get)
     if "FP32" in dom:
@@ -945,11 +945,11 @@ def main():
     roof["shares_ms_per_solve_batch"] = shares
     roof["solve_batch_ms"] = per_solve_ms
     roof["other_kernels"] = {
-        "k_sweep2d<float>": {"ms": ms32, "tflops": flops / (ms32 * 1e-3) / 1e12,
-                             "frac_of_fp32_peak": flops / (ms32 * 1e-3) / 1e12 / peaks["fp32_fma_tflops"]},
-        "k_sweep2d<double>": {"ms": ms64, "tflops": flops / (ms64 * 1e-3) / 1e12,
-                              "frac_of_fp64_peak": flops / (ms64 * 1e-3) / 1e12 / peaks["fp64_fma_tflops"]},
-        "k_sweep2d<dfloat>": {"ms": msdf, "tflops_df": flops / (msdf * 1e-3) / 1e12},
+        "k_wave<float>": {"ms": ms32, "tflops": flops / (ms32 * 1e-3) / 1e12,
+                          "frac_of_fp32_peak": flops / (ms32 * 1e-3) / 1e12 / peaks["fp32_fma_tflops"]},
+        "k_wave<double>": {"ms": ms64, "tflops": flops / (ms64 * 1e-3) / 1e12,
+                           "frac_of_fp64_peak": flops / (ms64 * 1e-3) / 1e12 / peaks["fp64_fma_tflops"]},
+        "k_wave<dfloat>": {"ms": msdf, "tflops_df": flops / (msdf * 1e-3) / 1e12},
         "k_dsa_vcycle": {"ms": ms_v}}
     del z64, w64, z32, w32
     torch.cuda.empty_cache()
@@ -1029,19 +1029,19 @@ def main():
 # fine cell).
 DSA_VCYCLE_BYTES_PER_CELL = 4 * 72
 
-# DRAM traffic of one A~ apply (the sweep kernel plus the reduce of its partial fluxes), dram__bytes_read.sum +
-# dram__bytes_write.sum from one ncu capture of each kernel (bench.py --profile ...), with the SHA-256 of the
-# sweep source it was taken on: reported only while that source is unchanged.  The FP64 capture ran 16 of the 64
-# instances; its traffic grows in proportion to the instances and is scaled by 4.
+# DRAM traffic of one A~ apply (the sweep kernel, the reduce of its partial fluxes and, in FP64, the pass that multiplies
+# the source by Sigma_s), dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture of each kernel (bench.py
+# --profile ...), with the SHA-256 of the sweep source it was taken on: reported only while that source is unchanged.
+# The FP64 capture ran 16 of the 64 instances; its traffic grows in proportion to the instances and is scaled by 4.
 NCU_TRAFFIC = {
-    ("large256_192", "k_sweep2d<float> (A~ apply, FP32)"): {
-        "bytes": (0.186164 + 1.575940 + 1.677866 + 0.066262) * 1e9, "instances_captured": 64,
-        "kernels": "k_sweep2d_bands<float, float, 4, 0> + k_reduce<float, float, float>",
-        "sweep_sha256": "ea85f47f3deb12d1da7f9e8a0a2d4e3c155404c397c62a958ab093216829f25d"},
-    ("large256_192", "k_sweep2d<double> (A~ apply, FP64)"): {
-        "bytes": 4 * (0.115022 + 1.554706 + 1.644242 + 0.034141) * 1e9, "instances_captured": 16,
-        "kernels": "k_sweep2d<double, double, 2, 0, 0> + k_reduce<double, double, double>",
-        "sweep_sha256": "ea85f47f3deb12d1da7f9e8a0a2d4e3c155404c397c62a958ab093216829f25d"},
+    ("large256_192", "k_wave<float> (A~ apply, FP32)"): {
+        "bytes": (0.15639 + 0.48452 + 0.60402 + 0.05708) * 1e9, "instances_captured": 64,
+        "kernels": "k_wave<float, float, Rot<float>, 2, 6, 1, 4> + k_reduce<float, float, float>",
+        "sweep_sha256": "3e58c749f15727325f72448e2da5341048f87ce38d61fedd05a7920af095b5ba"},
+    ("large256_192", "k_wave<double> (A~ apply, FP64)"): {
+        "bytes": 4 * (0.033571 + 0.000033 + 0.082610 + 1.015618 + 1.107505 + 0.030522) * 1e9, "instances_captured": 16,
+        "kernels": "k_scatter_source<0> + k_wave<double, double, Legendre<double, 0>, 1, 3, 1, 4> + k_reduce<double, double, double>",
+        "sweep_sha256": "3e58c749f15727325f72448e2da5341048f87ce38d61fedd05a7920af095b5ba"},
 }
 
 
@@ -1052,7 +1052,7 @@ def ncu_traffic(workload: str, kernel: str):
     rec = NCU_TRAFFIC.get((workload, kernel))
     if rec is None:
         return None
-    with open(os.path.join(ROOT, "paper_2410_08735_gb300", "csrc", "sweep.cu"), "rb") as fh:
+    with open(os.path.join(ROOT, "paper_2410_08735_gb300", "csrc", "wavefront.cu"), "rb") as fh:
         if hashlib.sha256(fh.read()).hexdigest() != rec["sweep_sha256"]:
             return None
     return rec["bytes"]
