@@ -147,6 +147,7 @@ struct rte_problem {
   rte::DevBuf<float> d_linv_df;               // as double-float pairs (hi, lo): 1D all entries, 2D the nine distinct ones
                                               // [10][2] in scaled modes (wavefront.cu)
   rte::DevBuf<float> d_rot32;                 // 2D: FP32 operator tables [B][nu][R][8] (wavefront.cu)
+  rte::DevBuf<double> d_inv64;                // 2D: nine entries of the cell inverses, rounded once, [B][nu][R][10]
   rte::DevBuf<float> d_sig_s_df;              // [B][R][2] sigma_s as double-float pairs
   rte::DevBuf<float> d_xdf;                   // [ntot][2] source of a double-float (pairs) or FP64 sweep
   // sweep scratch (grown on demand)

@@ -140,15 +140,6 @@ __global__ void k_linv(int B, int nu, int R, int dim, const InstInfo* inst, cons
       outdf[2 * (base + i) + 1] = (float)(X[i] - (double)h);
     }
   }
-  if (dim == 2) {   // the nine distinct entries in the scaled modes of the double-float sweeps (Scaled, wavefront.cu)
-    const double v[10] = {X[0], 3.0 * X[5], 3.0 * X[10], 9.0 * X[15], s3 * X[1], 3.0 * s3 * X[11], s3 * X[2],
-                          3.0 * s3 * X[7], 3.0 * X[3], 0.0};
-    for (int i = 0; i < 10; ++i) {
-      const float h = (float)v[i];
-      outdf[2 * (tid * 10 + i)] = h;
-      outdf[2 * (tid * 10 + i) + 1] = (float)(v[i] - (double)h);
-    }
-  }
 }
 
 // Cell inverses with a full Sigma_t block per cell (cross-section profiles): thread (b, u, c) inverts
@@ -528,7 +519,10 @@ static int create_impl(const rte_problem_desc* d, rte_problem* p) {
   {
     const size_t nt = (size_t)p->B * p->nu * p->R;
     RTE_TRY(p->d_linv_df.alloc(p->dim == 2 ? 20 * nt : 2 * nl));
-    if (p->dim == 2) RTE_TRY(p->d_rot32.alloc(8 * nt));
+    if (p->dim == 2) {
+      RTE_TRY(p->d_rot32.alloc(8 * nt));
+      RTE_TRY(p->d_inv64.alloc(10 * nt));
+    }
   }
   RTE_TRY(p->d_active.alloc(p->B));
   RTE_TRY(p->d_wq.alloc(p->ndir));

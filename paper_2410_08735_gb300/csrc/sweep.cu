@@ -670,7 +670,11 @@ __global__ void __launch_bounds__(128) k_sweep1d(SweepArgs a) {
   }
 }
 
-// out = sum_t partial[t]  (mode T),  z - sum (mode OP),  b - (z - sum) (mode RES); one instance per blockIdx.y.
+// out = sum_t partial[t]  (mode T),  z - sum (mode OP),  b - (z - sum) (mode RES); one instance per blockIdx.y.  Eight
+// partial fluxes at a time are added as a tree: in one chain their roundings were the larger part of an apply's error
+// (double-float 0.45 to 0.9 times now, one FP32 64^2 instance 4.7e-7 -> 3.0e-7), and mixed solves of 16 x 256^2 to 1e-12
+// stalled at 2e-12 to 4e-12 in 3 draws of 21, the certificate's own rounding.  (The loads of eight are in flight together:
+// one 64^2 instance 28.8 -> 26.7 us.)
 template <typename TP, typename TZ, typename TO>
 __global__ void k_reduce(const TP* partial, int ntask, const InstInfo* inst, int mode, const TZ* z, const TO* bvec,
                          TO* out, const int* active) {
@@ -680,7 +684,14 @@ __global__ void k_reduce(const TP* partial, int ntask, const InstInfo* inst, int
   const TP* pp = partial + (size_t)ntask * in.off;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < in.ndof; i += gridDim.x * blockDim.x) {
     TP s = 0;
-    for (int t = 0; t < ntask; ++t) s += pp[(size_t)t * in.ndof + i];
+    int t = 0;
+    for (; t + 8 <= ntask; t += 8) { 
+      TP x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = pp[(size_t)(t + e) * in.ndof + i];
+      s += ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+    }
+    for (; t < ntask; ++t) s += pp[(size_t)t * in.ndof + i];
     TO v = (TO)s;
     if (mode == MODE_OP) v = (TO)z[in.off + i] - v;
     if (mode == MODE_RES) v = bvec[in.off + i] - ((TO)z[in.off + i] - v);

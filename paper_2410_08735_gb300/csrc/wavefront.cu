@@ -21,10 +21,10 @@
 //    both components of a pair with the same weight -alpha (or -beta), the outflow is a plain sum, and L^{-1} has
 //    eight distinct entries: 8 + 16 + 4 multiply-adds and adds and 4 for the quadrature, against 9 + 16 + 4 + 4 and
 //    sixteen entries in the Legendre basis.  The source is brought to the basis, and the summed flux back, once per cell
-//    and task.  The error of an apply against 64-bit values is 0.6 to 1.1 times that of the former Legendre kernels (13
-//    batches of 1 to 256 instances; 2.4e-7 against 2.2e-7 on the uneven one below): the transforms add roundings that all
-//    directions of a task share, longer tasks save some in the sum of the partial fluxes.
-//  * Legendre (FP64): no change of basis, the cell inverses that the angular sweeps use.
+//    and task.  The error of an apply against 64-bit values is 0.5 to 1.1 times that of the former Legendre kernels (13
+//    batches of 1 to 256 instances; 2.3e-7 against 2.2e-7 on the uneven one below).
+//  * Legendre (FP64): no change of basis; tasks of one and two directions with the cell inverses that the angular sweeps
+//    use, wider ones with the nine entries that are distinct.
 //  * Scaled (double-float): the Legendre modes scaled, which saves products.
 // The eigenbasis of N (complex products, 24 operations a direction and 30 a cell for its transforms) is no better choice for
 // these two: it is not orthogonal (condition number 3.7), in double-float the error of an apply is 15 to 70 % larger, and
@@ -34,13 +34,13 @@
 //
 // Bounds and measurements (one operator apply with the sum of its partial fluxes, GB300; before: Legendre basis, sixteen
 // table entries per direction and region, D <= 8, one warp per task or per band).  FP32, 64 x 256^2, 192 directions,
-// 8 x 8 regions: 2.08 -> 0.98 ms (D = 12, W = 2; bound by the load/store data pipe); 256 instances on 32^2, 64^2 and 128^2,
-// 128 directions: 0.672 -> 0.336 ms (D = 8, two rows a lane: each table and shuffle serves two cells); one 64^2 instance:
-// 36.3 -> 28.8 us (latency of 131 steps).  FP64 is bound by the FP64 unit, which takes 64 cycles of an SM quarter for a warp
+// 8 x 8 regions: 2.08 -> 0.96 ms (D = 12, W = 2; bound by the load/store data pipe); 256 instances on 32^2, 64^2 and 128^2,
+// 128 directions: 0.672 -> 0.327 ms (D = 8, two rows a lane: each table and shuffle serves two cells); one 64^2 instance:
+// 36.3 -> 26.7 us (latency of 131 steps).  FP64 is bound by the FP64 unit, which takes 64 cycles of an SM quarter for a warp
 // instruction, whatever the number of lanes, and 76 with all four quarters busy: so by instructions per step.
-// 7.92 -> 6.75 ms on the 256 instances (D = 4), 0.919 -> 0.500 ms on 10 x 80^2 with CL(30, 6) (D = 1), one 40^2 instance
-// 154 -> 113 us.  Double-float is bound by FP32 issue: 3.61 -> 2.01 ms on 16 x 256^2 (D = 4, W = 4; the step loop not
-// unrolled: unrolled it missed the instruction cache, 3.48 ms); 2 x (160 x 186) 417 -> 177 us (238 while sources rotated
+// 7.92 -> 6.63 ms on the 256 instances (D = 4), 0.919 -> 0.500 ms on 10 x 80^2 with CL(30, 6) (D = 1), one 40^2 instance
+// 154 -> 113 us.  Double-float is bound by FP32 issue: 3.61 -> 2.00 ms on 16 x 256^2 (D = 4, W = 4; the step loop not
+// unrolled: unrolled it missed the instruction cache, 3.48 ms); 2 x (160 x 186) 417 -> 176 us (238 while sources rotated
 // through registers, whose moves waited for their loads).
 #include <algorithm>
 #include <cmath>
@@ -182,7 +182,8 @@ struct Rot {
   }
   // The transforms' rounding errors are shared by all directions of a task, so both are written for few roundings at the
   // size of the leading component: the higher modes are added up first and meet it in one multiply-add (to), the scalings
-  // are part of the sums (from).  Against sums of pairs and separate products: 4 to 8 % less error of an apply.
+  // are part of the sums (from).  Against sums of pairs and separate products: 1 % less error of an apply on average over
+  // those batches, up to 3 %.
   __device__ __forceinline__ static void to_basis(const T* t, T* S) {
     const T e = t[1] + t[2], f = t[1] - t[2];
     S[0] = t[0] + (t[3] + e);
@@ -277,13 +278,39 @@ struct Legendre {
   }
 };
 
+// The same with the nine distinct entries of a cell inverse, for FP64 tasks of three and more directions.  As a combination
+// of 1, N_x, N_y, N_x N_y, N = [[-1, sqrt3], [-sqrt3, 1]] / sqrt2, an inverse has its diagonal d0 .. d3, +-u0, +-u1 between the
+// x-modes, +-v0, +-v1 between the y-modes, and +-w.  Fewer loads and smaller tables (256 uneven instances 6.74 -> 6.63 ms), and
+// the entries are rounded once (k_wave_tables), which the certificate of a tight solve gains by: emulated against extended
+// precision, an apply's error is 2.5e-16 against 3.3e-16 with the inverses of the problem set-up on 40^2, 5.8e-16 against
+// 1.7e-15 on 128^2.
+template <typename T, bool SIG>
+struct Nine : Legendre<T, SIG> {
+  static constexpr int TW = 10;   // nine entries and a spare one, for 16-byte boundaries
+  template <typename V>
+  __device__ __forceinline__ static void cell(const V* S, V* X, V* Y, const V* m, const V* c, V* acc, bool zero) {
+    const T a = c[0].x, b = c[1].x, a3 = c[2].x, b3 = c[3].x, w = c[4].x, s3 = (T)1.7320508075688772;
+    const T x0 = X[0].x, x1 = X[1].x, y0 = Y[0].x, y1 = Y[1].x;
+    const T r0 = S[0].x + a * x0 + b * y0, r1 = S[1].x - a3 * x0 + b * y1;
+    const T r2 = S[2].x + a * x1 - b3 * y0, r3 = S[3].x - a3 * x1 - b3 * y1;
+    const T q[4] = {m[0].x * r0 + m[4].x * r1 + m[6].x * r2 + m[8].x * r3,
+                    m[1].x * r1 - m[4].x * r0 - m[8].x * r2 + m[7].x * r3,
+                    m[2].x * r2 - m[6].x * r0 - m[8].x * r1 + m[5].x * r3,
+                    m[3].x * r3 + m[8].x * r0 - m[7].x * r1 - m[5].x * r2};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i].x = zero ? w * q[i] : acc[i].x + w * q[i];
+    X[0].x = q[0] + s3 * q[1];
+    X[1].x = q[2] + s3 * q[3];
+    Y[0].x = q[0] + s3 * q[2];
+    Y[1].x = q[1] + s3 * q[3];
+  }
+};
+
 // Scaled Legendre modes (double-float): P = (1, sqrt3, sqrt3, 3) p, sources divided by the same, second traces times
 // sqrt3.  Outflows become plain sums and each product of a trace enters two components: 356 operations a cell and direction
 // against 400 in the Legendre basis, with the same rounding errors (in the eigenbasis of N 318 and transforms, and errors
 // 15 to 70 % larger).  The scalings cost nothing: they are part of the tables, the quadrature weights and the pass that
-// splits the source into pairs, which also multiplies it by Sigma_s.
-// As a combination of 1, N_x, N_y, N_x N_y, N = [[-1, sqrt3], [-sqrt3, 1]] / sqrt2, a cell inverse has nine distinct entries:
-// its diagonal d0 .. d3, +-u0, +-u1 between the x-modes, +-v0, +-v1 between the y-modes, and +-w.
+// splits the source into pairs, which also multiplies it by Sigma_s.  Nine entries an inverse, as above.
 struct Scaled {
   using T = dfloat;
   static constexpr int TW = 10, FW = 0, HD = 0;   // nine entries and a spare one, for 16-byte boundaries
@@ -332,33 +359,81 @@ struct Scaled {
   }
 };
 
-// FP32 tables [8] per (instance, unique direction, region).
-// l_1 = c_0 + i sqrt2 (alpha + beta), l_2 = c_0 + i sqrt2 (alpha - beta), c_0 = 2 (alpha + beta) + sigma_t, are the
-// eigenvalues of L on the products of eigenvectors of N; L^{-1} = g + g_x N_x + g_y N_y + g_xy N_x N_y follows from
-// 1 / l_1, 1 / l_2.
+// Unevaluated sums of two doubles, for the tables alone (two-sum and two-product as in dfloat.cuh)
+struct Dd {
+  double h, l;
+  __device__ Dd operator-() const { return Dd{-h, -l}; }
+};
+__device__ __forceinline__ Dd dd_sum(double a, double b) {
+  const double s = __dadd_rn(a, b), t = __dsub_rn(s, a);
+  return Dd{s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, t)), __dsub_rn(b, t))};
+}
+__device__ __forceinline__ Dd operator+(Dd a, Dd b) {
+  const Dd s = dd_sum(a.h, b.h);
+  return dd_sum(s.h, __dadd_rn(s.l, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Dd operator*(Dd a, Dd b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return dd_sum(p, __fma_rn(a.l, b.h, __fma_rn(a.h, b.l, __fma_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ Dd operator/(Dd a, Dd b) {
+  const double q = __ddiv_rn(a.h, b.h);
+  const Dd r = a + -(Dd{q, 0.0} * b);
+  return dd_sum(q, __ddiv_rn(r.h, b.h));
+}
+
+// Tables per (instance, unique direction, region): Rot FP32 [8], Nine FP64 [10] and Scaled double-float pairs [10].
+// l_1 = c_0 + i sqrt2 (alpha + beta) and l_2 = c_0 + i sqrt2 (alpha - beta), c_0 = 2 (alpha + beta) + sigma_t, are the
+// eigenvalues of L on the products of eigenvectors of N, n_1 and n_2 their squared moduli;
+// L^{-1} = g + g_x N_x + g_y N_y + g_xy N_x N_y follows from 1 / l_1, 1 / l_2.
 __global__ void k_wave_tables(int B, int nu, int R, const InstInfo* inst, const UDir* ud, const double* sig_t,
-                              float* rot) {
+                              float* rot, double* inv64, float2* inv_df) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (tid >= (long long)B * nu * R) return;
   const int r = (int)(tid % R), u = (int)((tid / R) % nu), b = (int)(tid / ((long long)R * nu));
   const double al = ud[u].ax / inst[b].hx, be = ud[u].ay / inst[b].hy, sg = sig_t[(size_t)b * R + r];
-  const double s2 = 1.4142135623730950488, c0 = 2.0 * (al + be) + sg;
-  const double i1 = s2 * (al + be), i2 = s2 * (al - be);
-  const double n1 = c0 * c0 + i1 * i1, n2 = c0 * c0 + i2 * i2, inv = 1.0 / (n1 * n2);
-  const double g = c0 * (c0 * c0 + 2.0 * (al * al + be * be)) * inv;
-  const double gx = -s2 * al * (c0 * c0 + 2.0 * (al - be) * (al + be)) * inv;
-  const double gy = -s2 * be * (c0 * c0 - 2.0 * (al - be) * (al + be)) * inv;
-  const double gxy = 4.0 * al * be * c0 * inv;
-  // scaled N of an axis: [[0, a^3], [-a^{-3}, 0]] (a^3: the turn's a and twice the scaling by q)
-  const double a3 = 7.2097685201075047693, b3 = 1.0 / a3;
-  const double t[8] = {g, gx * a3, -gx * b3, gy * a3, -gy * b3, gxy * a3 * a3, -gxy, gxy * b3 * b3};
-  for (int k = 0; k < 8; ++k) rot[tid * 8 + k] = (float)t[k];
+  {
+    const double s2 = 1.4142135623730950488, c0 = 2.0 * (al + be) + sg;
+    const double i1 = s2 * (al + be), i2 = s2 * (al - be);
+    const double n1 = c0 * c0 + i1 * i1, n2 = c0 * c0 + i2 * i2, inv = 1.0 / (n1 * n2);
+    const double g = c0 * (c0 * c0 + 2.0 * (al * al + be * be)) * inv;
+    const double gx = -s2 * al * (c0 * c0 + 2.0 * (al - be) * (al + be)) * inv;
+    const double gy = -s2 * be * (c0 * c0 - 2.0 * (al - be) * (al + be)) * inv;
+    const double gxy = 4.0 * al * be * c0 * inv;
+    // scaled N of an axis: [[0, a^3], [-a^{-3}, 0]] (a^3: the turn's a and twice the scaling by q)
+    const double a3 = 7.2097685201075047693, b3 = 1.0 / a3;
+    const double t[8] = {g, gx * a3, -gx * b3, gy * a3, -gy * b3, gxy * a3 * a3, -gxy, gxy * b3 * b3};
+    for (int k = 0; k < 8; ++k) rot[tid * 8 + k] = (float)t[k];
+  }
+  // A = c_0 / n_1, B = c_0 / n_2, C = (alpha + beta) / n_1, E = (alpha - beta) / n_2, k = (B - A) / 4:
+  // d0, d3 = B - k +- C; d2, d1 = A + k +- E; u0, u1 = -sqrt3/2 (C + E) -+ sqrt3 k; v0, v1 = -sqrt3/2 (C - E) -+ sqrt3 k; w = 3 k.
+  // In sums of two doubles, so that the entries are rounded once: what their rounding loses adds up along a ray.
+  const Dd sum = dd_sum(al, be), dif = dd_sum(al, -be);
+  const Dd c0 = Dd{2.0 * sum.h, 2.0 * sum.l} + Dd{sg, 0.0}, cc = c0 * c0, ss = sum * sum, dd = dif * dif;
+  const Dd n1 = cc + Dd{2.0 * ss.h, 2.0 * ss.l}, n2 = cc + Dd{2.0 * dd.h, 2.0 * dd.l};
+  const Dd A = c0 / n1, Bq = c0 / n2, C = sum / n1, E = dif / n2;
+  const Dd s3{1.7320508075688772, 1.0035084221806903e-16}, h3{0.8660254037844386, 5.0175421109034514e-17};
+  Dd k = Bq + -A;
+  k = Dd{0.25 * k.h, 0.25 * k.l};
+  const Dd p1 = Bq + -k, p2 = A + k, x = -(h3 * (C + E)), y = -(h3 * (C + -E)), sk = s3 * k;
+  const Dd m[9] = {p1 + C, p2 + -E, p2 + E, p1 + -C, x + -sk, x + sk, y + -sk, y + sk, k + Dd{2.0 * k.h, 2.0 * k.l}};
+  // of the scaled modes: rows and columns times (1, sqrt3, sqrt3, 3)
+  const Dd c3{3.0, 0.0}, c33 = s3 * c3;
+  const Dd f[9] = {Dd{1.0, 0.0}, c3, c3, Dd{9.0, 0.0}, s3, c33, s3, c33, c3};
+  for (int e = 0; e < 9; ++e) {
+    inv64[tid * 10 + e] = m[e].h;
+    const Dd v = m[e] * f[e];
+    const float h = (float)v.h;
+    inv_df[tid * 10 + e] = make_float2(h, (float)__dadd_rn(__dsub_rn(v.h, (double)h), v.l));
+  }
+  inv64[tid * 10 + 9] = 0.0;
+  inv_df[tid * 10 + 9] = make_float2(0.f, 0.f);
 }
 
 int build_wave_tables(rte_problem* p) {
   const long long n = (long long)p->B * p->nu * p->R;
   k_wave_tables<<<(unsigned)((n + 127) / 128), 128>>>(p->B, p->nu, p->R, p->d_inst.p, p->d_udir.p, p->d_sig_t.p,
-                                                      p->d_rot32.p);
+                                                      p->d_rot32.p, p->d_inv64.p, reinterpret_cast<float2*>(p->d_linv_df.p));
   count_launch();
   RTE_CHECK_CUDA(cudaGetLastError());
   return RTE_OK;
@@ -674,14 +749,15 @@ static size_t shape_smem(const rte_problem* p, int prec, WaveShape s, bool table
   const bool f32 = prec == PREC_F32;
   const int nc = f32 ? F::NC : (prec == PREC_F64 ? W::NC : Scaled::NC);
   const int rs = f32 ? table_stride(F::HD + s.D * F::TW, 4)
-                     : (prec == PREC_F64 ? table_stride(W::HD + s.D * W::TW, 8) : table_stride(s.D * Scaled::TW, 8));
+                     : (prec == PREC_F64 ? table_stride(W::HD + s.D * (s.D > 2 ? Nine<double, true>::TW : W::TW), 8)
+                                         : table_stride(s.D * Scaled::TW, 8));
   const size_t elems = (tables ? (size_t)(p->R + 1) * rs : 0) + ((s.D * nc + 3) & ~3) +
                        ((size_t)nx + (s.W - 1) * kRingCols) * s.D * 2;
   return elems * (f32 ? 4 : 8) + (prec == PREC_DF ? (size_t)s.W * 4 * 1024 : 0);   // and the ring of sources
 }
 
 // FP64 and double-float tables (144 and 80 bytes a region with one direction) stay in global memory where shared memory
-// does not hold them: 1,600 and 2,800 regions and more with one direction, 430 and 670 with four.
+// does not hold them: 1,600 and 2,800 regions and more with one direction, 690 and 670 with four.
 static bool global_tables(const rte_problem* p, int prec, WaveShape s) {
   return prec != PREC_F32 && shape_smem(p, prec, s, true) > kMaxSmem;
 }
@@ -745,21 +821,23 @@ static int with_kernel(int prec, WaveShape s, bool in64, bool sig, bool gt, int 
       }
     }
   } else if (prec == PREC_F64) {
-    auto pick = [&](auto alg) {
-      using A = decltype(alg);
+    auto pick = [&](auto few, auto many) {   // one and two directions a task, three and more
+      using A = decltype(few);
+      using M = decltype(many);
       switch (shape * 2 + gt) {
         case 22: return f(WaveKernel<double, double, A, 1, 1, 1, 4, BC, 2, false>{});
         case 42: return f(WaveKernel<double, double, A, 1, 2, 1, 4, BC, 2, false>{});
-        case 62: return f(WaveKernel<double, double, A, 1, 3, 1, 4, BC, 2, false>{});
-        case 82: return f(WaveKernel<double, double, A, 1, 4, 1, 4, BC, 1, false>{});
+        case 62: return f(WaveKernel<double, double, M, 1, 3, 1, 4, BC, 2, false>{});
+        case 82: return f(WaveKernel<double, double, M, 1, 4, 1, 4, BC, 1, false>{});
         case 23: return f(WaveKernel<double, double, A, 1, 1, 1, 4, BC, 1, true>{});
         case 43: return f(WaveKernel<double, double, A, 1, 2, 1, 4, BC, 1, true>{});
-        case 83: return f(WaveKernel<double, double, A, 1, 4, 1, 4, BC, 1, true>{});
+        case 83: return f(WaveKernel<double, double, M, 1, 4, 1, 4, BC, 1, true>{});
       }
       return none;
     };
-    if constexpr (BC) return pick(Legendre<double, false>{});
-    else return sig ? pick(Legendre<double, true>{}) : pick(Legendre<double, false>{});
+    if constexpr (!BC)
+      if (sig) return pick(Legendre<double, true>{}, Nine<double, true>{});
+    return pick(Legendre<double, false>{}, Nine<double, false>{});
   } else if (!BC) {
     using A = Scaled;
     switch (shape * 2 + gt) {
@@ -904,6 +982,7 @@ int launch_wave(const rte_problem* p, int prec, WaveShape s, bool in64, const Sw
   }
   SweepArgs a = args;
   if (prec == PREC_F32) a.linv = p->d_rot32.p;   // else the cell inverses of the arithmetic
+  if (prec == PREC_F64 && s.D > 2) a.linv = p->d_inv64.p;
   const size_t smem = wave_smem(p, prec, s);
   auto run = [&](auto k) { return decltype(k)::launch(a, s.W, smem, st); };
   const bool gt = global_tables(p, prec, s);
