@@ -1035,13 +1035,13 @@ DSA_VCYCLE_BYTES_PER_CELL = 4 * 72
 # The FP64 capture ran 16 of the 64 instances; its traffic grows in proportion to the instances and is scaled by 4.
 NCU_TRAFFIC = {
     ("large256_192", "k_wave<float> (A~ apply, FP32)"): {
-        "bytes": (0.15639 + 0.48452 + 0.60402 + 0.05708) * 1e9, "instances_captured": 64,
+        "bytes": (0.15688 + 0.48488 + 0.60409 + 0.05686) * 1e9, "instances_captured": 64,
         "kernels": "k_wave<float, float, Rot<float>, 2, 6, 1, 4> + k_reduce<float, float, float>",
-        "sweep_sha256": "3e58c749f15727325f72448e2da5341048f87ce38d61fedd05a7920af095b5ba"},
+        "sweep_sha256": "5822f55f5e1b277f836daca835f85247a193da3c082dfb48d1c63a5a11d31bb1"},
     ("large256_192", "k_wave<double> (A~ apply, FP64)"): {
-        "bytes": 4 * (0.033571 + 0.000033 + 0.082610 + 1.015618 + 1.107505 + 0.030522) * 1e9, "instances_captured": 16,
-        "kernels": "k_scatter_source<0> + k_wave<double, double, Legendre<double, 0>, 1, 3, 1, 4> + k_reduce<double, double, double>",
-        "sweep_sha256": "3e58c749f15727325f72448e2da5341048f87ce38d61fedd05a7920af095b5ba"},
+        "bytes": 4 * (0.033570 + 0.000013 + 0.076962 + 1.017778 + 1.107380 + 0.029891) * 1e9, "instances_captured": 16,
+        "kernels": "k_scatter_source<0> + k_wave<double, double, Nine<double, 0>, 1, 3, 1, 4> + k_reduce<double, double, double>",
+        "sweep_sha256": "5822f55f5e1b277f836daca835f85247a193da3c082dfb48d1c63a5a11d31bb1"},
 }
 
 
